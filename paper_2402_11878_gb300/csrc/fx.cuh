@@ -1,0 +1,145 @@
+// 64-bit block fixed point: the arithmetic of the FP64 ansatz passes.
+//
+// GB300 issues one FP64 multiply-add per 64 clocks and warp scheduler, against
+// one 32 x 32 + 64-bit integer multiply-add per 4.  A multiply-add of 64-bit
+// integers by a constant costs three of those and four cheap instructions: 15
+// clocks measured (a stand-alone loop of butterflies, eight to twelve warps per
+// scheduler), 4.2 times the rate of DFMA.  So a tile pass turns its tile into
+// integers V = x * 2^-E with one exponent E per tile and state, applies the
+// gates to the integers and turns the result back into doubles.
+//
+// Range.  E is chosen from the 2-norm of the tile, which no gate changes:
+// |V|_2 <= 2^61 at the start of a pass.  A butterfly without its scale lets
+// the norm grow; when the growth since the last shift reaches a factor of two
+// (forward; 2^0.75 backward) all values are shifted right by one, and the
+// slot's diagonal table carries the power of two back.  So |V|_2 stays below
+// 2^62.7 and every component below 2^63, for any input.
+//
+// Accuracy.  One operation adds an error of about half a unit, and the
+// root-mean-square component of a tile of 2^11 amplitudes has 54 bits or more
+// above the unit, so the error per operation is below a double's rounding of
+// a component of that size (2^-54.3 root mean square); it is relative to the
+// tile's norm rather than to the single amplitude.
+#pragma once
+
+#include <cstdint>
+
+namespace vqe {
+
+// Coefficient of one gated tile bit for the fixed-point passes.  With
+// alpha = theta/2,
+//     RY(theta) = J^q * 45^o * cos(beta) * [[1, -t], [t, 1]],   t = tan(beta),
+// J = [[0, -1], [1, 0]] (a quarter turn), 45^o the turn by pi/4 (o = 0 or 1),
+// alpha = q pi/2 + o pi/4 + beta and |beta| <= pi/8, so |t| < 0.4143 fits a
+// signed 64-bit fraction T = t 2^64.  A quarter turn exchanges the two
+// amplitudes of a pair: an odd q is kept as a flip of the tile bit (the
+// amplitude of logical index l sits at l ^ F, F the flips so far), its sign in
+// the diagonal table, so that no amplitude moves.  The turn by 45 degrees is
+// done as (x - y, x + y), its scale 1/sqrt(2) in the table like cos(beta).
+struct RotFx {
+    int th, tl;      // T = th 2^32 + tl, both signed
+    uint32_t meta;   // FX_* bits
+    int spare;
+    double gs;       // 1 / (scale of the buffers when this bit's theta gradient is taken)^2
+                     // / 4: the partials have two fraction bits
+};
+
+constexpr uint32_t kFxFlip = 1u;      // q is odd
+constexpr uint32_t kFx45 = 2u;        // o = 1
+constexpr uint32_t kFxBad = 4u;       // an angle of this qubit is not finite
+constexpr uint32_t kFxHalf = 8u;      // the slot's table holds d 2^62 (entries of modulus near 1)
+constexpr int kFxShiftF = 4;          // bits 4-5: shift after the gate, forward
+constexpr int kFxShiftB = 6;          // bits 6-7: shift after the gate, backward
+constexpr int kFxSlotShift = 8;       // bits 8-15: the slot's power of two in its table
+
+constexpr int kFxNormBits = 61;       // |V|_2 <= 2^61 when a tile is loaded
+
+#ifdef __CUDACC__
+
+__device__ __forceinline__ int fx_lo(long long v) { return (int)v; }
+// High half for a signed low half: v = hi 2^32 + lo with lo in [-2^31, 2^31).
+__device__ __forceinline__ int fx_hi(long long v) {
+    return (int)(v >> 32) + (int)((uint32_t)v >> 31);
+}
+
+__device__ __forceinline__ long long fx_madw(int a, int b, long long c) {
+    long long d;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
+    return d;
+}
+
+// a + T b / 2^64, T = th 2^32 + tl and b = bh 2^32 + bl in signed halves.  The
+// two cross products are added exactly (|T| < 2^62.8, |b| < 2^63, so their sum
+// fits 64 bits), rounded at 2^32; tl bl (below half a unit) is left out.
+__device__ __forceinline__ long long fx_ma(long long a, int th, int tl, int bh, int bl) {
+    long long r;
+    asm("{\n"
+        ".reg .s64 m, x, y;\n"
+        ".reg .s32 h, t;\n"
+        "mad.wide.s32 m, %1, %4, 0x80000000;\n"
+        "mad.wide.s32 m, %2, %3, m;\n"
+        "mad.wide.s32 x, %1, %3, %5;\n"
+        "mov.b64 {t, h}, m;\n"
+        "cvt.s64.s32 y, h;\n"
+        "add.s64 %0, x, y;\n"
+        "}"
+        : "=l"(r)
+        : "r"(th), "r"(tl), "r"(bh), "r"(bl), "l"(a));
+    return r;
+}
+
+// (x dr + y di) / 2^63: one component of the product of (x, y) with a table
+// entry d 2^-63.  With |(x, y)| <= 2^(61 + A), |d| = 2^(63 - A) and 0 <= A <= 1
+// the cross products sum to at most 2^62.9; xl dl is left out.
+__device__ __forceinline__ long long fx_dot(int xh, int xl, int drh, int drl, int yh, int yl,
+                                            int dih, int dil) {
+    long long m = fx_madw(xh, drl, 0x40000000ll);
+    m = fx_madw(xl, drh, m);
+    m = fx_madw(yh, dil, m);
+    m = fx_madw(yl, dih, m);
+    long long h = fx_madw(xh, drh, 0ll);
+    h = fx_madw(yh, dih, h);
+    return (h << 1) + (m >> 31);
+}
+
+// a b - c d for values of norm at most 2^61, as h 2^64 + m 2^35 (to about one
+// unit of 2^35; |m| <= 2^59).
+struct FxWide {
+    long long h, m;
+};
+__device__ __forceinline__ FxWide fx_cross(int ah, int al, int bh, int bl, int ch, int cl, int dh,
+                                           int dl) {
+    const long long m1 = fx_madw(al, bh, fx_madw(ah, bl, (long long)__mulhi(al, bl)));
+    const long long m2 = fx_madw(cl, dh, fx_madw(ch, dl, (long long)__mulhi(cl, dl)));
+    return FxWide{fx_madw(ah, bh, 0ll) - fx_madw(ch, dh, 0ll), (m1 - m2) >> 3};
+}
+
+// The double (as bits) x 2^-E to an integer, C = 1085 + E: the mantissa with its leading
+// bit at 62 is shifted right by C - exponent (>= 2).  Zeros, subnormals and
+// what lies below the unit give 0 (or -1: the shift rounds down).
+__device__ __forceinline__ long long fx_from_bits(long long bits, int C) {
+    const int hi = (int)(bits >> 32);
+    const int e = (hi >> 20) & 0x7ff;
+    const long long s = (long long)(hi >> 31);
+    const long long mant = ((bits & 0xfffffffffffffll) | 0x10000000000000ll) << 10;
+    const int r = C - e;
+    return (e == 0 || r > 63) ? 0ll : ((mant ^ s) - s) >> r;
+}
+
+// V 2^E to the bits of the nearest double, E1 = E + 1023 + 62 - 1.  The caller has
+// checked that every exponent a nonzero V can get is a normal one.
+__device__ __forceinline__ long long fx_to_bits(long long v, int E1) {
+    const long long s = v >> 63;
+    unsigned long long u = (unsigned long long)((v ^ s) - s);
+    const int lz = __clzll((long long)u) - 1;   // leading bit to 62
+    u <<= (lz & 63);
+    u = (u + 0x200ull) >> 10;                   // [2^52, 2^53]: the leading bit adds one to the exponent
+    const uint32_t hi = (uint32_t)(u >> 32) + ((uint32_t)(E1 - lz) << 20);
+    const uint32_t sh = hi | ((uint32_t)(s >> 32) & 0x80000000u);
+    const unsigned long long bits = ((unsigned long long)sh << 32) | (uint32_t)u;
+    return v == 0 ? 0ll : (long long)bits;
+}
+
+#endif
+
+}  // namespace vqe

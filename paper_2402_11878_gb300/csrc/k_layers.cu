@@ -345,10 +345,9 @@ struct FixedEntry {
 #define VQE_BWD(TT, RR, ...) \
     FixedEntry{int(2 * sizeof(TT)), RR, true, std::vector<int>{__VA_ARGS__}, &launch_fixed<TT, RR, true, __VA_ARGS__>}
 
-// The pass program shapes of the default plans (tiles of 2^11; FP32 with 16
-// amplitudes per thread: chunks 0, 4, 7; FP64 with 8: chunks 0, 3, 6, 8),
-// forward and backward, and of FP64 plans with 2^12 tiles (chunks 0, 3, 6, 9)
-// as the 32-qubit plan uses them.
+// The pass program shapes of the default FP32 plans (tiles of 2^11 with 16
+// amplitudes per thread: chunks 0, 4, 7), forward and backward.  FP64 plans
+// with 8 amplitudes per thread run in fixed point (k_layers_fx.cu).
 const std::vector<FixedEntry> &fixed_programs() {
     static const std::vector<FixedEntry> table = {
         VQE_FWD(float, 4, VQE_RD(7), VQE_B, VQE_RD(4), VQE_B, VQE_D, VQE_RD(7)),
@@ -358,17 +357,6 @@ const std::vector<FixedEntry> &fixed_programs() {
         VQE_FWD(float, 4, VQE_RD(7), VQE_B, VQE_RD(4), VQE_B, VQE_D, VQE_B, VQE_RD(7), VQE_B, VQE_D),
         VQE_FWD(float, 4, VQE_RD(7), VQE_B, VQE_D, VQE_B, VQE_D),
         VQE_FWD(float, 4, VQE_RD(7), VQE_B, VQE_D),
-        VQE_FWD(double, 3, VQE_RD(8), VQE_B, VQE_RD(6), VQE_B, VQE_RD(3), VQE_B, VQE_D, VQE_RD(8)),
-        VQE_FWD(double, 3, VQE_RD(8), VQE_B, VQE_RD(6), VQE_B, VQE_RD(3), VQE_B, VQE_RD(0), VQE_B,
-                VQE_D, VQE_RD(8)),
-        VQE_FWD(double, 3, VQE_RD(8), VQE_B, VQE_RD(6), VQE_B, VQE_RD(3), VQE_B, VQE_RD(0), VQE_B,
-                VQE_D, VQE_B, VQE_RD(3), VQE_B, VQE_RD(6), VQE_B, VQE_RD(8), VQE_B, VQE_D),
-        VQE_FWD(double, 3, VQE_RD(8), VQE_B, VQE_RD(6), VQE_B, VQE_RD(3), VQE_B, VQE_D, VQE_B,
-                VQE_RD(6), VQE_B, VQE_RD(8), VQE_B, VQE_D),
-        VQE_FWD(double, 3, VQE_RD(8), VQE_B, VQE_RD(6), VQE_B, VQE_D, VQE_B, VQE_RD(8), VQE_B, VQE_D),
-        VQE_FWD(double, 3, VQE_RD(8), VQE_B, VQE_RD(6), VQE_B, VQE_D, VQE_RD(8)),
-        VQE_FWD(double, 3, VQE_RD(8), VQE_B, VQE_D, VQE_B, VQE_D),
-        VQE_FWD(double, 3, VQE_RD(8), VQE_B, VQE_D),
         VQE_BWD(float, 4, VQE_RD(7), VQE_RD(4), VQE_D, VQE_B, VQE_RD(7), VQE_B, VQE_F),
         VQE_BWD(float, 4, VQE_RD(7), VQE_RD(0), VQE_D, VQE_B, VQE_RD(4), VQE_B, VQE_RD(7), VQE_B, VQE_F),
         VQE_BWD(float, 4, VQE_RD(7), VQE_D, VQE_B, VQE_RD(4), VQE_B, VQE_RD(0), VQE_B, VQE_F, VQE_D,
@@ -377,28 +365,6 @@ const std::vector<FixedEntry> &fixed_programs() {
                 VQE_B, VQE_F),
         VQE_BWD(float, 4, VQE_RD(7), VQE_D, VQE_B, VQE_F, VQE_D, VQE_B, VQE_F),
         VQE_BWD(float, 4, VQE_RD(7), VQE_D, VQE_B, VQE_F),
-        VQE_BWD(double, 3, VQE_RD(8), VQE_RD(3), VQE_D, VQE_B, VQE_RD(6), VQE_B, VQE_RD(8), VQE_B, VQE_F),
-        VQE_BWD(double, 3, VQE_RD(8), VQE_RD(0), VQE_D, VQE_B, VQE_RD(3), VQE_B, VQE_RD(6), VQE_B,
-                VQE_RD(8), VQE_B, VQE_F),
-        VQE_BWD(double, 3, VQE_RD(8), VQE_D, VQE_B, VQE_RD(6), VQE_B, VQE_RD(3), VQE_B, VQE_RD(0),
-                VQE_B, VQE_F, VQE_D, VQE_B, VQE_RD(3), VQE_B, VQE_RD(6), VQE_B, VQE_RD(8), VQE_B, VQE_F),
-        VQE_BWD(double, 3, VQE_RD(8), VQE_D, VQE_B, VQE_RD(6), VQE_B, VQE_RD(3), VQE_B, VQE_F, VQE_D,
-                VQE_B, VQE_RD(6), VQE_B, VQE_RD(8), VQE_B, VQE_F),
-        VQE_BWD(double, 3, VQE_RD(8), VQE_D, VQE_B, VQE_RD(6), VQE_B, VQE_F, VQE_D, VQE_B, VQE_RD(8),
-                VQE_B, VQE_F),
-        VQE_BWD(double, 3, VQE_RD(8), VQE_RD(6), VQE_D, VQE_B, VQE_RD(8), VQE_B, VQE_F),
-        VQE_BWD(double, 3, VQE_RD(8), VQE_D, VQE_B, VQE_F, VQE_D, VQE_B, VQE_F),
-        VQE_BWD(double, 3, VQE_RD(8), VQE_D, VQE_B, VQE_F),
-        // FP64 with 2^12-amplitude tiles (512 threads): three qubit groups
-        // instead of four at 32 qubits, so fewer slots (diagonal ops) per layer
-        VQE_FWD(double, 3, VQE_RD(9), VQE_B, VQE_RD(6), VQE_B, VQE_RD(3), VQE_B, VQE_RD(0), VQE_B,
-                VQE_D, VQE_B, VQE_RD(3), VQE_B, VQE_RD(6), VQE_B, VQE_RD(9), VQE_B, VQE_D),
-        VQE_FWD(double, 3, VQE_RD(9), VQE_B, VQE_RD(6), VQE_B, VQE_RD(3), VQE_B, VQE_RD(0), VQE_B,
-                VQE_D, VQE_RD(9)),
-        VQE_BWD(double, 3, VQE_RD(9), VQE_D, VQE_B, VQE_RD(6), VQE_B, VQE_RD(3), VQE_B, VQE_RD(0),
-                VQE_B, VQE_F, VQE_D, VQE_B, VQE_RD(3), VQE_B, VQE_RD(6), VQE_B, VQE_RD(9), VQE_B, VQE_F),
-        VQE_BWD(double, 3, VQE_RD(9), VQE_RD(0), VQE_D, VQE_B, VQE_RD(3), VQE_B, VQE_RD(6), VQE_B,
-                VQE_RD(9), VQE_B, VQE_F),
     };
     return table;
 }
@@ -483,7 +449,15 @@ cudaError_t launch_pass(const PassDesc *desc_dev, const PassDesc &dh, int n_qubi
     switch (dh.R) {
         VQE_PASS_CASE(1)
         VQE_PASS_CASE(2)
-        VQE_PASS_CASE(3)
+        case 3:   // FP64: in fixed point (launch_pass_fx)
+            if constexpr (sizeof(T) == 4)
+                return backward ? launch_pass_r<T, 3, true>(desc_dev, dh, n_qubits, batch, psi, lam, stride,
+                                                            coefs, coef_stride, dtab, dtab_stride, gpart,
+                                                            grad_stride, 0, s)
+                                : launch_pass_r<T, 3, false>(desc_dev, dh, n_qubits, batch, psi, nullptr,
+                                                             stride, coefs, coef_stride, dtab, dtab_stride,
+                                                             gpart, grad_stride, init_zero, s);
+            return cudaErrorInvalidValue;
         VQE_PASS_CASE(4)
         case 5:   // forward only (the backward buffers would not fit in registers)
             if (backward) return cudaErrorInvalidValue;

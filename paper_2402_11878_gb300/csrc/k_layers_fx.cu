@@ -1,0 +1,740 @@
+// FP64 ansatz passes in block fixed point: staging and the tile-pass kernel.
+//
+// Same pass programs, tiles and memory traffic as the floating-point kernels of
+// k_layers.cu: a tile of 2^k amplitudes goes through registers (8 per thread)
+// and shared memory, and a program of rounds, butterflies, diagonals and
+// (backward) flushes runs on it.  The arithmetic is that of fx.cuh: doubles in
+// global memory, 64-bit integers in registers and shared memory.  One compiled
+// body serves every program: the 3 register bits of a round are the same code
+// wherever the round's chunk lies, only the addresses depend on it.
+#include <cstddef>
+
+#include "fx.cuh"
+#include "pass_core.cuh"
+#include "vqe_internal.h"
+
+namespace vqe {
+
+static_assert(sizeof(RotFx) == sizeof(RotCoef<double>), "the coefficient buffer holds either");
+
+namespace {
+
+constexpr int kR = 3, kNR = 8;
+
+// ---------------------------------------------------------------- staging
+
+// Integers scaled by 2^62: every factor of a diagonal table and every scale is
+// made unitary to 2^-60 (one Newton step on the rounded FP64 values) and the
+// products are taken in integers, so a table entry's modulus is exact to about
+// 2^-57; only the angles carry FP64 rounding.
+__device__ __forceinline__ long long mul62(long long a, long long b) { return __mul64hi(a, b) << 2; }
+
+__device__ __forceinline__ longlong2 cmul62(longlong2 a, longlong2 b) {
+    return make_longlong2((__mul64hi(a.x, b.x) - __mul64hi(a.y, b.y)) << 2,
+                          (__mul64hi(a.x, b.y) + __mul64hi(a.y, b.x)) << 2);
+}
+
+// x (1 + r) scaled by 2^62, |x| <= 1, r a small correction
+__device__ __forceinline__ long long to62(double x, double r) {
+    return __double2ll_rn(x * 0x1p62) + __double2ll_rn(x * r * 0x1p62);
+}
+
+// One block per slot and state: coefficients, gradient scales and shift
+// schedule of the slot's gated bits, and the slot's diagonal table
+//   d[l] = 2^S sigma prod_j (phase and quarter-turn sign of bit j of l),
+// sigma the product of the gates' scales, S the shifts made in the slot, so
+// that 1/2 < 2^S sigma <= 1.  The table is the product of one factor for the
+// low and one for the high half of the tile bits.
+__global__ void k_stage_fx(const StageSlot *__restrict__ slots, int n, int depth,
+                           const double *__restrict__ params, RotFx *__restrict__ coefs,
+                           size_t coef_stride, longlong2 *__restrict__ dtab, size_t dtab_stride) {
+    __shared__ longlong2 half_tab[2][1 << (kMaxTileBits / 2)];
+    __shared__ longlong2 d0[kMaxTileBits], d1[kMaxTileBits];
+    __shared__ long long scl[kMaxTileBits];
+    __shared__ double lg[kMaxTileBits];
+    __shared__ RotFx rot[kMaxTileBits];
+    __shared__ long long sigma;   // 2^S sigma
+    __shared__ int table_shift;
+    const StageSlot S = slots[blockIdx.x];
+    const int b = blockIdx.y;
+    const double *pr = params + (size_t)b * (2 * (size_t)n * depth);
+    if (threadIdx.x < (unsigned)S.n_gated) {
+        const int j = threadIdx.x;
+        const int q = S.qubit[j];
+        const double th = pr[((size_t)S.layer * n + q) * 2];
+        const double phi = pr[((size_t)S.layer * n + q) * 2 + 1];
+        double s, c;
+        sincos(0.5 * th, &s, &c);
+        // quarter turns taken off until the angle lies in [-pi/8, 3 pi/8):
+        // the turn nearest pi/8, cos(pi/8) = 0.9239, sin(pi/8) = 0.3827
+        int turns = 0;
+        double best = -2.0, cq = c, sq = s;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const double ct = t == 0 ? c : t == 1 ? s : t == 2 ? -c : -s;
+            const double st = t == 0 ? s : t == 1 ? -c : t == 2 ? -s : c;
+            const double v = 0.9238795325112867 * ct + 0.3826834323650898 * st;
+            if (v > best) {
+                best = v;
+                turns = t;
+                cq = ct;
+                sq = st;
+            }
+        }
+        const bool half_turn = sq > 0.4142135623730950 * cq;
+        const double tt = half_turn ? (sq - cq) / (sq + cq) : sq / cq;
+        // scale 1 / sqrt(1 + t^2), its residual 1 - s^2 (1 + t^2) without rounding
+        const double s0 = 1.0 / sqrt(fma(tt, tt, 1.0));
+        const double p = s0 * s0, pe = fma(s0, s0, -p), u = tt * tt, ue = fma(tt, tt, -u);
+        const double pu = p * u, pue = fma(p, u, -pu);
+        const double res = ((((1.0 - p) - pu) - pue) - pe * (1.0 + u)) - p * ue;
+        long long sc = to62(s0, 0.5 * res);
+        if (half_turn) sc = __mul64hi(sc, 0x5A827999FCEF3242ll) << 1;   // 2^63 / sqrt(2)
+        scl[j] = sc;
+        lg[j] = -log2((double)sc * 0x1p-62);
+        const bool bad = !(isfinite(th) && isfinite(phi));
+        const long long T = bad ? 0ll : __double2ll_rn(tt * 0x1p64);
+        rot[j].tl = fx_lo(T);
+        rot[j].th = fx_hi(T);
+        rot[j].meta = ((turns & 1) ? kFxFlip : 0u) | (half_turn ? kFx45 : 0u) | (bad ? kFxBad : 0u);
+        rot[j].spare = 0;
+        double sp, cp;
+        sincos(0.5 * phi, &sp, &cp);
+        const double c2 = cp * cp, c2e = fma(cp, cp, -c2), s2 = sp * sp, s2e = fma(sp, sp, -s2);
+        const double half_res = 0.5 * ((((1.0 - fmax(c2, s2)) - fmin(c2, s2)) - c2e) - s2e);
+        const long long ci = to62(cp, half_res), si = to62(sp, half_res);
+        // J^q: logical bit 0 takes -1 for q = 1, 2 and bit 1 for q = 2, 3
+        const bool n0 = turns == 1 || turns == 2, n1 = turns >= 2;
+        d0[j] = n0 ? make_longlong2(-ci, si) : make_longlong2(ci, -si);
+        d1[j] = n1 ? make_longlong2(-ci, -si) : make_longlong2(ci, si);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        // shift schedule: A = log2 of the norm's growth since the slot began
+        const int ng = S.n_gated;
+        int order[kMaxTileBits], shb[kMaxTileBits];
+        double A = 0.0;
+        int total = 0;
+        long long sig = 1ll << 62;
+        for (int j = 0; j < ng; ++j) order[__popc(S.fbefore[j])] = j;
+        for (int i = 0; i < ng; ++i) {
+            const int j = order[i];
+            A += lg[j];
+            const int sh = A >= 1.0 ? 1 : 0;   // lg < 0.62: at most one
+            A -= sh;
+            total += sh;
+            sig = mul62(sig, scl[j]) << sh;
+            rot[j].meta |= (uint32_t)sh << kFxShiftF;
+        }
+        const bool near_one = sig > (1ll << 62) - (1ll << 32);
+        sigma = sig;
+        table_shift = near_one ? 0 : 1;
+        for (int j = 0; j < ng; ++j) order[__popc(S.before[j])] = j;
+        A = total;
+        for (int j = 0; j < ng; ++j) A -= lg[j];
+        int done = 0;
+        for (int i = 0; i < ng; ++i) {
+            A += lg[order[i]];
+            int sh = A >= 0.75 && done < total ? 1 : 0;
+            A -= sh;
+            if (i == ng - 1) sh = min(3, total - done);
+            done += sh;
+            shb[i] = sh;
+        }
+        long long f = 1ll << 62;   // scale of the buffers, back from the slot's end
+        for (int i = ng - 1; i >= 0; --i) {
+            const int j = order[i];
+            f = mul62(f, scl[j]) << shb[i];
+            const double fd = (double)f * 0x1p-62;
+            // the theta gradient is taken after the bit's 45-degree turn (x sqrt 2)
+            rot[j].gs = 0.25 / (fd * fd * ((rot[j].meta & kFx45) ? 2.0 : 1.0));
+            rot[j].meta |= ((uint32_t)shb[i] << kFxShiftB) | ((uint32_t)total << kFxSlotShift) |
+                           (near_one ? kFxHalf : 0u);
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < (unsigned)S.n_gated)
+        coefs[(size_t)b * coef_stride + S.coef_off + S.tile_bit[threadIdx.x]] = rot[threadIdx.x];
+    const int kl = S.k >> 1, kh = S.k - kl;
+    for (uint32_t i = threadIdx.x; i < (1u << kl) + (1u << kh); i += blockDim.x) {
+        const bool high = i >= (1u << kl);
+        const uint32_t e = high ? (i - (1u << kl)) << kl : i;
+        longlong2 v = make_longlong2(high ? sigma : 1ll << 62, 0ll);
+        for (int j = 0; j < S.n_gated; ++j)
+            if ((S.tile_bit[j] >= kl) == high)
+                v = cmul62(v, ((e >> S.tile_bit[j]) & 1u) ? d1[j] : d0[j]);
+        half_tab[high][high ? i - (1u << kl) : i] = v;
+    }
+    __syncthreads();
+    longlong2 *tab = dtab + (size_t)b * dtab_stride + S.dtab_off;
+    for (uint32_t l = threadIdx.x; l < (1u << S.k); l += blockDim.x) {
+        const longlong2 v = cmul62(half_tab[0][l & ((1u << kl) - 1u)], half_tab[1][l >> kl]);
+        tab[l] = make_longlong2(v.x << table_shift, v.y << table_shift);
+    }
+}
+
+// ---------------------------------------------------------------- tile pass
+
+struct FxShared {
+    PassDesc d;
+    uint32_t flip[kMaxSlots];      // tile bits with an odd number of quarter turns, per slot
+    uint32_t half[kMaxSlots];      // the slot's table is scaled by 2^62 (kFxHalf)
+    uint32_t wmax[2][16];
+    float wsum[2][16];
+};
+
+// Sum over the lanes of a warp (the low `lanes` of them, a power of two).
+__device__ __forceinline__ long long warp_sum64(long long v, unsigned mask, int lanes) {
+    for (int o = lanes >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
+    return v;
+}
+
+__device__ __forceinline__ uint32_t abs_hi(long long bits) {
+    return (uint32_t)((unsigned long long)bits >> 32) & 0x7fffffffu;
+}
+
+// Doubles to integers in place: the tile's exponent from its largest component
+// and its 2-norm (in FP32 relative to that component: no overflow, no FP64),
+// both block-wide.  E: unit exponent, V = x 2^-E.  bad: the tile holds an
+// infinity or a NaN.
+template <int NB>
+__device__ __forceinline__ void fx_load_tile(long long (&re)[NB][kNR], long long (&im)[NB][kNR],
+                                             FxShared &sh, unsigned wmask, int nwarps, int (&E)[NB],
+                                             bool (&bad)[NB]) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+        uint32_t mx = 0u;
+#pragma unroll
+        for (int r = 0; r < kNR; ++r) mx = max(mx, max(abs_hi(re[u][r]), abs_hi(im[u][r])));
+        mx = __reduce_max_sync(wmask, mx);
+        if (lane == 0) sh.wmax[u][warp] = mx;
+    }
+    __syncthreads();
+    int ef[NB];
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+        uint32_t mx = 0u;
+        for (int w = 0; w < nwarps; ++w) mx = max(mx, sh.wmax[u][w]);
+        ef[u] = (int)(mx >> 20);
+        const int base = (ef[u] - 127) * (1 << 20);
+        float sum = 0.f;
+#pragma unroll
+        for (int r = 0; r < kNR; ++r) {
+            const float x = __int_as_float(max((int)abs_hi(re[u][r]) - base, 0) << 3);
+            const float y = __int_as_float(max((int)abs_hi(im[u][r]) - base, 0) << 3);
+            sum = fmaf(x, x, sum);
+            sum = fmaf(y, y, sum);
+        }
+        for (int o = 16; o > 0; o >>= 1)
+            if ((wmask >> o) & 1u) sum += __shfl_xor_sync(wmask, sum, o);
+        if (lane == 0) sh.wsum[u][warp] = sum;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+        float tot = 0.f;
+        for (int w = 0; w < nwarps; ++w) tot += sh.wsum[u][w];
+        // |tile| < 2^((es + 1) / 2) 2^(ef - 1023); 1.001 covers the truncated mantissas
+        const int es = (int)(__float_as_uint(tot * 1.001f) >> 23) - 127;
+        E[u] = ef[u] - 1023 + ((es + 2) >> 1) - kFxNormBits;
+        bad[u] = ef[u] == 0x7ff;
+        if (ef[u] == 0) E[u] = 0;   // all zero (or subnormal)
+        const int C = 1085 + E[u];
+#pragma unroll
+        for (int r = 0; r < kNR; ++r) {
+            re[u][r] = fx_from_bits(re[u][r], C);
+            im[u][r] = fx_from_bits(im[u][r], C);
+        }
+    }
+}
+
+// One tile bit's gate on the thread's 8 amplitudes of each buffer, register
+// bit J.  Forward: RY; backward: its inverse, and the theta gradient
+//   Re<l1|p0> - Re<l0|p1>
+// of the thread's pairs (buffer 0 = psi, 1 = lambda), in units of 2^62.
+template <int J, bool BWD>
+__device__ __forceinline__ long long fx_gate(long long (&re)[BWD ? 2 : 1][kNR],
+                                             long long (&im)[BWD ? 2 : 1][kNR], const RotFx &c,
+                                             bool neg) {
+    constexpr int NB = BWD ? 2 : 1;
+    if (c.meta & kFx45) {
+#pragma unroll
+        for (int u = 0; u < NB; ++u) {
+#pragma unroll
+            for (int r = 0; r < kNR; ++r) {
+                if (r & (1 << J)) continue;
+                const int r1 = r | (1 << J);
+                const long long a = re[u][r], b = re[u][r1], x = im[u][r], y = im[u][r1];
+                re[u][r] = neg ? a + b : a - b;
+                re[u][r1] = neg ? b - a : a + b;
+                im[u][r] = neg ? x + y : x - y;
+                im[u][r1] = neg ? y - x : x + y;
+            }
+        }
+    }
+    const long long T = ((long long)c.th << 32) + c.tl;
+    const long long Tp = neg ? -T : T, Tn = neg ? T : -T;
+    const int ph = fx_hi(Tp), pl = fx_lo(Tp), nh = fx_hi(Tn), nl = fx_lo(Tn);
+    long long hp = 0, ap = 0, bp = 0, hn = 0, an = 0, bn = 0;
+    int cp = 0, cn = 0;
+#pragma unroll
+    for (int r = 0; r < kNR; ++r) {
+        if (r & (1 << J)) continue;
+        const int r1 = r | (1 << J);
+#pragma unroll
+        for (int c2 = 0; c2 < 2; ++c2) {
+            long long(&v)[NB][kNR] = c2 ? im : re;
+            int xh[NB], xl[NB], yh[NB], yl[NB];
+#pragma unroll
+            for (int u = 0; u < NB; ++u) {
+                xh[u] = fx_hi(v[u][r]);
+                xl[u] = fx_lo(v[u][r]);
+                yh[u] = fx_hi(v[u][r1]);
+                yl[u] = fx_lo(v[u][r1]);
+            }
+            if constexpr (BWD) {
+                hp = fx_madw(yh[1], xh[0], hp);   // l1 p0
+                ap = fx_madw(yh[1], xl[0], ap);
+                bp = fx_madw(yl[1], xh[0], bp);
+                cp += __mulhi(xl[0], yl[1] >> 3);
+                hn = fx_madw(xh[1], yh[0], hn);   // l0 p1
+                an = fx_madw(xh[1], yl[0], an);
+                bn = fx_madw(xl[1], yh[0], bn);
+                cn += __mulhi(yl[0], xl[1] >> 3);
+            }
+#pragma unroll
+            for (int u = 0; u < NB; ++u) {
+                const long long x = v[u][r], y = v[u][r1];
+                v[u][r] = fx_ma(x, nh, nl, yh[u], yl[u]);
+                v[u][r1] = fx_ma(y, ph, pl, xh[u], xl[u]);
+            }
+        }
+    }
+    if constexpr (!BWD) return 0ll;
+    // h 2^64 + (a + b) 2^32 + c 2^35 in units of 2^62
+    const long long lo = ((ap >> 2) - (an >> 2)) + ((bp >> 2) - (bn >> 2)) + 2ll * ((long long)cp - cn);
+    return ((hp - hn) << 2) + ((lo + (1ll << 27)) >> 28);   // rounded: a bias would add up over threads
+}
+
+// The first forward pass when it holds one slot: its only nonzero tile (base
+// 0) starts as |0...0>, so element e of the tile is the product of one factor
+// per tile bit, and the slot's table entry and CZ sign at logical index
+// e ^ flips follow.  In FP64: one tile per state.
+__device__ __forceinline__ void write_product_tile_fx(const PassDesc &d, const RotFx *cf,
+                                                      const longlong2 *tab, uint32_t flips,
+                                                      double2 *P, uint32_t lowmask, int m, int a,
+                                                      int k) {
+    const uint32_t gated = d.slot_gated[0], cz = d.slot_czmask[0];
+    const int slot_shift = gated ? (int)((cf[__ffs(gated) - 1].meta >> kFxSlotShift) & 255u) : 0;
+    const int half = gated ? (int)(cf[__ffs(gated) - 1].meta & kFxHalf) : 0;
+    const double unit = ldexp(1.0, (half ? -62 : -63) - slot_shift);
+    for (uint32_t e = threadIdx.x; e < (1u << k); e += blockDim.x) {
+        double f = unit;
+        bool bad = false;
+        for (int j = 0; j < k; ++j) {
+            const bool bit = (e >> j) & 1u;
+            if (!((gated >> j) & 1u)) {
+                if (bit) f = 0.0;
+                continue;
+            }
+            const RotFx c = cf[j];
+            const double t = ((double)c.th * 0x1p32 + (double)c.tl) * 0x1p-64;
+            if (c.meta & kFx45) f *= bit ? 1.0 + t : 1.0 - t;
+            else if (bit) f *= t;
+            bad |= (c.meta & kFxBad) != 0u;
+        }
+        const uint32_t l = e ^ flips;
+        const uint32_t g = (l & lowmask) | ((l >> m) << a);
+        const longlong2 y = tab[l];
+        const double s = (__popc(g & (g >> 1) & cz) & 1) ? -f : f;
+        const double nan = __longlong_as_double(0x7ff8000000000000ll);
+        P[g] = bad ? make_double2(nan, nan) : make_double2((double)y.x * s, (double)y.y * s);
+    }
+}
+
+// One CTA per (tile, state).  Bound by instruction issue (integer multiplies
+// and their adds).  Against the same passes in FP64 multiply-adds, whole calls:
+// 28-qubit energy + gradient (depth 8) 961 -> 516 ms, 64 energies at 20 qubits
+// (depth 10) 54.6 -> 31.3 ms, gradient at 13 qubits (depth 6) 707 -> 546 us.
+template <bool BWD, int MAXT, int MINB>
+__global__ void __launch_bounds__(MAXT, MINB)
+k_pass_fx(const PassDesc *__restrict__ desc, int init_zero, double2 *__restrict__ psi,
+          double2 *__restrict__ lam, size_t stride, const RotFx *__restrict__ coefs,
+          size_t coef_stride, const longlong2 *__restrict__ dtab, size_t dtab_stride,
+          double *__restrict__ gpart, size_t grad_stride) {
+    constexpr int NB = BWD ? 2 : 1;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ FxShared sh;
+    const int b = blockIdx.y;
+    const uint32_t t = threadIdx.x;
+    const int kk = desc->k;
+    // dynamic shared memory: tile(s) | gradient rows (backward) | coefficient rows
+    const uint32_t size = tile_buf_elems(kk, 16);
+    longlong2 *sbuf = reinterpret_cast<longlong2 *>(smem_raw);
+    long long *rows = reinterpret_cast<long long *>(sbuf + NB * size);
+    RotFx *scf = reinterpret_cast<RotFx *>(rows + (BWD ? (size_t)blockDim.x * (kk + 1 + kR) : 0));
+    {
+        static_assert(sizeof(PassDesc) % 4 == 0, "descriptor copied in words");
+        const uint32_t *src = reinterpret_cast<const uint32_t *>(desc);
+        uint32_t *dst = reinterpret_cast<uint32_t *>(&sh.d);
+        for (int i = t; i < (int)(sizeof(PassDesc) / 4); i += blockDim.x) dst[i] = src[i];
+    }
+    __syncthreads();
+    const PassDesc &d = sh.d;
+    const int k = d.k, m = d.m, a = d.a;
+    int any_bad = 0;
+    for (int i = t; i < d.n_slots * k; i += blockDim.x) {
+        const RotFx c = coefs[(size_t)b * coef_stride + d.slot_coef_off[i / k] + (i % k)];
+        scf[i] = c;
+        if ((d.slot_gated[i / k] >> (i % k)) & 1u) any_bad |= (int)(c.meta & kFxBad);
+    }
+    any_bad = __syncthreads_or(any_bad);
+    for (int s = t; s < d.n_slots; s += blockDim.x) {
+        uint32_t f = 0u, half = 0u;
+        for (int j = 0; j < k; ++j) {
+            if (!((d.slot_gated[s] >> j) & 1u)) continue;
+            const uint32_t meta = scf[s * k + j].meta;
+            if (meta & kFxFlip) f |= 1u << j;
+            half |= meta & kFxHalf;
+        }
+        sh.flip[s] = f;
+        sh.half[s] = half;
+    }
+    const int mid = a - m;
+    const uint32_t lowmask = (1u << m) - 1u;
+    const uint64_t tile = blockIdx.x;
+    const uint64_t base = ((tile & ((1ull << mid) - 1ull)) << m) | ((tile >> mid) << (a + (k - m)));
+    double2 *P = psi + (size_t)b * stride;
+    double2 *L = BWD ? lam + (size_t)b * stride : nullptr;
+    double *gout = BWD ? gpart + (size_t)b * grad_stride : nullptr;
+    const longlong2 *dt = dtab + (size_t)b * dtab_stride;
+    auto g32 = [&](uint32_t e) -> uint32_t {
+        return (uint32_t)(base | (uint64_t)(e & lowmask) | ((uint64_t)(e >> m) << a));
+    };
+    if (base & d.zmask) {   // block-uniform: psi is zero on this tile (see PassDesc::zmask)
+        if (BWD) {
+            for (int i = t; i < d.n_slots * 2 * k; i += blockDim.x)
+                gout[d.slot_grad_off[i / (2 * k)] + tile * (uint64_t)(2 * k) + i % (2 * k)] = 0.0;
+        } else {
+            for (uint32_t e = t; e < (1u << k); e += blockDim.x) P[g32(e)] = make_double2(0.0, 0.0);
+        }
+        return;
+    }
+    __syncthreads();
+    if (!BWD && init_zero && d.n_slots == 1) {   // the tile at base 0
+        write_product_tile_fx(d, scf, dt + d.slot_dtab_off[0], sh.flip[0], P, lowmask, m, a, k);
+        return;
+    }
+    const uint32_t nthr = blockDim.x;   // 2^(k - 3)
+    const int nwarps = (int)((nthr + 31) >> 5);
+    const int warp = t >> 5, lane = t & 31;
+    const unsigned wmask = nthr >= 32 ? 0xffffffffu : ((1u << nthr) - 1u);
+    const int wlanes = nthr >= 32 ? 32 : (int)nthr;
+
+    // Global position of the register bits of a round: tile bit b sits at
+    // global bit b below m and a + b - m above.
+    auto reg_strides = [&](int p, uint32_t (&gs)[kR]) {
+#pragma unroll
+        for (int j = 0; j < kR; ++j) gs[j] = p + j < m ? 1u << (p + j) : 1u << (a + p + j - m);
+    };
+    auto reg_xor = [](int r, const uint32_t (&gs)[kR]) -> uint32_t {
+        uint32_t x = 0u;
+#pragma unroll
+        for (int j = 0; j < kR; ++j)
+            if ((r >> j) & 1) x ^= gs[j];
+        return x;
+    };
+
+    long long re[NB][kNR], im[NB][kNR];
+    int E[NB];
+    bool bad[NB];
+    int chunk = d.ops[0].chunk;
+    {
+        const uint32_t g0 = g32(elem_of(t, 0, chunk, kR));
+        uint32_t gs[kR];
+        reg_strides(chunk, gs);
+        if (!BWD && init_zero) {
+#pragma unroll
+            for (int r = 0; r < kNR; ++r) {
+                re[0][r] = (g0 ^ reg_xor(r, gs)) == 0u ? 1ll << (kFxNormBits - 1) : 0ll;
+                im[0][r] = 0ll;
+            }
+            E[0] = 1 - kFxNormBits;
+            bad[0] = false;
+        } else {
+#pragma unroll
+            for (int r = 0; r < kNR; ++r) {
+                const uint32_t g = g0 ^ reg_xor(r, gs);
+                const longlong2 x = *reinterpret_cast<const longlong2 *>(P + g);
+                re[0][r] = x.x;
+                im[0][r] = x.y;
+                if constexpr (BWD) {
+                    const longlong2 y = *reinterpret_cast<const longlong2 *>(L + g);
+                    re[1][r] = y.x;
+                    im[1][r] = y.y;
+                }
+            }
+            fx_load_tile<NB>(re, im, sh, wmask, nwarps, E, bad);
+        }
+    }
+    const int gexp = 64 + E[0] + E[NB - 1];   // gradient partials: integers scaled by 2^gexp
+    const bool gbad = any_bad || bad[0] || bad[NB - 1];
+    uint32_t F = 0u;          // flips: stored element e holds logical index e ^ F
+    uint32_t Fdiag = 0u;      // F at the last diagonal (phi gradients)
+    int dchunk = 0;
+    for (int oi = 1; oi < d.n_ops; ++oi) {
+        const PassOp op = d.ops[oi];
+        if (op.kind == OP_ROUND) {
+            const int p = op.chunk;
+            uint32_t o[kR];
+            __syncthreads();
+            {
+                longlong2 *bp = sbuf + pad_of<double>(elem_of(t, 0, chunk, kR));
+#pragma unroll
+                for (int j = 0; j < kR; ++j) o[j] = pad_of<double>(1u << (chunk + j));
+#pragma unroll
+                for (int r = 0; r < kNR; ++r) {
+                    const uint32_t x = ((r & 1) ? o[0] : 0u) + ((r & 2) ? o[1] : 0u) + ((r & 4) ? o[2] : 0u);
+#pragma unroll
+                    for (int u = 0; u < NB; ++u) bp[u * size + x] = make_longlong2(re[u][r], im[u][r]);
+                }
+            }
+            __syncthreads();
+            {
+                const longlong2 *bp = sbuf + pad_of<double>(elem_of(t, 0, p, kR));
+#pragma unroll
+                for (int j = 0; j < kR; ++j) o[j] = pad_of<double>(1u << (p + j));
+#pragma unroll
+                for (int r = 0; r < kNR; ++r) {
+                    const uint32_t x = ((r & 1) ? o[0] : 0u) + ((r & 2) ? o[1] : 0u) + ((r & 4) ? o[2] : 0u);
+#pragma unroll
+                    for (int u = 0; u < NB; ++u) {
+                        const longlong2 y = bp[u * size + x];
+                        re[u][r] = y.x;
+                        im[u][r] = y.y;
+                    }
+                }
+            }
+            chunk = p;
+        } else if (op.kind == OP_BF) {
+            auto gate = [&](auto jc) {
+                constexpr int j = decltype(jc)::value;
+                if (!((op.mask >> j) & 1)) return;
+                const RotFx c = scf[op.slot * k + chunk + j];
+                const bool neg = (((F >> (chunk + j)) & 1u) != 0u) != BWD;
+                const long long g = fx_gate<j, BWD>(re, im, c, neg);
+                if constexpr (BWD) rows[(chunk + j) * nthr + t] = g;
+                const int s = (int)((c.meta >> (BWD ? kFxShiftB : kFxShiftF)) & 3u);
+                if (s) {
+#pragma unroll
+                    for (int u = 0; u < NB; ++u) {
+#pragma unroll
+                        for (int r = 0; r < kNR; ++r) {
+                            re[u][r] >>= s;
+                            im[u][r] >>= s;
+                        }
+                    }
+                }
+            };
+            gate(IdxC<0>{});
+            gate(IdxC<1>{});
+            gate(IdxC<2>{});
+        } else if (op.kind == OP_DIAG) {
+            const uint32_t cz = d.slot_czmask[op.slot];
+            if constexpr (!BWD) F ^= sh.flip[op.slot];
+            const uint32_t e0 = elem_of(t, 0, chunk, kR) ^ F;   // logical index of register 0
+            const uint32_t g0 = g32(e0);
+            // CZ signs of the 8 registers as one mask (see run_tile in pass_core.cuh)
+            const uint32_t W = ((g0 & cz) << 1) ^ ((g0 >> 1) & cz);
+            const int lo_cnt = min(max(m - chunk, 0), kR);
+            uint32_t wv = (W >> chunk) & ((1u << lo_cnt) - 1u);
+            if (lo_cnt < kR)
+                wv |= ((W >> (a + max(chunk - m, 0))) & ((1u << (kR - lo_cnt)) - 1u)) << lo_cnt;
+            uint32_t czt = 0u;
+            if (m >= 1) {
+                czt = cz & ((1u << (m - 1)) - 1u);
+                if (a == m && k > m) czt |= cz & (1u << (m - 1));
+            }
+            if (k - m >= 2) czt |= ((cz >> a) & ((1u << (k - m - 1)) - 1u)) << m;
+            const uint32_t adj = czt >> chunk;
+            uint32_t sm = (__popc(g0 & (g0 >> 1) & cz) & 1u) ? 0xffu : 0u;
+#pragma unroll
+            for (int j = 0; j < kR; ++j) {
+                if ((wv >> j) & 1u) sm ^= reg_bit_table(j);
+                if (j + 1 < kR && ((adj >> j) & 1u)) sm ^= reg_bit_table(j) & reg_bit_table(j + 1);
+            }
+            const longlong2 *tab = dt + d.slot_dtab_off[op.slot];
+            const uint32_t half = sh.half[op.slot];   // 2 entries per unit: one more doubling
+            FxWide ua[BWD ? kNR : 1];
+#pragma unroll
+            for (int r = 0; r < kNR; ++r) {
+                const longlong2 e = __ldg(tab + (e0 ^ ((uint32_t)r << chunk)));
+                const long long sg = -(long long)((sm >> r) & 1u);
+                const long long dre = (e.x ^ sg) - sg, dim = (e.y ^ sg) - sg;
+                const int drh = fx_hi(dre), drl = fx_lo(dre), dih = fx_hi(dim), dil = fx_lo(dim);
+                const int dnh = fx_hi(-dim), dnl = fx_lo(-dim);
+                int xh[NB], xl[NB], yh[NB], yl[NB];
+#pragma unroll
+                for (int u = 0; u < NB; ++u) {
+                    xh[u] = fx_hi(re[u][r]);
+                    xl[u] = fx_lo(re[u][r]);
+                    yh[u] = fx_hi(im[u][r]);
+                    yl[u] = fx_lo(im[u][r]);
+                }
+                // dE/dphi_q = Im<l|Z_q|p> = sum_i u_i (-1)^{bit_q(i)}, u = Im(conj(l) p)
+                if constexpr (BWD)
+                    ua[r] = fx_cross(xh[1], xl[1], yh[0], yl[0], yh[1], yl[1], xh[0], xl[0]);
+#pragma unroll
+                for (int u = 0; u < NB; ++u) {
+                    if constexpr (!BWD) {
+                        re[u][r] = fx_dot(xh[u], xl[u], drh, drl, yh[u], yl[u], dnh, dnl);
+                        im[u][r] = fx_dot(xh[u], xl[u], dih, dil, yh[u], yl[u], drh, drl);
+                    } else {
+                        re[u][r] = fx_dot(xh[u], xl[u], drh, drl, yh[u], yl[u], dih, dil);
+                        im[u][r] = fx_dot(xh[u], xl[u], dnh, dnl, yh[u], yl[u], drh, drl);
+                    }
+                }
+            }
+            if (half) {
+#pragma unroll
+                for (int u = 0; u < NB; ++u) {
+#pragma unroll
+                    for (int r = 0; r < kNR; ++r) {
+                        re[u][r] <<= 1;
+                        im[u][r] <<= 1;
+                    }
+                }
+            }
+            if constexpr (BWD) {
+                // the thread's total (row k) and its signed sums over the chunk's
+                // bits (rows k + 1 + j), in units of 2^60; the flush takes the sign
+                // of the other bits from the thread's element base
+                Fdiag = F;
+                dchunk = chunk;
+#pragma unroll
+                for (int j = 0; j < kR; ++j) {
+                    long long dh = 0, dm = 0;
+#pragma unroll
+                    for (int c = 0; c < (kNR >> (j + 1)); ++c) {
+                        const FxWide x0 = ua[2 * c], x1 = ua[2 * c + 1];
+                        dh += x0.h - x1.h;
+                        dm += x0.m - x1.m;
+                        ua[c] = FxWide{x0.h + x1.h, x0.m + x1.m};
+                    }
+                    rows[(k + 1 + j) * nthr + t] = (dh << 4) + ((dm + (1ll << 24)) >> 25);
+                }
+                rows[k * nthr + t] = (ua[0].h << 4) + ((ua[0].m + (1ll << 24)) >> 25);
+                F ^= sh.flip[op.slot];
+            }
+        } else if (BWD) {   // OP_FLUSH: block totals of the slot's gradient partials
+            // Integer sums: exact and independent of their order.
+            __syncthreads();
+            const uint32_t gated = d.slot_gated[op.slot];
+            for (int idx = warp; idx < 2 * k; idx += nwarps) {
+                const int q = idx >> 1;
+                if (!((gated >> q) & 1u)) continue;
+                const bool theta = (idx & 1) == 0;
+                const bool in_chunk = q >= dchunk && q < dchunk + kR;
+                const long long *src = rows + (theta ? q : (in_chunk ? k + 1 + q - dchunk : k)) * nthr;
+                long long sum = 0;
+                for (uint32_t tt = lane; tt < nthr; tt += 32) {
+                    const long long v = src[tt];
+                    const bool flip = !theta && !in_chunk && ((elem_of(tt, 0, dchunk, kR) >> q) & 1u);
+                    sum += flip ? -v : v;
+                }
+                sum = warp_sum64(sum, wmask, wlanes);
+                if (lane == 0) {
+                    const RotFx c = scf[op.slot * k + q];
+                    const bool ng = (((theta ? F : Fdiag) >> q) & 1u) != 0u;
+                    double v = ldexp((double)sum * (theta ? c.gs : 0.0625), gexp);
+                    if (ng) v = -v;
+                    if (gbad) v = __longlong_as_double(0x7ff8000000000000ll);
+                    gout[d.slot_grad_off[op.slot] + tile * (uint64_t)(2 * k) + idx] = v;
+                }
+            }
+            __syncthreads();
+        }
+    }
+    {   // store: logical index e ^ F
+        const uint32_t g0 = g32(elem_of(t, 0, chunk, kR) ^ F);
+        uint32_t gs[kR];
+        reg_strides(chunk, gs);
+#pragma unroll
+        for (int u = 0; u < NB; ++u) {
+            double2 *out = u ? L : P;
+            // every exponent from the unit's to 63 above it is a normal double's
+            const bool plain = E[u] > -1022 && E[u] < 1023 - 64 && !any_bad && !bad[u];
+            if (plain) {
+                const int E1 = E[u] + 1023 + 62 - 1;
+#pragma unroll
+                for (int r = 0; r < kNR; ++r)
+                    *reinterpret_cast<longlong2 *>(out + (g0 ^ reg_xor(r, gs))) =
+                        make_longlong2(fx_to_bits(re[u][r], E1), fx_to_bits(im[u][r], E1));
+            } else {
+                const double nan = __longlong_as_double(0x7ff8000000000000ll);
+                const bool poison = any_bad || bad[u];
+#pragma unroll
+                for (int r = 0; r < kNR; ++r)
+                    out[g0 ^ reg_xor(r, gs)] =
+                        poison ? make_double2(nan, nan)
+                               : make_double2(ldexp((double)re[u][r], E[u]), ldexp((double)im[u][r], E[u]));
+            }
+        }
+    }
+}
+
+template <bool BWD, int MAXT, int MINB>
+cudaError_t launch_k(const PassDesc *desc_dev, const PassDesc &dh, int n_qubits, int batch, void *psi,
+                     void *lam, size_t stride, const RotFx *coefs, size_t coef_stride,
+                     const void *dtab, size_t dtab_stride, double *gpart, size_t grad_stride,
+                     int init_zero, cudaStream_t s) {
+    const int threads = 1 << (dh.k - kR);
+    size_t smem = size_t(tile_buf_elems(dh.k, 16)) * 16 * (BWD ? 2 : 1) +
+                  size_t(dh.n_slots) * dh.k * sizeof(RotFx);
+    if (BWD) smem += size_t(threads) * (dh.k + 1 + kR) * sizeof(long long);
+    auto kern = k_pass_fx<BWD, MAXT, MINB>;
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    dim3 grid((unsigned)(1ull << (n_qubits - dh.k)), batch);
+    kern<<<grid, threads, smem, s>>>(desc_dev, init_zero, static_cast<double2 *>(psi),
+                                     static_cast<double2 *>(lam), stride, coefs, coef_stride,
+                                     static_cast<const longlong2 *>(dtab), dtab_stride, gpart,
+                                     grad_stride);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_stage_fx(const StageSlot *slots_dev, int n_slots, int n_qubits, int depth,
+                            const double *params, int batch, RotFx *coefs, size_t coef_stride,
+                            void *dtab, size_t dtab_stride, cudaStream_t s) {
+    if (n_slots == 0 || batch == 0) return cudaSuccess;
+    dim3 grid(n_slots, batch);
+    k_stage_fx<<<grid, 256, 0, s>>>(slots_dev, n_qubits, depth, params, coefs, coef_stride,
+                                    static_cast<longlong2 *>(dtab), dtab_stride);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pass_fx(const PassDesc *desc_dev, const PassDesc &dh, int n_qubits, int batch,
+                           void *psi, void *lam, size_t stride, const RotFx *coefs,
+                           size_t coef_stride, const void *dtab, size_t dtab_stride, double *gpart,
+                           size_t grad_stride, bool backward, int init_zero, cudaStream_t s) {
+    const int threads = 1 << (dh.k - kR);
+    if (dh.R != kR || threads > 512) return cudaErrorInvalidConfiguration;
+    if (threads <= 256)
+        return backward ? launch_k<true, 256, 2>(desc_dev, dh, n_qubits, batch, psi, lam, stride, coefs,
+                                                 coef_stride, dtab, dtab_stride, gpart, grad_stride, 0, s)
+                        : launch_k<false, 256, 3>(desc_dev, dh, n_qubits, batch, psi, nullptr, stride,
+                                                  coefs, coef_stride, dtab, dtab_stride, gpart,
+                                                  grad_stride, init_zero, s);
+    return backward ? launch_k<true, 512, 1>(desc_dev, dh, n_qubits, batch, psi, lam, stride, coefs,
+                                             coef_stride, dtab, dtab_stride, gpart, grad_stride, 0, s)
+                    : launch_k<false, 512, 1>(desc_dev, dh, n_qubits, batch, psi, nullptr, stride, coefs,
+                                              coef_stride, dtab, dtab_stride, gpart, grad_stride,
+                                              init_zero, s);
+}
+
+}  // namespace vqe

@@ -574,8 +574,8 @@ __device__ __forceinline__ void run_tile_fixed(const PassDesc &d, const PassOp *
                                                typename V2<T>::type *lbuf, double *gsh,
                                                Env &env) {
     static_assert(Env::kLoad == 1 && Env::kStore == 1 && Env::kDiagRow, "direct environment");
-    static_assert(!(BWD && sizeof(T) == 8) || R == 3, "FP64 gradient rows are sized for R = 3");
-    static_assert(!(BWD && sizeof(T) == 4) || R == 4, "FP32 gradient rows are sized for R = 4");
+    static_assert(sizeof(T) == 4, "FP64 plans of fixed shape run in fixed point (k_layers_fx.cu)");
+    static_assert(!BWD || R == 4, "gradient rows are sized for R = 4");
     using C = typename V2<T>::type;
     constexpr int NR = 1 << R;
     constexpr int N = sizeof...(Codes);
@@ -662,64 +662,23 @@ __device__ __forceinline__ void run_tile_fixed(const PassDesc &d, const PassOp *
                 const uint32_t md = (uint32_t)rc.mode;
                 if constexpr (BWD) {
                     // dE/dtheta = Im<l|Y|p>; per pair Re(conj(l1) p0) - Re(conj(l0) p1)
-                    T gt = T(0);
-                    if constexpr (sizeof(T) == 4) {
-                        // packed: both components in f32x2 accumulators, the two
-                        // orientations apart (no negation per pair)
-                        float2 gp = make_float2(0.f, 0.f), gn = make_float2(0.f, 0.f);
+                    // packed: both components in f32x2 accumulators, the two
+                    // orientations apart (no negation per pair)
+                    float2 gp = make_float2(0.f, 0.f), gn = make_float2(0.f, 0.f);
 #pragma unroll
-                        for (int r = 0; r < NR; ++r) {
-                            if (r & (1 << j)) continue;
-                            gp = __ffma2_rn(w[r | (1 << j)], v[r], gp);
-                            gn = __ffma2_rn(w[r], v[r | (1 << j)], gn);
-                        }
-                        gt = (gp.x + gp.y) - (gn.x + gn.y);
-                    } else {
-#pragma unroll
-                        for (int r = 0; r < NR; ++r) {
-                            if (r & (1 << j)) continue;
-                            const C p0 = v[r], p1 = v[r | (1 << j)];
-                            const C l0 = w[r], l1 = w[r | (1 << j)];
-                            gt = fma(l1.x, p0.x, gt);
-                            gt = fma(l1.y, p0.y, gt);
-                            gt = fma(-l0.x, p1.x, gt);
-                            gt = fma(-l0.y, p1.y, gt);
-                        }
+                    for (int r = 0; r < NR; ++r) {
+                        if (r & (1 << j)) continue;
+                        gp = __ffma2_rn(w[r | (1 << j)], v[r], gp);
+                        gn = __ffma2_rn(w[r], v[r | (1 << j)], gn);
                     }
-                    if constexpr (sizeof(T) == 4) {
-                        // FP32: row P + j, already scaled by gs, summed at the flush
-                        reinterpret_cast<float *>(gsh)[(P + j) * nthr + t] = gt * rc.gs;
-                    } else {
-                        // FP64: row P + j of per-thread partials, summed (and scaled by gs)
-                        // at the flush: no shuffle tree per bit on the scarce FP64 pipe
-                        gsh[(P + j) * nthr + t] = gt;
-                    }
+                    const T gt = (gp.x + gp.y) - (gn.x + gn.y);
+                    // row P + j, already scaled by gs, summed at the flush
+                    reinterpret_cast<float *>(gsh)[(P + j) * nthr + t] = gt * rc.gs;
                 }
 #pragma unroll
                 for (int bufi = 0; bufi < (BWD ? 2 : 1); ++bufi) {
                     C *u = bufi ? w : v;
-                    if constexpr (sizeof(T) == 8) {
-#pragma unroll
-                        for (int r = 0; r < NR; ++r) {
-                            if (r & (1 << j)) continue;
-                            const int r1 = r | (1 << j);
-                            const C x = u[r], y = u[r1];
-                            C Pp, Q;
-                            Pp.x = md ? y.x : x.x;  Pp.y = md ? y.y : x.y;
-                            Q.x = md ? x.x : y.x;   Q.y = md ? x.y : y.y;
-                            if (!BWD) {
-                                u[r1].x = fma(cv, Pp.x, Q.x);
-                                u[r1].y = fma(cv, Pp.y, Q.y);
-                                u[r].x = flip_sign(fma(-cv, Q.x, Pp.x), md);
-                                u[r].y = flip_sign(fma(-cv, Q.y, Pp.y), md);
-                            } else {
-                                u[r].x = fma(cv, Q.x, Pp.x);
-                                u[r].y = fma(cv, Q.y, Pp.y);
-                                u[r1].x = flip_sign(fma(-cv, Pp.x, Q.x), md);
-                                u[r1].y = flip_sign(fma(-cv, Pp.y, Q.y), md);
-                            }
-                        }
-                    } else if (md == 0) {
+                    if (md == 0) {
 #pragma unroll
                         for (int r = 0; r < NR; ++r) {
                             if (r & (1 << j)) continue;
@@ -846,7 +805,7 @@ __device__ __forceinline__ void run_tile_fixed(const PassDesc &d, const PassOp *
             static_assert(NT >= 32, "fixed programs run whole warps");
             static_assert(2 * KT <= 32, "one lane per row in the second stage");
             if constexpr (BWD) {
-                using A = typename std::conditional<sizeof(T) == 4, F32c, double>::type;
+                using A = F32c;   // compensated FP32 pairs
                 // stage-2 partials go to the psi tile buffer, free between rounds
                 // (the tile is in registers; the next round exchange starts
                 // with a barrier): 2 KT rows of 33
@@ -869,28 +828,16 @@ __device__ __forceinline__ void run_tile_fixed(const PassDesc &d, const PassOp *
                             const T v = src[tt];
                             return signed_total ? flip_sign(v, (elem_of(tt, 0, dp, R) >> q) & 1u) : v;
                         };
-                        A part;
-                        if constexpr (sizeof(T) == 4) {
-                            part = F32c{term(lane), 0.f};
+                        A part = F32c{term(lane), 0.f};
 #pragma unroll
-                            for (int c = 1; c < NT / 32; ++c) f32c_add(part, term(lane + 32 * c));
-                        } else {
-                            part = term(lane);
-#pragma unroll
-                            for (int c = 1; c < NT / 32; ++c) part += term(lane + 32 * c);
-                        }
+                        for (int c = 1; c < NT / 32; ++c) f32c_add(part, term(lane + 32 * c));
                         sp2[idx * 33 + lane] = part;
                     }
                 };
-                if constexpr (sizeof(T) == 4) {
-                    // one row at a time (its NT / 32 loads together): the
-                    // tile's registers stay live across the flush
+                // one row at a time (its NT / 32 loads together): the
+                // tile's registers stay live across the flush
 #pragma unroll 1
-                    for (int r = 0; r < RPW; ++r) stage1(r);
-                } else {
-#pragma unroll
-                    for (int r = 0; r < RPW; ++r) stage1(r);
-                }
+                for (int r = 0; r < RPW; ++r) stage1(r);
                 __syncthreads();
                 if (warp == 0) {
                     const int idx = lane, q = idx >> 1, comp = idx & 1;
@@ -902,22 +849,11 @@ __device__ __forceinline__ void run_tile_fixed(const PassDesc &d, const PassOp *
 #pragma unroll
                         for (int l = 4; l < 32; l += 4) {
 #pragma unroll
-                            for (int m = 0; m < 4; ++m) {
-                                if constexpr (sizeof(T) == 4) ch[m] = f32c_add_lazy(ch[m], row[l + m]);
-                                else ch[m] += row[l + m];
-                            }
+                            for (int m = 0; m < 4; ++m) ch[m] = f32c_add_lazy(ch[m], row[l + m]);
                         }
-                        A tot;
-                        if constexpr (sizeof(T) == 4)
-                            tot = f32c_add_lazy(f32c_add_lazy(ch[0], ch[1]), f32c_add_lazy(ch[2], ch[3]));
-                        else
-                            tot = (ch[0] + ch[1]) + (ch[2] + ch[3]);
-                        if constexpr (sizeof(T) == 4) {
-                            // theta rows came scaled by gs
-                            env.grad(op.slot, q, comp, f32c_value(tot));
-                        } else {
-                            env.grad(op.slot, q, comp, comp == 0 ? tot * (double)env.coef(op.slot, q).gs : tot);
-                        }
+                        const A tot = f32c_add_lazy(f32c_add_lazy(ch[0], ch[1]), f32c_add_lazy(ch[2], ch[3]));
+                        // theta rows came scaled by gs
+                        env.grad(op.slot, q, comp, f32c_value(tot));
                     }
                 }
                 __syncthreads();

@@ -119,6 +119,7 @@ struct vqe_ctx {
         std::vector<PassDesc> fwd, bwd;
         DevBuf d_fwd, d_bwd, d_stage, d_goff, d_gcnt, d_gstep;
         int n_stage = 0;
+        bool fx = false;   // FP64 passes in block fixed point (k_layers_fx.cu)
         size_t coef_stride = 0, dtab_stride = 0, grad_stride = 0;
         void release() {
             for (DevBuf *b : {&d_fwd, &d_bwd, &d_stage, &d_goff, &d_gcnt, &d_gstep}) b->release();
@@ -512,25 +513,31 @@ bool make_plan(int n, int D, vqe_precision prec, const PlanOptions &opt, HostPla
         emit_forward(d, rounds);
         hp.bwd[p] = d;
         emit_backward(hp.bwd[p], rounds, d.n_slots);
-        // order in which the backward program un-rotates each slot's bits
-        std::vector<uint32_t> done(d.n_slots, 0);
-        std::vector<std::vector<uint16_t>> before(d.n_slots, std::vector<uint16_t>(G.k, 0));
-        int chunk = -1;
-        const PassDesc &bd = hp.bwd[p];
-        for (int oi = 0; oi < bd.n_ops; ++oi) {
-            const PassOp &o = bd.ops[oi];
-            if (o.kind == OP_ROUND) chunk = o.chunk;
-            if (o.kind != OP_BF) continue;
-            for (int j = 0; j < R; ++j) {
-                if (!((o.mask >> j) & 1)) continue;
-                before[o.slot][chunk + j] = uint16_t(done[o.slot]);
-                done[o.slot] |= 1u << (chunk + j);
+        // order in which the programs rotate and un-rotate each slot's bits
+        auto earlier_bits = [&](const PassDesc &pd) {
+            std::vector<uint32_t> done(pd.n_slots, 0);
+            std::vector<std::vector<uint16_t>> before(pd.n_slots, std::vector<uint16_t>(G.k, 0));
+            int chunk = -1;
+            for (int oi = 0; oi < pd.n_ops; ++oi) {
+                const PassOp &o = pd.ops[oi];
+                if (o.kind == OP_ROUND) chunk = o.chunk;
+                if (o.kind != OP_BF) continue;
+                for (int j = 0; j < R; ++j) {
+                    if (!((o.mask >> j) & 1)) continue;
+                    before[o.slot][chunk + j] = uint16_t(done[o.slot]);
+                    done[o.slot] |= 1u << (chunk + j);
+                }
             }
-        }
+            return before;
+        };
+        const auto before = earlier_bits(hp.bwd[p]), fbefore = earlier_bits(d);
         const size_t first_stage = stage.size() - d.n_slots;
         for (int s = 0; s < d.n_slots; ++s) {
             StageSlot &ss = stage[first_stage + s];
-            for (int u = 0; u < ss.n_gated; ++u) ss.before[u] = before[s][ss.tile_bit[u]];
+            for (int u = 0; u < ss.n_gated; ++u) {
+                ss.before[u] = before[s][ss.tile_bit[u]];
+                ss.fbefore[u] = fbefore[s][ss.tile_bit[u]];
+            }
         }
     }
     // Support of the state before each forward pass (it starts from |0...0>):
@@ -606,6 +613,7 @@ vqe_status build_one_plan(vqe_ctx *h, int which) {
     P.dtab_stride = hp.dtab_stride;
     P.grad_stride = hp.grad_stride;
     P.n_stage = int(hp.stage.size());
+    P.fx = h->prec == VQE_C128 && P.fwd[0].R == 3;   // all passes of a plan share R
     h->n_params = hp.n_params;
     vqe_status st;
     if ((st = upload(h, P.d_fwd, P.fwd, "pass plan")) != VQE_OK) return st;
@@ -1702,6 +1710,10 @@ template <typename T>
 cudaError_t launch_any_pass(vqe_ctx *h, const vqe_ctx::DevPlan &P, const PassDesc *dd,
                             const PassDesc &dh, int B, void *psi, void *lam, RotCoef<T> *coefs,
                             double *gpart, bool backward, int init_zero) {
+    if (P.fx)
+        return launch_pass_fx(dd, dh, h->n, B, psi, lam, h->state_elems(),
+                              reinterpret_cast<const RotFx *>(coefs), P.coef_stride, h->d_dtab.p,
+                              P.dtab_stride, gpart, P.grad_stride, backward, init_zero, h->stream);
     return launch_pass<T>(dd, dh, h->n, B, psi, lam, h->state_elems(), coefs, P.coef_stride,
                           h->d_dtab.p, P.dtab_stride, gpart, P.grad_stride, backward, init_zero,
                           h->stream);
@@ -1750,9 +1762,14 @@ vqe_status run_forward(vqe_ctx *h, int which, const double *params_dev, int B, v
     cudaStream_t s = h->stream;
     const vqe_ctx::DevPlan &P = h->plan[which];
     auto *coefs = static_cast<RotCoef<T> *>(h->d_coefs.p);
-    VQE_CUDA(h, launch_stage<T>(static_cast<const StageSlot *>(P.d_stage.p), P.n_stage, h->n,
-                                h->depth, params_dev, B, coefs, P.coef_stride, h->d_dtab.p,
-                                P.dtab_stride, s));
+    const auto *slots = static_cast<const StageSlot *>(P.d_stage.p);
+    if (P.fx)
+        VQE_CUDA(h, launch_stage_fx(slots, P.n_stage, h->n, h->depth, params_dev, B,
+                                    reinterpret_cast<RotFx *>(coefs), P.coef_stride, h->d_dtab.p,
+                                    P.dtab_stride, s));
+    else
+        VQE_CUDA(h, launch_stage<T>(slots, P.n_stage, h->n, h->depth, params_dev, B, coefs,
+                                    P.coef_stride, h->d_dtab.p, P.dtab_stride, s));
     h->stats.kernel_launches++;
     const PassDesc *dd = static_cast<const PassDesc *>(P.d_fwd.p);
     const int mk = prof_begin(h, 0);

@@ -90,6 +90,7 @@ struct StageSlot {
     uint8_t tile_bit[kMaxTileBits];  // gated tile bits
     uint8_t qubit[kMaxTileBits];     // their global qubits
     uint16_t before[kMaxTileBits];   // tile bits un-rotated before this one in the backward sweep
+    uint16_t fbefore[kMaxTileBits];  // tile bits rotated before this one in the forward sweep
 };
 
 // ---------------------------------------------------------------- particle-conserving ansatz
@@ -300,6 +301,18 @@ cudaError_t launch_pass(const PassDesc *desc_dev, const PassDesc &desc_host, int
                         const RotCoef<T> *coefs, size_t coef_stride, const void *dtab,
                         size_t dtab_stride, double *grad_part, size_t grad_stride, bool backward,
                         int init_zero, cudaStream_t s);
+
+// The same in block fixed point (k_layers_fx.cu): FP64 plans with 8 amplitudes
+// per thread (R = 3), with their own coefficients and tables in the same buffers.
+struct RotFx;
+cudaError_t launch_stage_fx(const StageSlot *slots_dev, int n_slots, int n_qubits, int depth,
+                            const double *params, int batch, RotFx *coefs, size_t coef_stride,
+                            void *dtab, size_t dtab_stride, cudaStream_t s);
+cudaError_t launch_pass_fx(const PassDesc *desc_dev, const PassDesc &desc_host, int n_qubits,
+                           int batch, void *psi, void *lam, size_t state_stride, const RotFx *coefs,
+                           size_t coef_stride, const void *dtab, size_t dtab_stride,
+                           double *grad_part, size_t grad_stride, bool backward, int init_zero,
+                           cudaStream_t s);
 
 template <typename T>
 cudaError_t launch_energy(const GroupDesc *groups, int n_groups, const uint32_t *tz,

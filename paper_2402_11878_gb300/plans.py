@@ -41,7 +41,8 @@ class StageSlot(ctypes.Structure):
                 ("dtab_off", ctypes.c_int), ("n_gated", ctypes.c_int),
                 ("tile_bit", ctypes.c_uint8 * K_MAX_TILE_BITS),
                 ("qubit", ctypes.c_uint8 * K_MAX_TILE_BITS),
-                ("before", ctypes.c_uint16 * K_MAX_TILE_BITS)]
+                ("before", ctypes.c_uint16 * K_MAX_TILE_BITS),
+                ("fbefore", ctypes.c_uint16 * K_MAX_TILE_BITS)]
 
 
 class GroupDesc(ctypes.Structure):
