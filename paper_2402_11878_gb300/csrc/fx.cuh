@@ -41,7 +41,7 @@ struct RotFx {
     uint32_t meta;   // FX_* bits
     int spare;
     double gs;       // 1 / (scale of the buffers when this bit's theta gradient is taken)^2
-                     // / 4: the partials have two fraction bits
+                     // / 8: the partials have three fraction bits
 };
 
 constexpr uint32_t kFxFlip = 1u;      // q is odd
@@ -59,7 +59,16 @@ constexpr int kFxNormBits = 61;       // |V|_2 <= 2^61 when a tile is loaded
 __device__ __forceinline__ int fx_lo(long long v) { return (int)v; }
 // High half for a signed low half: v = hi 2^32 + lo with lo in [-2^31, 2^31).
 __device__ __forceinline__ int fx_hi(long long v) {
-    return (int)(v >> 32) + (int)((uint32_t)v >> 31);
+    int h;
+    asm("{\n"
+        ".reg .b32 l, t;\n"
+        "mov.b64 {l, %0}, %1;\n"
+        "shr.u32 t, l, 31;\n"
+        "add.s32 %0, %0, t;\n"
+        "}"
+        : "=r"(h)
+        : "l"(v));
+    return h;
 }
 
 __device__ __forceinline__ long long fx_madw(int a, int b, long long c) {
@@ -68,15 +77,20 @@ __device__ __forceinline__ long long fx_madw(int a, int b, long long c) {
     return d;
 }
 
+__device__ __forceinline__ void fx_acc(long long &c, int a, int b) {
+    asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(c) : "r"(a), "r"(b));
+}
+
 // a + T b / 2^64, T = th 2^32 + tl and b = bh 2^32 + bl in signed halves.  The
 // two cross products are added exactly (|T| < 2^62.8, |b| < 2^63, so their sum
-// fits 64 bits), rounded at 2^32; tl bl (below half a unit) is left out.
+// fits 64 bits) and cut at 2^32; tl bl (below half a unit) is left out.  A
+// rounding constant in the first product costs two more instructions.
 __device__ __forceinline__ long long fx_ma(long long a, int th, int tl, int bh, int bl) {
     long long r;
     asm("{\n"
         ".reg .s64 m, x, y;\n"
         ".reg .s32 h, t;\n"
-        "mad.wide.s32 m, %1, %4, 0x80000000;\n"
+        "mul.wide.s32 m, %1, %4;\n"
         "mad.wide.s32 m, %2, %3, m;\n"
         "mad.wide.s32 x, %1, %3, %5;\n"
         "mov.b64 {t, h}, m;\n"
@@ -93,7 +107,7 @@ __device__ __forceinline__ long long fx_ma(long long a, int th, int tl, int bh, 
 // the cross products sum to at most 2^62.9; xl dl is left out.
 __device__ __forceinline__ long long fx_dot(int xh, int xl, int drh, int drl, int yh, int yl,
                                             int dih, int dil) {
-    long long m = fx_madw(xh, drl, 0x40000000ll);
+    long long m = fx_madw(xh, drl, 0ll);
     m = fx_madw(xl, drh, m);
     m = fx_madw(yh, dil, m);
     m = fx_madw(yl, dih, m);
@@ -114,30 +128,31 @@ __device__ __forceinline__ FxWide fx_cross(int ah, int al, int bh, int bl, int c
     return FxWide{fx_madw(ah, bh, 0ll) - fx_madw(ch, dh, 0ll), (m1 - m2) >> 3};
 }
 
-// The double (as bits) x 2^-E to an integer, C = 1085 + E: the mantissa with its leading
-// bit at 62 is shifted right by C - exponent (>= 2).  Zeros, subnormals and
-// what lies below the unit give 0 (or -1: the shift rounds down).
-__device__ __forceinline__ long long fx_from_bits(long long bits, int C) {
-    const int hi = (int)(bits >> 32);
-    const int e = (hi >> 20) & 0x7ff;
-    const long long s = (long long)(hi >> 31);
-    const long long mant = ((bits & 0xfffffffffffffll) | 0x10000000000000ll) << 10;
-    const int r = C - e;
-    return (e == 0 || r > 63) ? 0ll : ((mant ^ s) - s) >> r;
+// Doubles (as bits) to integers x 2^-E and back.  The exponent is moved by
+// integer adds; the conversions themselves are two FP64-pipe instructions, a
+// pipe that is otherwise idle here (in integer instructions alone a
+// conversion takes about 25 of the issue-bound kind each way).  For
+// -1020 < E < 0, the largest exponent of the tile being E + 1084 at most.
+__device__ __forceinline__ bool fx_plain_exponent(int E) { return E > -960 && E < 0; }
+__device__ __forceinline__ long long fx_from_bits(long long bits, int E) {
+    // a zero becomes 2^(-E - 1023), far below the unit
+    const int hi = (int)(bits >> 32) - E * (1 << 20);
+    return __double2ll_rn(__hiloint2double(hi, (int)bits));
 }
-
-// V 2^E to the bits of the nearest double, E1 = E + 1023 + 62 - 1.  The caller has
-// checked that every exponent a nonzero V can get is a normal one.
-__device__ __forceinline__ long long fx_to_bits(long long v, int E1) {
-    const long long s = v >> 63;
-    unsigned long long u = (unsigned long long)((v ^ s) - s);
-    const int lz = __clzll((long long)u) - 1;   // leading bit to 62
-    u <<= (lz & 63);
-    u = (u + 0x200ull) >> 10;                   // [2^52, 2^53]: the leading bit adds one to the exponent
-    const uint32_t hi = (uint32_t)(u >> 32) + ((uint32_t)(E1 - lz) << 20);
-    const uint32_t sh = hi | ((uint32_t)(s >> 32) & 0x80000000u);
-    const unsigned long long bits = ((unsigned long long)sh << 32) | (uint32_t)u;
-    return v == 0 ? 0ll : (long long)bits;
+__device__ __forceinline__ long long fx_to_bits(long long v, int E) {
+    const double d = __ll2double_rn(v);
+    const int hi = __double2hiint(d);
+    return __double_as_longlong(
+        __hiloint2double(hi == 0 ? 0 : hi + E * (1 << 20), __double2loint(d)));
+}
+// Any E (denormal results are rounded twice).
+__device__ __forceinline__ long long fx_from_bits_any(long long bits, int E) {
+    const double x = __longlong_as_double(bits);
+    const int h = -E / 2;
+    return __double2ll_rn(ldexp(ldexp(x, h), -E - h));
+}
+__device__ __forceinline__ long long fx_to_bits_any(long long v, int E) {
+    return __double_as_longlong(ldexp((double)v, E));
 }
 
 #endif

@@ -134,8 +134,10 @@ __global__ void k_stage_fx(const StageSlot *__restrict__ slots, int n, int depth
         for (int j = 0; j < ng; ++j) A -= lg[j];
         int done = 0;
         for (int i = 0; i < ng; ++i) {
+            // A < 0.75 where the next gate's theta gradient is taken (after its turn)
             A += lg[order[i]];
-            int sh = A >= 0.75 && done < total ? 1 : 0;
+            const double limit = i + 1 < ng && (rot[order[i + 1]].meta & kFx45) ? 0.25 : 0.75;
+            int sh = A >= limit && done < total ? 1 : 0;
             A -= sh;
             if (i == ng - 1) sh = min(3, total - done);
             done += sh;
@@ -147,27 +149,29 @@ __global__ void k_stage_fx(const StageSlot *__restrict__ slots, int n, int depth
             f = mul62(f, scl[j]) << shb[i];
             const double fd = (double)f * 0x1p-62;
             // the theta gradient is taken after the bit's 45-degree turn (x sqrt 2)
-            rot[j].gs = 0.25 / (fd * fd * ((rot[j].meta & kFx45) ? 2.0 : 1.0));
+            rot[j].gs = 0.125 / (fd * fd * ((rot[j].meta & kFx45) ? 2.0 : 1.0));
             rot[j].meta |= ((uint32_t)shb[i] << kFxShiftB) | ((uint32_t)total << kFxSlotShift) |
                            (near_one ? kFxHalf : 0u);
         }
     }
     __syncthreads();
-    if (threadIdx.x < (unsigned)S.n_gated)
-        coefs[(size_t)b * coef_stride + S.coef_off + S.tile_bit[threadIdx.x]] = rot[threadIdx.x];
-    const int kl = S.k >> 1, kh = S.k - kl;
+    // one row per tile bit; the gated bits are the tile's top ones (all of them in
+    // the low group), and the table has no index bits below them
+    const int t0 = S.tile_bit[0], kt = S.k - t0;
+    if (threadIdx.x < (unsigned)S.k)
+        coefs[(size_t)b * coef_stride + S.coef_off + threadIdx.x] =
+            (int)threadIdx.x < t0 ? RotFx{0, 0, 0u, 0, 0.0} : rot[threadIdx.x - t0];
+    const int kl = kt >> 1, kh = kt - kl;
     for (uint32_t i = threadIdx.x; i < (1u << kl) + (1u << kh); i += blockDim.x) {
         const bool high = i >= (1u << kl);
         const uint32_t e = high ? (i - (1u << kl)) << kl : i;
         longlong2 v = make_longlong2(high ? sigma : 1ll << 62, 0ll);
-        for (int j = 0; j < S.n_gated; ++j)
-            if ((S.tile_bit[j] >= kl) == high)
-                v = cmul62(v, ((e >> S.tile_bit[j]) & 1u) ? d1[j] : d0[j]);
+        for (int j = high ? kl : 0; j < (high ? kt : kl); ++j) v = cmul62(v, ((e >> j) & 1u) ? d1[j] : d0[j]);
         half_tab[high][high ? i - (1u << kl) : i] = v;
     }
     __syncthreads();
     longlong2 *tab = dtab + (size_t)b * dtab_stride + S.dtab_off;
-    for (uint32_t l = threadIdx.x; l < (1u << S.k); l += blockDim.x) {
+    for (uint32_t l = threadIdx.x; l < (1u << kt); l += blockDim.x) {
         const longlong2 v = cmul62(half_tab[0][l & ((1u << kl) - 1u)], half_tab[1][l >> kl]);
         tab[l] = make_longlong2(v.x << table_shift, v.y << table_shift);
     }
@@ -175,18 +179,67 @@ __global__ void k_stage_fx(const StageSlot *__restrict__ slots, int n, int depth
 
 // ---------------------------------------------------------------- tile pass
 
+// The parts of a pass that the kernel needs before its shared copy of the
+// descriptor has arrived, by value.
+struct FxHead {
+    int k, m, a, n_ops, n_slots, chunk0;
+    uint32_t zmask, gated;   // every slot of a pass gates the same tile bits
+    int coef0, grad0;        // first slot's offsets; the slots follow one another
+};
+
 struct FxShared {
     PassDesc d;
     uint32_t flip[kMaxSlots];      // tile bits with an odd number of quarter turns, per slot
     uint32_t half[kMaxSlots];      // the slot's table is scaled by 2^62 (kFxHalf)
     uint32_t wmax[2][16];
     float wsum[2][16];
+    long long total[2 * kMaxTileBits];   // block totals of a flush
 };
 
 // Sum over the lanes of a warp (the low `lanes` of them, a power of two).
 __device__ __forceinline__ long long warp_sum64(long long v, unsigned mask, int lanes) {
+    if (lanes == 32) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+    }
     for (int o = lanes >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(mask, v, o);
     return v;
+}
+
+// Block sums of one value per thread (256 threads) with the sign of each of the
+// 8 thread bits, by one warp in one butterfly: entry 2 q + 1 of `out` for thread
+// bit tb, q = tb below the chunk and tb + 3 above.
+__device__ __forceinline__ void total_row_sums(const long long *src, int lane, int chunk, long long *out) {
+    long long v[8], d[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[i] = src[lane + 32 * i];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {   // thread bits 5, 6, 7
+        d[5 + j] = 0;
+#pragma unroll
+        for (int c = 0; c < (8 >> (j + 1)); ++c) {
+            const long long x0 = v[2 * c], x1 = v[2 * c + 1];
+            d[5 + j] += x0 - x1;
+            v[c] = x0 + x1;
+        }
+    }
+    long long s = v[0];
+#pragma unroll
+    for (int b = 0; b < 5; ++b) {
+        const long long o = __shfl_xor_sync(0xffffffffu, s, 1 << b);
+        d[b] = ((lane >> b) & 1) ? o - s : s - o;
+        s += o;
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            if (c < b || c >= 5) d[c] += __shfl_xor_sync(0xffffffffu, d[c], 1 << b);
+    }
+    if (lane < 8) {
+        long long x = d[0];
+#pragma unroll
+        for (int c = 1; c < 8; ++c) x = lane == c ? d[c] : x;
+        out[2 * (lane < chunk ? lane : lane + kR) + 1] = x;
+    }
 }
 
 __device__ __forceinline__ uint32_t abs_hi(long long bits) {
@@ -240,11 +293,18 @@ __device__ __forceinline__ void fx_load_tile(long long (&re)[NB][kNR], long long
         E[u] = ef[u] - 1023 + ((es + 2) >> 1) - kFxNormBits;
         bad[u] = ef[u] == 0x7ff;
         if (ef[u] == 0) E[u] = 0;   // all zero (or subnormal)
-        const int C = 1085 + E[u];
+        if (fx_plain_exponent(E[u])) {
 #pragma unroll
-        for (int r = 0; r < kNR; ++r) {
-            re[u][r] = fx_from_bits(re[u][r], C);
-            im[u][r] = fx_from_bits(im[u][r], C);
+            for (int r = 0; r < kNR; ++r) {
+                re[u][r] = fx_from_bits(re[u][r], E[u]);
+                im[u][r] = fx_from_bits(im[u][r], E[u]);
+            }
+        } else {
+#pragma unroll
+            for (int r = 0; r < kNR; ++r) {
+                re[u][r] = fx_from_bits_any(re[u][r], E[u]);
+                im[u][r] = fx_from_bits_any(im[u][r], E[u]);
+            }
         }
     }
 }
@@ -252,24 +312,32 @@ __device__ __forceinline__ void fx_load_tile(long long (&re)[NB][kNR], long long
 // One tile bit's gate on the thread's 8 amplitudes of each buffer, register
 // bit J.  Forward: RY; backward: its inverse, and the theta gradient
 //   Re<l1|p0> - Re<l0|p1>
-// of the thread's pairs (buffer 0 = psi, 1 = lambda), in units of 2^62.
+// of the thread's pairs (buffer 0 = psi, 1 = lambda), in units of 2^61.
 template <int J, bool BWD>
 __device__ __forceinline__ long long fx_gate(long long (&re)[BWD ? 2 : 1][kNR],
                                              long long (&im)[BWD ? 2 : 1][kNR], const RotFx &c,
                                              bool neg) {
     constexpr int NB = BWD ? 2 : 1;
     if (c.meta & kFx45) {
+        // (x - y, x + y), or (x + y, y - x); the difference as 2x minus the sum,
+        // so that no operand is copied
+        auto turn = [](long long &x, long long &y) {
+            y += x;
+            x = (x + x) - y;
+        };
 #pragma unroll
         for (int u = 0; u < NB; ++u) {
 #pragma unroll
             for (int r = 0; r < kNR; ++r) {
-                if (r & (1 << J)) continue;
-                const int r1 = r | (1 << J);
-                const long long a = re[u][r], b = re[u][r1], x = im[u][r], y = im[u][r1];
-                re[u][r] = neg ? a + b : a - b;
-                re[u][r1] = neg ? b - a : a + b;
-                im[u][r] = neg ? x + y : x - y;
-                im[u][r1] = neg ? y - x : x + y;
+                if ((r & (1 << J)) || neg) continue;
+                turn(re[u][r], re[u][r | (1 << J)]);
+                turn(im[u][r], im[u][r | (1 << J)]);
+            }
+#pragma unroll
+            for (int r = 0; r < kNR; ++r) {
+                if ((r & (1 << J)) || !neg) continue;
+                turn(re[u][r | (1 << J)], re[u][r]);
+                turn(im[u][r | (1 << J)], im[u][r]);
             }
         }
     }
@@ -294,13 +362,13 @@ __device__ __forceinline__ long long fx_gate(long long (&re)[BWD ? 2 : 1][kNR],
                 yl[u] = fx_lo(v[u][r1]);
             }
             if constexpr (BWD) {
-                hp = fx_madw(yh[1], xh[0], hp);   // l1 p0
-                ap = fx_madw(yh[1], xl[0], ap);
-                bp = fx_madw(yl[1], xh[0], bp);
+                fx_acc(hp, yh[1], xh[0]);   // l1 p0
+                fx_acc(ap, yh[1], xl[0]);
+                fx_acc(bp, yl[1], xh[0]);
                 cp += __mulhi(xl[0], yl[1] >> 3);
-                hn = fx_madw(xh[1], yh[0], hn);   // l0 p1
-                an = fx_madw(xh[1], yl[0], an);
-                bn = fx_madw(xl[1], yh[0], bn);
+                fx_acc(hn, xh[1], yh[0]);   // l0 p1
+                fx_acc(an, xh[1], yl[0]);
+                fx_acc(bn, xl[1], yh[0]);
                 cn += __mulhi(yl[0], xl[1] >> 3);
             }
 #pragma unroll
@@ -312,9 +380,12 @@ __device__ __forceinline__ long long fx_gate(long long (&re)[BWD ? 2 : 1][kNR],
         }
     }
     if constexpr (!BWD) return 0ll;
-    // h 2^64 + (a + b) 2^32 + c 2^35 in units of 2^62
-    const long long lo = ((ap >> 2) - (an >> 2)) + ((bp >> 2) - (bn >> 2)) + 2ll * ((long long)cp - cn);
-    return ((hp - hn) << 2) + ((lo + (1ll << 27)) >> 28);   // rounded: a bias would add up over threads
+    // h 2^64 + (a + b) 2^32 + c 2^35 in units of 2^61, rounded (a bias would add
+    // up over the threads).  The norms are at most 2^61.75 here and the 16
+    // high halves of a thread sum to at most 4 times theirs, so ap - an and
+    // bp - bn stay below 2^62.8.
+    const long long lo = ((ap - an) >> 1) + ((bp - bn) >> 1) + 4ll * ((long long)cp - cn);
+    return ((hp - hn) << 3) + ((lo + (1ll << 27)) >> 28);
 }
 
 // The first forward pass when it holds one slot: its only nonzero tile (base
@@ -322,7 +393,7 @@ __device__ __forceinline__ long long fx_gate(long long (&re)[BWD ? 2 : 1][kNR],
 // per tile bit, and the slot's table entry and CZ sign at logical index
 // e ^ flips follow.  In FP64: one tile per state.
 __device__ __forceinline__ void write_product_tile_fx(const PassDesc &d, const RotFx *cf,
-                                                      const longlong2 *tab, uint32_t flips,
+                                                      const longlong2 *tab, int t0, uint32_t flips,
                                                       double2 *P, uint32_t lowmask, int m, int a,
                                                       int k) {
     const uint32_t gated = d.slot_gated[0], cz = d.slot_czmask[0];
@@ -346,20 +417,26 @@ __device__ __forceinline__ void write_product_tile_fx(const PassDesc &d, const R
         }
         const uint32_t l = e ^ flips;
         const uint32_t g = (l & lowmask) | ((l >> m) << a);
-        const longlong2 y = tab[l];
+        const longlong2 y = tab[l >> t0];
         const double s = (__popc(g & (g >> 1) & cz) & 1) ? -f : f;
         const double nan = __longlong_as_double(0x7ff8000000000000ll);
         P[g] = bad ? make_double2(nan, nan) : make_double2((double)y.x * s, (double)y.y * s);
     }
 }
 
-// One CTA per (tile, state).  Bound by instruction issue (integer multiplies
-// and their adds).  Against the same passes in FP64 multiply-adds, whole calls:
-// 28-qubit energy + gradient (depth 8) 961 -> 516 ms, 64 energies at 20 qubits
-// (depth 10) 54.6 -> 31.3 ms, gradient at 13 qubits (depth 6) 707 -> 546 us.
+// One CTA per (tile, state).  A tile's phases (load, conversion, diagonal,
+// gates, exchanges, store) use different pipes, so what counts beside the
+// instructions (backward 760, forward 330 per amplitude in a slot of 7 gates) is
+// how well the CTAs of an SM overlap: 4 forward CTAs of 64 registers (28 qubits:
+// 92.7 ms against 97.2 with 3 of 80), 2 backward ones of 128, few barriers, and
+// loads issued before anything else.  4 or 16 amplitudes per thread instead of 8
+// are slower backward (348 and 375 against 276 ms).
+// Against the same passes in FP64 multiply-adds, whole calls: 28-qubit energy +
+// gradient (depth 8) 961 -> 397 ms, 64 energies at 20 qubits (depth 10) 54.6 ->
+// 24.7 ms, gradient at 13 qubits (depth 6) 706 -> 513 us.
 template <bool BWD, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB)
-k_pass_fx(const PassDesc *__restrict__ desc, int init_zero, double2 *__restrict__ psi,
+k_pass_fx(const FxHead H, const PassDesc *__restrict__ desc, int init_zero, double2 *__restrict__ psi,
           double2 *__restrict__ lam, size_t stride, const RotFx *__restrict__ coefs,
           size_t coef_stride, const longlong2 *__restrict__ dtab, size_t dtab_stride,
           double *__restrict__ gpart, size_t grad_stride) {
@@ -368,69 +445,35 @@ k_pass_fx(const PassDesc *__restrict__ desc, int init_zero, double2 *__restrict_
     __shared__ FxShared sh;
     const int b = blockIdx.y;
     const uint32_t t = threadIdx.x;
-    const int kk = desc->k;
+    const int k = H.k, m = H.m, a = H.a;
     // dynamic shared memory: tile(s) | gradient rows (backward) | coefficient rows
-    const uint32_t size = tile_buf_elems(kk, 16);
+    const uint32_t size = tile_buf_elems(k, 16);
     longlong2 *sbuf = reinterpret_cast<longlong2 *>(smem_raw);
     long long *rows = reinterpret_cast<long long *>(sbuf + NB * size);
-    RotFx *scf = reinterpret_cast<RotFx *>(rows + (BWD ? (size_t)blockDim.x * (kk + 1 + kR) : 0));
-    {
-        static_assert(sizeof(PassDesc) % 4 == 0, "descriptor copied in words");
-        const uint32_t *src = reinterpret_cast<const uint32_t *>(desc);
-        uint32_t *dst = reinterpret_cast<uint32_t *>(&sh.d);
-        for (int i = t; i < (int)(sizeof(PassDesc) / 4); i += blockDim.x) dst[i] = src[i];
-    }
-    __syncthreads();
-    const PassDesc &d = sh.d;
-    const int k = d.k, m = d.m, a = d.a;
-    int any_bad = 0;
-    for (int i = t; i < d.n_slots * k; i += blockDim.x) {
-        const RotFx c = coefs[(size_t)b * coef_stride + d.slot_coef_off[i / k] + (i % k)];
-        scf[i] = c;
-        if ((d.slot_gated[i / k] >> (i % k)) & 1u) any_bad |= (int)(c.meta & kFxBad);
-    }
-    any_bad = __syncthreads_or(any_bad);
-    for (int s = t; s < d.n_slots; s += blockDim.x) {
-        uint32_t f = 0u, half = 0u;
-        for (int j = 0; j < k; ++j) {
-            if (!((d.slot_gated[s] >> j) & 1u)) continue;
-            const uint32_t meta = scf[s * k + j].meta;
-            if (meta & kFxFlip) f |= 1u << j;
-            half |= meta & kFxHalf;
-        }
-        sh.flip[s] = f;
-        sh.half[s] = half;
-    }
+    RotFx *scf = reinterpret_cast<RotFx *>(rows + (BWD ? (size_t)blockDim.x * (k + 1 + kR) : 0));
     const int mid = a - m;
     const uint32_t lowmask = (1u << m) - 1u;
     const uint64_t tile = blockIdx.x;
     const uint64_t base = ((tile & ((1ull << mid) - 1ull)) << m) | ((tile >> mid) << (a + (k - m)));
     double2 *P = psi + (size_t)b * stride;
     double2 *L = BWD ? lam + (size_t)b * stride : nullptr;
-    double *gout = BWD ? gpart + (size_t)b * grad_stride : nullptr;
+    // gradient partials: slot s at s * gridDim.x * 2 k, then tile-major
+    double *gout = BWD ? gpart + (size_t)b * grad_stride + H.grad0 + tile * (uint64_t)(2 * k) : nullptr;
+    const uint64_t gslot = (uint64_t)gridDim.x * (2 * k);
     const longlong2 *dt = dtab + (size_t)b * dtab_stride;
+    const int t0 = __ffs(H.gated) - 1;   // the tables have no index bits below t0
     auto g32 = [&](uint32_t e) -> uint32_t {
         return (uint32_t)(base | (uint64_t)(e & lowmask) | ((uint64_t)(e >> m) << a));
     };
-    if (base & d.zmask) {   // block-uniform: psi is zero on this tile (see PassDesc::zmask)
+    if (base & H.zmask) {   // block-uniform: psi is zero on this tile (see PassDesc::zmask)
         if (BWD) {
-            for (int i = t; i < d.n_slots * 2 * k; i += blockDim.x)
-                gout[d.slot_grad_off[i / (2 * k)] + tile * (uint64_t)(2 * k) + i % (2 * k)] = 0.0;
+            for (int s = 0; s < H.n_slots; ++s)
+                for (int i = t; i < 2 * k; i += blockDim.x) gout[s * gslot + i] = 0.0;
         } else {
             for (uint32_t e = t; e < (1u << k); e += blockDim.x) P[g32(e)] = make_double2(0.0, 0.0);
         }
         return;
     }
-    __syncthreads();
-    if (!BWD && init_zero && d.n_slots == 1) {   // the tile at base 0
-        write_product_tile_fx(d, scf, dt + d.slot_dtab_off[0], sh.flip[0], P, lowmask, m, a, k);
-        return;
-    }
-    const uint32_t nthr = blockDim.x;   // 2^(k - 3)
-    const int nwarps = (int)((nthr + 31) >> 5);
-    const int warp = t >> 5, lane = t & 31;
-    const unsigned wmask = nthr >= 32 ? 0xffffffffu : ((1u << nthr) - 1u);
-    const int wlanes = nthr >= 32 ? 32 : (int)nthr;
 
     // Global position of the register bits of a round: tile bit b sits at
     // global bit b below m and a + b - m above.
@@ -446,49 +489,90 @@ k_pass_fx(const PassDesc *__restrict__ desc, int init_zero, double2 *__restrict_
         return x;
     };
 
+    // the tile's loads first: the descriptor and the coefficients arrive under them.
+    // The state streams past L1, which the tables then stay in.
     long long re[NB][kNR], im[NB][kNR];
-    int E[NB];
-    bool bad[NB];
-    int chunk = d.ops[0].chunk;
+    int chunk = H.chunk0;
     {
         const uint32_t g0 = g32(elem_of(t, 0, chunk, kR));
         uint32_t gs[kR];
         reg_strides(chunk, gs);
-        if (!BWD && init_zero) {
 #pragma unroll
-            for (int r = 0; r < kNR; ++r) {
-                re[0][r] = (g0 ^ reg_xor(r, gs)) == 0u ? 1ll << (kFxNormBits - 1) : 0ll;
+        for (int r = 0; r < kNR; ++r) {
+            const uint32_t g = g0 ^ reg_xor(r, gs);
+            if (!BWD && init_zero) {
+                re[0][r] = g == 0u ? 1ll << (kFxNormBits - 1) : 0ll;
                 im[0][r] = 0ll;
-            }
-            E[0] = 1 - kFxNormBits;
-            bad[0] = false;
-        } else {
-#pragma unroll
-            for (int r = 0; r < kNR; ++r) {
-                const uint32_t g = g0 ^ reg_xor(r, gs);
-                const longlong2 x = *reinterpret_cast<const longlong2 *>(P + g);
+            } else {
+                const longlong2 x = __ldcg(reinterpret_cast<const longlong2 *>(P + g));
                 re[0][r] = x.x;
                 im[0][r] = x.y;
-                if constexpr (BWD) {
-                    const longlong2 y = *reinterpret_cast<const longlong2 *>(L + g);
-                    re[1][r] = y.x;
-                    im[1][r] = y.y;
-                }
             }
-            fx_load_tile<NB>(re, im, sh, wmask, nwarps, E, bad);
+            if constexpr (BWD) {
+                const longlong2 y = __ldcg(reinterpret_cast<const longlong2 *>(L + g));
+                re[1][r] = y.x;
+                im[1][r] = y.y;
+            }
         }
     }
+    {
+        static_assert(sizeof(PassDesc) % 4 == 0, "descriptor copied in words");
+        const uint32_t *src = reinterpret_cast<const uint32_t *>(desc);
+        uint32_t *dst = reinterpret_cast<uint32_t *>(&sh.d);
+        for (int i = t; i < (int)(offsetof(PassDesc, ops) / 4) + H.n_ops; i += blockDim.x) dst[i] = src[i];
+    }
+    const PassDesc &d = sh.d;
+    int any_bad = 0;
+    {
+        const RotFx *src = coefs + (size_t)b * coef_stride + H.coef0;
+        for (int i = t; i < H.n_slots * k; i += blockDim.x) {
+            const RotFx c = src[i];
+            scf[i] = c;
+            any_bad |= (int)(c.meta & kFxBad);
+        }
+    }
+    any_bad = __syncthreads_or(any_bad);
+    for (int s = t; s < H.n_slots; s += blockDim.x) {
+        uint32_t f = 0u;
+        for (int j = t0; j < k; ++j)
+            if (scf[s * k + j].meta & kFxFlip) f |= 1u << j;
+        sh.flip[s] = f;
+        sh.half[s] = scf[s * k + t0].meta & kFxHalf;
+    }
+    if (!BWD && init_zero) {
+        __syncthreads();
+        if (H.n_slots == 1) {   // the tile at base 0
+            write_product_tile_fx(d, scf, dt + d.slot_dtab_off[0], t0, sh.flip[0], P, lowmask, m, a, k);
+            return;
+        }
+    }
+    const uint32_t nthr = blockDim.x;   // 2^(k - 3)
+    const int nwarps = (int)((nthr + 31) >> 5);
+    const int warp = t >> 5, lane = t & 31;
+    const unsigned wmask = nthr >= 32 ? 0xffffffffu : ((1u << nthr) - 1u);
+    const int wlanes = nthr >= 32 ? 32 : (int)nthr;
+
+    int E[NB];
+    bool bad[NB];
+    if (!BWD && init_zero) {
+        E[0] = 1 - kFxNormBits;
+        bad[0] = false;
+    } else {
+        fx_load_tile<NB>(re, im, sh, wmask, nwarps, E, bad);
+    }
     const int gexp = 64 + E[0] + E[NB - 1];   // gradient partials: integers scaled by 2^gexp
+    const bool gplain = gexp > -900 && gexp < 900;
+    const double gscale = gplain ? __hiloint2double((gexp + 1023) * (1 << 20), 0) : 0.0;
     const bool gbad = any_bad || bad[0] || bad[NB - 1];
     uint32_t F = 0u;          // flips: stored element e holds logical index e ^ F
     uint32_t Fdiag = 0u;      // F at the last diagonal (phi gradients)
     int dchunk = 0;
-    for (int oi = 1; oi < d.n_ops; ++oi) {
+    for (int oi = 1; oi < H.n_ops; ++oi) {
         const PassOp op = d.ops[oi];
         if (op.kind == OP_ROUND) {
             const int p = op.chunk;
             uint32_t o[kR];
-            __syncthreads();
+            // no barrier before the write: a thread writes the places it read last
             {
                 longlong2 *bp = sbuf + pad_of<double>(elem_of(t, 0, chunk, kR));
 #pragma unroll
@@ -500,7 +584,10 @@ k_pass_fx(const PassDesc *__restrict__ desc, int init_zero, double2 *__restrict_
                     for (int u = 0; u < NB; ++u) bp[u * size + x] = make_longlong2(re[u][r], im[u][r]);
                 }
             }
-            __syncthreads();
+            // with both chunks at or below 5 the warp's number is tile bits 8 and up
+            // on both sides: the exchange stays inside the warp
+            if (chunk <= 5 && p <= 5) __syncwarp(wmask);
+            else __syncthreads();
             {
                 const longlong2 *bp = sbuf + pad_of<double>(elem_of(t, 0, p, kR));
 #pragma unroll
@@ -569,11 +656,12 @@ k_pass_fx(const PassDesc *__restrict__ desc, int init_zero, double2 *__restrict_
             FxWide ua[BWD ? kNR : 1];
 #pragma unroll
             for (int r = 0; r < kNR; ++r) {
-                const longlong2 e = __ldg(tab + (e0 ^ ((uint32_t)r << chunk)));
+                const longlong2 e = __ldg(tab + ((e0 ^ ((uint32_t)r << chunk)) >> t0));
+                // signs by complement: one unit of 2^-63 off
                 const long long sg = -(long long)((sm >> r) & 1u);
-                const long long dre = (e.x ^ sg) - sg, dim = (e.y ^ sg) - sg;
+                const long long dre = e.x ^ sg, dim = e.y ^ sg, dng = e.y ^ ~sg;
                 const int drh = fx_hi(dre), drl = fx_lo(dre), dih = fx_hi(dim), dil = fx_lo(dim);
-                const int dnh = fx_hi(-dim), dnl = fx_lo(-dim);
+                const int dnh = fx_hi(dng), dnl = fx_lo(dng);
                 int xh[NB], xl[NB], yh[NB], yl[NB];
 #pragma unroll
                 for (int u = 0; u < NB; ++u) {
@@ -630,30 +718,58 @@ k_pass_fx(const PassDesc *__restrict__ desc, int init_zero, double2 *__restrict_
         } else if (BWD) {   // OP_FLUSH: block totals of the slot's gradient partials
             // Integer sums: exact and independent of their order.
             __syncthreads();
-            const uint32_t gated = d.slot_gated[op.slot];
-            for (int idx = warp; idx < 2 * k; idx += nwarps) {
-                const int q = idx >> 1;
-                if (!((gated >> q) & 1u)) continue;
-                const bool theta = (idx & 1) == 0;
-                const bool in_chunk = q >= dchunk && q < dchunk + kR;
-                const long long *src = rows + (theta ? q : (in_chunk ? k + 1 + q - dchunk : k)) * nthr;
-                long long sum = 0;
-                for (uint32_t tt = lane; tt < nthr; tt += 32) {
-                    const long long v = src[tt];
-                    const bool flip = !theta && !in_chunk && ((elem_of(tt, 0, dchunk, kR) >> q) & 1u);
-                    sum += flip ? -v : v;
+            const uint32_t gated = H.gated;
+            if (nthr == 256) {
+                if (warp == 0) {
+                    total_row_sums(rows + k * nthr, lane, dchunk, sh.total);
+                } else {
+                    // the theta rows and the chunk's phi rows
+                    for (int row = warp - 1; row < k + kR; row += 7) {
+                        const int q = row < k ? row : dchunk + row - k;
+                        if (!((gated >> q) & 1u)) continue;
+                        const long long *src = rows + (row < k ? row : row + 1) * 256;
+                        long long sum = src[lane];
+#pragma unroll
+                        for (int i = 1; i < 8; ++i) sum += src[lane + 32 * i];
+                        sum = warp_sum64(sum, wmask, 32);
+                        if (lane == 0) sh.total[2 * q + (row < k ? 0 : 1)] = sum;
+                    }
                 }
-                sum = warp_sum64(sum, wmask, wlanes);
-                if (lane == 0) {
-                    const RotFx c = scf[op.slot * k + q];
-                    const bool ng = (((theta ? F : Fdiag) >> q) & 1u) != 0u;
-                    double v = ldexp((double)sum * (theta ? c.gs : 0.0625), gexp);
-                    if (ng) v = -v;
-                    if (gbad) v = __longlong_as_double(0x7ff8000000000000ll);
-                    gout[d.slot_grad_off[op.slot] + tile * (uint64_t)(2 * k) + idx] = v;
+            } else {
+                for (int idx = warp; idx < 2 * k; idx += nwarps) {
+                    const int q = idx >> 1;
+                    if (!((gated >> q) & 1u)) continue;
+                    const bool theta = (idx & 1) == 0;
+                    const bool in_chunk = q >= dchunk && q < dchunk + kR;
+                    const long long *src = rows + (theta ? q : (in_chunk ? k + 1 + q - dchunk : k)) * nthr;
+                    // phi of a bit outside the chunk: the total row with the sign of
+                    // thread bit tb; bits below 5 are the lane's
+                    const int tb = theta || in_chunk ? -1 : (q < dchunk ? q : q - kR);
+                    const uint32_t imask = tb >= 5 ? 1u << (tb - 5) : 0u;
+                    long long sum = 0;
+                    for (uint32_t i = 0; i < (uint32_t)nwarps; ++i) {
+                        const long long v = src[lane + 32 * i];
+                        sum += (i & imask) ? -v : v;
+                    }
+                    if (tb >= 0 && tb < 5 && ((lane >> tb) & 1)) sum = -sum;
+                    sum = warp_sum64(sum, wmask, wlanes);
+                    if (lane == 0) sh.total[idx] = sum;
                 }
             }
             __syncthreads();
+            // one thread per row: to doubles, scaled
+            if (t < 2u * k || nthr < 2u * k) {
+                for (int idx = t; idx < 2 * k; idx += nthr) {
+                    const int q = idx >> 1;
+                    if (!((gated >> q) & 1u)) continue;
+                    const bool theta = (idx & 1) == 0;
+                    double v = (double)sh.total[idx] * (theta ? scf[op.slot * k + q].gs : 0.0625);
+                    v = gplain ? v * gscale : ldexp(v, gexp);
+                    if (((theta ? F : Fdiag) >> q) & 1u) v = -v;
+                    if (gbad) v = __longlong_as_double(0x7ff8000000000000ll);
+                    gout[op.slot * gslot + idx] = v;
+                }
+            }
         }
     }
     {   // store: logical index e ^ F
@@ -663,22 +779,20 @@ k_pass_fx(const PassDesc *__restrict__ desc, int init_zero, double2 *__restrict_
 #pragma unroll
         for (int u = 0; u < NB; ++u) {
             double2 *out = u ? L : P;
-            // every exponent from the unit's to 63 above it is a normal double's
-            const bool plain = E[u] > -1022 && E[u] < 1023 - 64 && !any_bad && !bad[u];
-            if (plain) {
-                const int E1 = E[u] + 1023 + 62 - 1;
+            if (any_bad || bad[u]) {
+                const double nan = __longlong_as_double(0x7ff8000000000000ll);
+#pragma unroll
+                for (int r = 0; r < kNR; ++r) out[g0 ^ reg_xor(r, gs)] = make_double2(nan, nan);
+            } else if (fx_plain_exponent(E[u])) {
 #pragma unroll
                 for (int r = 0; r < kNR; ++r)
                     *reinterpret_cast<longlong2 *>(out + (g0 ^ reg_xor(r, gs))) =
-                        make_longlong2(fx_to_bits(re[u][r], E1), fx_to_bits(im[u][r], E1));
+                        make_longlong2(fx_to_bits(re[u][r], E[u]), fx_to_bits(im[u][r], E[u]));
             } else {
-                const double nan = __longlong_as_double(0x7ff8000000000000ll);
-                const bool poison = any_bad || bad[u];
 #pragma unroll
                 for (int r = 0; r < kNR; ++r)
-                    out[g0 ^ reg_xor(r, gs)] =
-                        poison ? make_double2(nan, nan)
-                               : make_double2(ldexp((double)re[u][r], E[u]), ldexp((double)im[u][r], E[u]));
+                    *reinterpret_cast<longlong2 *>(out + (g0 ^ reg_xor(r, gs))) =
+                        make_longlong2(fx_to_bits_any(re[u][r], E[u]), fx_to_bits_any(im[u][r], E[u]));
             }
         }
     }
@@ -699,7 +813,9 @@ cudaError_t launch_k(const PassDesc *desc_dev, const PassDesc &dh, int n_qubits,
         if (e != cudaSuccess) return e;
     }
     dim3 grid((unsigned)(1ull << (n_qubits - dh.k)), batch);
-    kern<<<grid, threads, smem, s>>>(desc_dev, init_zero, static_cast<double2 *>(psi),
+    const FxHead head{dh.k, dh.m, dh.a, dh.n_ops, dh.n_slots, dh.ops[0].chunk, dh.zmask,
+                      dh.slot_gated[0], dh.slot_coef_off[0], dh.slot_grad_off[0]};
+    kern<<<grid, threads, smem, s>>>(head, desc_dev, init_zero, static_cast<double2 *>(psi),
                                      static_cast<double2 *>(lam), stride, coefs, coef_stride,
                                      static_cast<const longlong2 *>(dtab), dtab_stride, gpart,
                                      grad_stride);
@@ -727,7 +843,7 @@ cudaError_t launch_pass_fx(const PassDesc *desc_dev, const PassDesc &dh, int n_q
     if (threads <= 256)
         return backward ? launch_k<true, 256, 2>(desc_dev, dh, n_qubits, batch, psi, lam, stride, coefs,
                                                  coef_stride, dtab, dtab_stride, gpart, grad_stride, 0, s)
-                        : launch_k<false, 256, 3>(desc_dev, dh, n_qubits, batch, psi, nullptr, stride,
+                        : launch_k<false, 256, 4>(desc_dev, dh, n_qubits, batch, psi, nullptr, stride,
                                                   coefs, coef_stride, dtab, dtab_stride, gpart,
                                                   grad_stride, init_zero, s);
     return backward ? launch_k<true, 512, 1>(desc_dev, dh, n_qubits, batch, psi, lam, stride, coefs,
