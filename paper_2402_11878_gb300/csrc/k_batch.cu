@@ -8,8 +8,12 @@
 // product is the entry), runs the forward passes, lambda = H psi with the
 // energy, and the adjoint backward passes, accumulating the gradient in
 // shared memory in a fixed order.  An instance whose state fits one tile
-// (all passes span all qubits) never leaves shared memory; larger ones go
-// tile by tile through a per-CTA slice of global memory.
+// (all passes span all qubits) never leaves shared memory; the rounds of larger
+// ones read and write a per-CTA slice of global memory (in L2).  One CTA of 512
+// threads per SM, so barriers and single-threaded sections are what costs: with
+// copies through the tile buffer, two barriers per round and one thread adding
+// up the gradient partials, 512 instances of 12-18 qubits took 34.1 ms instead
+// of 20.8.
 #include "batch_internal.h"
 #include "pass_core.cuh"
 
@@ -20,7 +24,7 @@ namespace {
 template <typename T>
 struct BatchEnv {
     using C = typename V2<T>::type;
-    static constexpr int kLoad = 0, kStore = 0;   // the tile is in shared memory, plain order
+    static constexpr int kLoad = 0;
     const PassDesc *d;
     const RotCoef<T> *coef_s;   // shared: all slots of the instance (plan's coef offsets)
     const C *lo_s;              // shared: per plan slot, 2^kl low half-table entries
@@ -30,6 +34,11 @@ struct BatchEnv {
     double *gacc;               // shared: gradient accumulators (2 n D)
     int n;
     int a, m;
+    // An instance that fits one tile stays in shared memory (plain order); of a
+    // larger one the rounds read and write its slice of global memory.
+    C *P, *L;
+    bool direct;
+    int init_zero;
     __device__ RotCoef<T> coef(int slot, int bit) const { return coef_s[d->slot_coef_off[slot] + bit]; }
     __device__ C diag(int slot, uint32_t e) const {
         const int ps = slot_base[slot];
@@ -191,33 +200,21 @@ k_batch(BatchArgs args) {
                 slot_base[s] = PL.slot_first[p] + s;
             __syncthreads();
             BatchEnv<T> env{&d, coef_s, lo_s, hi_s, slot_base, PL.kl, PL.lo_stride, PL.hi_stride,
-                            gacc, n, d.a, d.m};
+                            gacc, n, d.a, d.m, gpsi, nullptr, !in_smem, p == 0};
             const int k = d.k, m = d.m, a = d.a, mid = a - m;
             const uint64_t tiles = 1ull << (n - k);
             for (uint64_t tile = 0; tile < tiles; ++tile) {
                 const uint64_t base = ((tile & ((1ull << mid) - 1ull)) << m) | ((tile >> mid) << (a + (k - m)));
-                if (!in_smem) {
-                    for (uint32_t e = threadIdx.x; e < (1u << k); e += blockDim.x) {
-                        const uint64_t g = base | (e & ((1u << m) - 1u)) | ((uint64_t)(e >> m) << a);
-                        if (p == 0) {
-                            C z;
-                            z.x = (g == 0) ? T(1) : T(0);
-                            z.y = T(0);
-                            sp[e] = z;
-                        } else {
-                            sp[e] = gpsi[g];
-                        }
+                if (!in_smem && (base & d.zmask)) {   // zero before and after this pass
+                    if (p == 0) {
+                        const C z{};
+                        for (uint32_t e = threadIdx.x; e < (1u << k); e += blockDim.x)
+                            gpsi[base | (e & ((1u << m) - 1u)) | ((uint64_t)(e >> m) << a)] = z;
                     }
-                    __syncthreads();
+                    continue;
                 }
                 run_tile_any<T, false, R4>(d.R, d, base, sp, nullptr, gsh, env);
-                if (!in_smem) {
-                    for (uint32_t e = threadIdx.x; e < (1u << k); e += blockDim.x) {
-                        const uint64_t g = base | (e & ((1u << m) - 1u)) | ((uint64_t)(e >> m) << a);
-                        gpsi[g] = sp[e];
-                    }
-                    __syncthreads();
-                }
+                __syncthreads();   // the next tile starts in the same buffer
             }
         }
 
@@ -275,28 +272,13 @@ k_batch(BatchArgs args) {
                 slot_base[s] = PL.slot_first[p] + s;
             __syncthreads();
             BatchEnv<T> env{&d, coef_s, lo_s, hi_s, slot_base, PL.kl, PL.lo_stride, PL.hi_stride,
-                            gacc, n, d.a, d.m};
+                            gacc, n, d.a, d.m, gpsi, glam, !in_smem, 0};
             const int k = d.k, m = d.m, a = d.a, mid = a - m;
             const uint64_t tiles = 1ull << (n - k);
             for (uint64_t tile = 0; tile < tiles; ++tile) {
                 const uint64_t base = ((tile & ((1ull << mid) - 1ull)) << m) | ((tile >> mid) << (a + (k - m)));
-                if (!in_smem) {
-                    for (uint32_t e = threadIdx.x; e < (1u << k); e += blockDim.x) {
-                        const uint64_t g = base | (e & ((1u << m) - 1u)) | ((uint64_t)(e >> m) << a);
-                        sp[e] = gpsi[g];
-                        sl[e] = glam[g];
-                    }
-                    __syncthreads();
-                }
                 run_tile_any<T, true, R4>(d.R, d, base, sp, sl, gsh, env);
-                if (!in_smem) {
-                    for (uint32_t e = threadIdx.x; e < (1u << k); e += blockDim.x) {
-                        const uint64_t g = base | (e & ((1u << m) - 1u)) | ((uint64_t)(e >> m) << a);
-                        gpsi[g] = sp[e];
-                        glam[g] = sl[e];
-                    }
-                    __syncthreads();
-                }
+                __syncthreads();
             }
         }
         __syncthreads();

@@ -13,16 +13,13 @@
 // The Env policy supplies the per-state data:
 //   RotCoef<T> coef(int slot, int tile_bit)    RY coefficient of a gated bit
 //   C diag(int slot, uint32_t e)               diagonal table entry of tile element e
-//   static constexpr bool kDiagRow  true: the slot's table is stored in full and
-//        const C *diag_row(int slot, uint32_t e0) points at entry e0 (entry e0 + j at [j])
 //   void grad(int slot, int tile_bit, int comp, double v)   (backward) block total of
-//        a gradient partial: comp 0 = theta (RY), 1 = phi (RZ); called by thread 0
+//        a gradient partial: comp 0 = theta (RY), 1 = phi (RZ); called by one thread
+//        per (bit, comp)
 //   static constexpr int kLoad    where the first round reads the tile:
-//        0 = `buf`/`lbuf` in plain order, 1 = the state in global memory
-//        (members P, L and init_zero: start from |0...0>), 2 = `buf`/`lbuf` in
-//        the padded layout of the first round's chunk (a prefetched tile)
-//   static constexpr int kStore   where the last round writes the tile:
-//        0 = `buf`/`lbuf` in plain order, 1 = the state in global memory (P, L)
+//        1 = the state in global memory (members P, L and init_zero: start from
+//        |0...0>), 0 = that where the member `direct` is set, else `buf`/`lbuf`
+//        in plain order; the last round writes to the same place
 #pragma once
 
 #include <type_traits>
@@ -59,30 +56,6 @@ template <typename T> __host__ __device__ constexpr uint32_t pad_of(uint32_t e) 
     return e + (e >> PadShift<T>::value);
 }
 
-// A chunk known only at run time, with the same `value` member as ChunkC: code
-// written against `pc.value` compiles for both (constant-folded for ChunkC).
-struct RtChunk {
-    int value;
-};
-
-// Calls f(std::integral_constant<int, P>) for the runtime chunk p, P in [0, 14 - R].
-template <int R, class F>
-__device__ __forceinline__ void with_chunk(int p, F &&f) {
-    switch (p) {
-#define VQE_CHUNK_CASE(PP) \
-    case PP:               \
-        if constexpr (PP + R <= kMaxTileBits) f(ChunkC<PP>{}); \
-        break;
-        VQE_CHUNK_CASE(0) VQE_CHUNK_CASE(1) VQE_CHUNK_CASE(2) VQE_CHUNK_CASE(3)
-        VQE_CHUNK_CASE(4) VQE_CHUNK_CASE(5) VQE_CHUNK_CASE(6) VQE_CHUNK_CASE(7)
-        VQE_CHUNK_CASE(8) VQE_CHUNK_CASE(9) VQE_CHUNK_CASE(10) VQE_CHUNK_CASE(11)
-        VQE_CHUNK_CASE(12) VQE_CHUNK_CASE(13)
-#undef VQE_CHUNK_CASE
-        default:
-            break;
-    }
-}
-
 __device__ __forceinline__ double flip_sign(double v, uint32_t s) {
     return __longlong_as_double(__double_as_longlong(v) ^ ((unsigned long long)s << 63));
 }
@@ -95,6 +68,14 @@ __device__ __forceinline__ float flip_sign(float v, uint32_t s) {
 __host__ __device__ constexpr uint32_t reg_bit_table(int j) {
     return j == 0 ? 0xAAAAAAAAu : j == 1 ? 0xCCCCCCCCu : j == 2 ? 0xF0F0F0F0u
          : j == 3 ? 0xFF00FF00u : 0xFFFF0000u;
+}
+
+// Barrier between the write and the read of a round change.  Thread bits 5 and
+// up (the warp) hold tile bits 5 + R and up in a round whose chunk starts at 5
+// or below: between two such rounds the exchange stays inside each warp.
+__device__ __forceinline__ void exchange_barrier(int from, int to) {
+    if (from <= 5 && to <= 5) __syncwarp();
+    else __syncthreads();
 }
 
 // a * x + y on both components of a complex value: FP32 issues one packed
@@ -153,124 +134,112 @@ __device__ __forceinline__ void run_tile(const PassDesc &d, const PassOp *ops, i
     C v[NR];
     C w[NR];
 
-    // Global loads (first round) and stores (last round) at compile-time
-    // chunk P: register r holds global index g0 + off_r, off_r the sum of the
-    // global strides of the set bits of r (tile bit b sits at global position
-    // b below m and a + b - m above).  When the chunk lies in the low
-    // contiguous part the offsets are compile-time constants.
-    auto reg_offset = [&](auto pc, int r, const uint32_t (&gst)[R]) -> uint32_t {
-        constexpr int P = decltype(pc)::value;
+    // Global loads (first round) and stores (last round) at chunk p: register r
+    // holds global index g0 + off_r, off_r the sum of the global strides of the
+    // set bits of r (tile bit b sits at global position b below m and a + b - m
+    // above).  Likewise off_r in the padded shared layout.  All chunks share one
+    // body: with one per chunk behind a switch the registers spill.
+    auto reg_offset = [&](int r, const uint32_t (&gst)[R]) -> uint32_t {
         uint32_t off = 0;
 #pragma unroll
         for (int j = 0; j < R; ++j)
-            if ((r >> j) & 1) off += (P + R <= m) ? (1u << (P + j)) : gst[j];
+            if ((r >> j) & 1) off += gst[j];
         return off;
     };
-    auto global_strides = [&](auto pc, uint32_t (&gst)[R]) {
-        constexpr int P = decltype(pc)::value;
+    auto global_strides = [&](int p, uint32_t (&gst)[R]) {
 #pragma unroll
         for (int j = 0; j < R; ++j) {
-            const int bt = P + j;
+            const int bt = p + j;
             gst[j] = bt < m ? (1u << bt) : (1u << (a + bt - m));
         }
     };
-    auto direct_load = [&](auto pc) {
-        if constexpr (Env::kLoad == 1) {
-            constexpr int P = decltype(pc)::value;
-            const uint32_t g0 = g32(elem_of(t, 0, P, R));
-            uint32_t gst[R];
-            global_strides(pc, gst);
-            const C *Pb = env.P + g0;
-            const C *Lb = BWD ? env.L + g0 : nullptr;
+    auto pad_strides = [&](int p, uint32_t (&st)[R]) {
 #pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const uint32_t off = reg_offset(pc, r, gst);
-                if (env.init_zero) {
-                    v[r].x = (g0 + off == 0u) ? T(1) : T(0);
-                    v[r].y = T(0);
-                } else {
-                    v[r] = Pb[off];
-                }
-                if (BWD) w[r] = Lb[off];
+        for (int j = 0; j < R; ++j) st[j] = pad_of<T>(1u << (p + j));
+    };
+    auto direct_load = [&](int p) {
+        const uint32_t g0 = g32(elem_of(t, 0, p, R));
+        uint32_t gst[R];
+        global_strides(p, gst);
+        const C *Pb = env.P + g0;
+        const C *Lb = BWD ? env.L + g0 : nullptr;
+#pragma unroll
+        for (int r = 0; r < NR; ++r) {
+            const uint32_t off = reg_offset(r, gst);
+            if (env.init_zero) {
+                v[r].x = (g0 + off == 0u) ? T(1) : T(0);
+                v[r].y = T(0);
+            } else {
+                v[r] = Pb[off];
             }
+            if (BWD) w[r] = Lb[off];
         }
     };
-    auto direct_store = [&](auto pc) {
-        if constexpr (Env::kStore == 1) {
-            constexpr int P = decltype(pc)::value;
-            const uint32_t g0 = g32(elem_of(t, 0, P, R));
-            uint32_t gst[R];
-            global_strides(pc, gst);
-            C *Pb = env.P + g0;
-            C *Lb = BWD ? env.L + g0 : nullptr;
+    auto direct_store = [&](int p) {
+        const uint32_t g0 = g32(elem_of(t, 0, p, R));
+        uint32_t gst[R];
+        global_strides(p, gst);
+        C *Pb = env.P + g0;
+        C *Lb = BWD ? env.L + g0 : nullptr;
 #pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                const uint32_t off = reg_offset(pc, r, gst);
-                Pb[off] = v[r];
-                if (BWD) Lb[off] = w[r];
-            }
+        for (int r = 0; r < NR; ++r) {
+            const uint32_t off = reg_offset(r, gst);
+            Pb[off] = v[r];
+            if (BWD) Lb[off] = w[r];
         }
     };
+    bool direct = true;
+    if constexpr (Env::kLoad == 0) direct = env.direct;
 
     int chunk = -1;
+    bool first_exchange = true;
     for (int oi = 0; oi < n_ops; ++oi) {
         const PassOp op = ops[oi];
         if (op.kind == OP_ROUND) {
             const int p = op.chunk;
             if (chunk < 0) {
                 if (active) {
-                    auto first_round = [&](auto pc) {
-                        if constexpr (Env::kLoad == 1) {
-                            direct_load(pc);
-                        } else if constexpr (Env::kLoad == 2) {
-                            constexpr int P = decltype(pc)::value;
-                            const uint32_t sb = pad_of<T>(elem_of(t, 0, P, R));
-#pragma unroll
-                            for (int r = 0; r < NR; ++r) {
-                                v[r] = buf[sb + pad_of<T>((uint32_t)r << P)];
-                                if (BWD) w[r] = lbuf[sb + pad_of<T>((uint32_t)r << P)];
-                            }
-                        }
-                    };
-                    if constexpr (Env::kLoad == 0) {   // plain order: one runtime instance
+                    if (direct) {
+                        direct_load(p);
+                    } else {   // plain order
                         const uint32_t e0 = elem_of(t, 0, p, R);
 #pragma unroll
                         for (int r = 0; r < NR; ++r) {
                             v[r] = buf[e0 + ((uint32_t)r << p)];
                             if (BWD) w[r] = lbuf[e0 + ((uint32_t)r << p)];
                         }
-                    } else {
-                        with_chunk<R>(p, first_round);
                     }
                 }
             } else {
-                __syncthreads();
+                // A thread writes the places it read last (the padded places do
+                // not depend on the chunk), so no barrier goes before the write,
+                // except the first after reading a tile in plain order.
+                if (!direct && first_exchange) __syncthreads();
+                first_exchange = false;
                 if (active) {
-                    with_chunk<R>(chunk, [&](auto pc) {
-                        constexpr int P = decltype(pc)::value;
-                        const uint32_t sb = pad_of<T>(elem_of(t, 0, P, R));
-                        C *bp = buf + sb;
-                        C *lp = BWD ? lbuf + sb : nullptr;
+                    const uint32_t sb = pad_of<T>(elem_of(t, 0, chunk, R));
+                    uint32_t st[R];
+                    pad_strides(chunk, st);
+                    C *bp = buf + sb;
+                    C *lp = BWD ? lbuf + sb : nullptr;
 #pragma unroll
-                        for (int r = 0; r < NR; ++r) {
-                            bp[pad_of<T>((uint32_t)r << P)] = v[r];
-                            if (BWD) lp[pad_of<T>((uint32_t)r << P)] = w[r];
-                        }
-                    });
+                    for (int r = 0; r < NR; ++r) {
+                        bp[reg_offset(r, st)] = v[r];
+                        if (BWD) lp[reg_offset(r, st)] = w[r];
+                    }
                 }
-                __syncthreads();
+                exchange_barrier(chunk, p);
                 if (active) {
-                    with_chunk<R>(p, [&](auto pc) {
-                        constexpr int P = decltype(pc)::value;
-                        const uint32_t sb = pad_of<T>(elem_of(t, 0, P, R));
-                        const C *bp = buf + sb;
-                        const C *lp = BWD ? lbuf + sb : nullptr;
+                    const uint32_t sb = pad_of<T>(elem_of(t, 0, p, R));
+                    uint32_t st[R];
+                    pad_strides(p, st);
+                    const C *bp = buf + sb;
+                    const C *lp = BWD ? lbuf + sb : nullptr;
 #pragma unroll
-                        for (int r = 0; r < NR; ++r) {
-                            v[r] = bp[pad_of<T>((uint32_t)r << P)];
-                            if (BWD) w[r] = lp[pad_of<T>((uint32_t)r << P)];
-                        }
-                    });
+                    for (int r = 0; r < NR; ++r) {
+                        v[r] = bp[reg_offset(r, st)];
+                        if (BWD) w[r] = lp[reg_offset(r, st)];
+                    }
                 }
             }
             chunk = p;
@@ -423,90 +392,80 @@ __device__ __forceinline__ void run_tile(const PassDesc &d, const PassOp *ops, i
                 }
             }
             if (active) {
-                // compile-time chunk (constant register offsets) only where the
-                // diagonal is read as full table rows; else one runtime instance
-                auto diag_body = [&](auto pc) {
-                    const int P = pc.value;
-                    const uint32_t e0 = elem_of(t, 0, P, R);
-                    const uint32_t g0 = g32(e0);
-                    // CZ signs of all NR registers as one mask (bit r = register r).
-                    // Register r holds global index g = g0 ^ L_r, L_r the global
-                    // image of r << P, and the CZ chain sign is Q(g) =
-                    // parity(g & (g >> 1) & cz).  Q is quadratic over GF(2):
-                    //   Q(g0 ^ L) = Q(g0) ^ Q(L) ^ parity(L & W),
-                    //   W = ((g0 & cz) << 1) ^ ((g0 >> 1) & cz),
-                    // where parity(L_r & W) is linear in the bits of r (the bits of
-                    // W at the chunk's global positions) and Q(L_r) comes from the
-                    // CZ pairs that join two adjacent bits of the chunk.
-                    uint32_t sm;
-                    {
-                        constexpr uint32_t kFull = NR >= 32 ? 0xffffffffu : ((1u << NR) - 1u);
-                        const uint32_t W = ((g0 & cz) << 1) ^ ((g0 >> 1) & cz);
-                        const int lo_cnt = min(max(m - P, 0), R);
-                        uint32_t wv = (W >> P) & ((1u << lo_cnt) - 1u);
-                        if (lo_cnt < R)
-                            wv |= ((W >> (a + max(P - m, 0))) & ((1u << (R - lo_cnt)) - 1u)) << lo_cnt;
-                        // tile bits b whose qubits b, b+1 are adjacent and CZ-coupled
-                        uint32_t czt = 0u;
-                        if (m >= 1) {
-                            czt = cz & ((1u << (m - 1)) - 1u);
-                            if (a == m && k > m) czt |= cz & (1u << (m - 1));
-                        }
-                        if (k - m >= 2) czt |= ((cz >> a) & ((1u << (k - m - 1)) - 1u)) << m;
-                        const uint32_t adj = czt >> P;
-                        sm = (__popc(g0 & (g0 >> 1) & cz) & 1u) ? kFull : 0u;
-    #pragma unroll
-                        for (int j = 0; j < R; ++j) {
-                            if ((wv >> j) & 1u) sm ^= reg_bit_table(j);
-                            if (j + 1 < R && ((adj >> j) & 1u)) sm ^= reg_bit_table(j) & reg_bit_table(j + 1);
-                        }
-                        sm &= kFull;
+                const int P = chunk;
+                const uint32_t e0 = elem_of(t, 0, P, R);
+                const uint32_t g0 = g32(e0);
+                // CZ signs of all NR registers as one mask (bit r = register r).
+                // Register r holds global index g = g0 ^ L_r, L_r the global
+                // image of r << P, and the CZ chain sign is Q(g) =
+                // parity(g & (g >> 1) & cz).  Q is quadratic over GF(2):
+                //   Q(g0 ^ L) = Q(g0) ^ Q(L) ^ parity(L & W),
+                //   W = ((g0 & cz) << 1) ^ ((g0 >> 1) & cz),
+                // where parity(L_r & W) is linear in the bits of r (the bits of
+                // W at the chunk's global positions) and Q(L_r) comes from the
+                // CZ pairs that join two adjacent bits of the chunk.
+                uint32_t sm;
+                {
+                    constexpr uint32_t kFull = NR >= 32 ? 0xffffffffu : ((1u << NR) - 1u);
+                    const uint32_t W = ((g0 & cz) << 1) ^ ((g0 >> 1) & cz);
+                    const int lo_cnt = min(max(m - P, 0), R);
+                    uint32_t wv = (W >> P) & ((1u << lo_cnt) - 1u);
+                    if (lo_cnt < R)
+                        wv |= ((W >> (a + max(P - m, 0))) & ((1u << (R - lo_cnt)) - 1u)) << lo_cnt;
+                    // tile bits b whose qubits b, b+1 are adjacent and CZ-coupled
+                    uint32_t czt = 0u;
+                    if (m >= 1) {
+                        czt = cz & ((1u << (m - 1)) - 1u);
+                        if (a == m && k > m) czt |= cz & (1u << (m - 1));
                     }
-                        // diagonal entries e0 + (r << P): with a full table, one row
-                    // pointer and constant offsets
+                    if (k - m >= 2) czt |= ((cz >> a) & ((1u << (k - m - 1)) - 1u)) << m;
+                    const uint32_t adj = czt >> P;
+                    sm = (__popc(g0 & (g0 >> 1) & cz) & 1u) ? kFull : 0u;
 #pragma unroll
-                    for (int r = 0; r < NR; ++r) {
-                        const uint32_t sgn = (sm >> r) & 1u;
-                        C dv;
-                        if constexpr (Env::kDiagRow) dv = env.diag_row(op.slot, e0)[(uint32_t)r << P];
-                        else dv = env.diag(op.slot, e0 + ((uint32_t)r << P));
-                        if (!BWD) {
-                            C y = cmul(v[r], dv);
-                            y.x = flip_sign(y.x, sgn);
-                            y.y = flip_sign(y.y, sgn);
-                            v[r] = y;
-                        } else {
-                            C y = cmul_conj(v[r], dv);
-                            y.x = flip_sign(y.x, sgn);
-                            y.y = flip_sign(y.y, sgn);
-                            v[r] = y;
-                            C z = cmul_conj(w[r], dv);
-                            z.x = flip_sign(z.x, sgn);
-                            z.y = flip_sign(z.y, sgn);
-                            w[r] = z;
-                        }
+                    for (int j = 0; j < R; ++j) {
+                        if ((wv >> j) & 1u) sm ^= reg_bit_table(j);
+                        if (j + 1 < R && ((adj >> j) & 1u)) sm ^= reg_bit_table(j) & reg_bit_table(j + 1);
                     }
-                };
-                if constexpr (Env::kDiagRow) with_chunk<R>(chunk, diag_body);
-                else diag_body(RtChunk{chunk});
+                    sm &= kFull;
+                }
+#pragma unroll
+                for (int r = 0; r < NR; ++r) {
+                    const uint32_t sgn = (sm >> r) & 1u;
+                    const C dv = env.diag(op.slot, e0 + ((uint32_t)r << P));
+                    if (!BWD) {
+                        C y = cmul(v[r], dv);
+                        y.x = flip_sign(y.x, sgn);
+                        y.y = flip_sign(y.y, sgn);
+                        v[r] = y;
+                    } else {
+                        C y = cmul_conj(v[r], dv);
+                        y.x = flip_sign(y.x, sgn);
+                        y.y = flip_sign(y.y, sgn);
+                        v[r] = y;
+                        C z = cmul_conj(w[r], dv);
+                        z.x = flip_sign(z.x, sgn);
+                        z.y = flip_sign(z.y, sgn);
+                        w[r] = z;
+                    }
+                }
             }
         } else if (BWD && op.kind == OP_FLUSH) {
             __syncthreads();
             const uint32_t gated = d.slot_gated[op.slot];
             const int used_warps = (int)((nthr + 31) >> 5);
-            if (threadIdx.x == 0) {
-                for (int idx = 0; idx < 2 * k; ++idx) {
-                    if (!((gated >> (idx >> 1)) & 1u)) continue;
-                    double s = 0.0;
-                    for (int wi = 0; wi < used_warps; ++wi) s += gsh[wi * 2 * k + idx];
-                    env.grad(op.slot, idx >> 1, idx & 1, s);
-                }
+            // one thread per total, the warps in order (one thread for all of them
+            // kept the block waiting for 2 k times the warps dependent FP64 adds)
+            for (int idx = threadIdx.x; idx < 2 * k; idx += blockDim.x) {
+                if (!((gated >> (idx >> 1)) & 1u)) continue;
+                double s = 0.0;
+                for (int wi = 0; wi < used_warps; ++wi) s += gsh[wi * 2 * k + idx];
+                env.grad(op.slot, idx >> 1, idx & 1, s);
             }
             __syncthreads();
         }
     }
-    if constexpr (Env::kStore == 1) {
-        if (active) with_chunk<R>(chunk, [&](auto pc) { direct_store(pc); });
+    if (direct) {
+        if (active) direct_store(chunk);
     } else {
         // back to plain order in shared memory
         __syncthreads();
@@ -531,7 +490,9 @@ __device__ __forceinline__ void run_tile(const PassDesc &d, const PassOp *ops, i
 // runs fully unrolled: every chunk is a compile-time constant, the op list is
 // read at constant indices, and no value has to return to a fixed register
 // at an interpreter back-edge.  Forward only, for environments that read and
-// write the state directly (kLoad == 1, kStore == 1) with full diagonal rows.
+// write the state directly (kLoad == 1).  `stage` is called once the tile's loads
+// are on their way: it fills the shared copies of the descriptor and the
+// coefficients and ends with a barrier.
 
 constexpr int prog_round(int chunk) { return 256 | chunk; }
 constexpr int kProgBF = 512, kProgDiag = 768, kProgFlush = 1024;
@@ -568,21 +529,22 @@ __host__ __device__ constexpr int prog_top_chunk() {
     return top;
 }
 
-template <typename T, int R, bool BWD, class Env, int... Codes>
+template <typename T, int R, bool BWD, class Env, class Stage, int... Codes>
 __device__ __forceinline__ void run_tile_fixed(const PassDesc &d, const PassOp *ops, uint64_t gbase,
                                                typename V2<T>::type *buf,
                                                typename V2<T>::type *lbuf, double *gsh,
-                                               Env &env) {
-    static_assert(Env::kLoad == 1 && Env::kStore == 1 && Env::kDiagRow, "direct environment");
+                                               Env &env, Stage &&stage) {
+    static_assert(Env::kLoad == 1, "direct environment");
     static_assert(sizeof(T) == 4, "FP64 plans of fixed shape run in fixed point (k_layers_fx.cu)");
     static_assert(!BWD || R == 4, "gradient rows are sized for R = 4");
     using C = typename V2<T>::type;
     constexpr int NR = 1 << R;
     constexpr int N = sizeof...(Codes);
     constexpr int code[] = {Codes...};
-    const int k = d.k, m = d.m, a = d.a;
+    constexpr int k = prog_top_chunk<Codes...>() + R;
+    const int m = env.m, a = env.a;
     const uint32_t t = threadIdx.x;
-    const uint32_t nthr = 1u << (k - R);   // == blockDim.x for these kernels
+    constexpr uint32_t nthr = 1u << (k - R);   // == blockDim.x for these kernels
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t lowmask = (1u << m) - 1u;
     auto g32 = [&](uint32_t e) -> uint32_t {
@@ -626,13 +588,15 @@ __device__ __forceinline__ void run_tile_fixed(const PassDesc &d, const PassOp *
                     v[r].x = (g0 + off == 0u) ? T(1) : T(0);
                     v[r].y = T(0);
                 } else {
-                    v[r] = Pb[off];
+                    v[r] = __ldcg(Pb + off);   // past L1, which the tables then stay in
                 }
-                if (BWD) w[r] = Lb[off];
+                if (BWD) w[r] = __ldcg(Lb + off);
             }
+            stage();
         } else if constexpr (kind == 1) {       // round change through shared memory
             constexpr int PO = prog_chunk_at<Codes...>(i - 1);
-            __syncthreads();
+            // no barrier before the write: a thread writes the places it read last
+            // (a flush, which uses the psi buffer, ends with a barrier)
             {
                 C *bp = buf + pad_of<T>(elem_of(t, 0, PO, R));
                 C *lp = BWD ? lbuf + pad_of<T>(elem_of(t, 0, PO, R)) : nullptr;
@@ -642,7 +606,7 @@ __device__ __forceinline__ void run_tile_fixed(const PassDesc &d, const PassOp *
                     if (BWD) lp[pad_of<T>((uint32_t)r << PO)] = w[r];
                 }
             }
-            __syncthreads();
+            exchange_barrier(PO, P);
             {
                 const C *bp = buf + pad_of<T>(elem_of(t, 0, P, R));
                 const C *lp = BWD ? lbuf + pad_of<T>(elem_of(t, 0, P, R)) : nullptr;
@@ -768,11 +732,10 @@ __device__ __forceinline__ void run_tile_fixed(const PassDesc &d, const PassOp *
                 if (j + 1 < R && ((adj >> j) & 1u)) sm ^= reg_bit_table(j) & reg_bit_table(j + 1);
             }
             sm &= kFull;
-            const C *drow = env.diag_row(op.slot, e0);
 #pragma unroll
             for (int r = 0; r < NR; ++r) {
                 const uint32_t sgn = (sm >> r) & 1u;
-                const C dv = drow[(uint32_t)r << P];
+                const C dv = env.diag(op.slot, e0 + ((uint32_t)r << P));
                 C y = BWD ? cmul_conj(v[r], dv) : cmul(v[r], dv);
                 y.x = flip_sign(y.x, sgn);
                 y.y = flip_sign(y.y, sgn);
