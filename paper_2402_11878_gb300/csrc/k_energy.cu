@@ -15,6 +15,7 @@
 #include <algorithm>
 
 #include "csum.cuh"
+#include "pdl.cuh"
 #include "vqe_internal.h"
 
 namespace vqe {
@@ -113,6 +114,8 @@ k_energy_cols(const GroupDesc *__restrict__ groups, int n_groups, const uint32_t
               const T *__restrict__ tc, const T *__restrict__ hdiag, int n,
               const typename EV2<T>::type *__restrict__ psi, size_t stride,
               double *__restrict__ partials, int block_off, int bps_total) {
+    pdl_trigger();
+    pdl_wait();
     using C = typename EV2<T>::type;
     constexpr int J = 4;   // pairs per thread and iteration: one load of each term serves J pairs
     __shared__ double sh[2 * (kEnergyThreads / 32)];
@@ -221,6 +224,8 @@ k_apply_h(const GroupDesc *__restrict__ groups, int n_groups, const uint32_t *__
           const T *__restrict__ tc, const T *__restrict__ hdiag, int n,
           const typename EV2<T>::type *__restrict__ psi, typename EV2<T>::type *__restrict__ lam,
           size_t stride, double *__restrict__ partials) {
+    pdl_trigger();
+    pdl_wait();
     using C = typename EV2<T>::type;
     constexpr int J = 4;
     __shared__ double sh[2 * (kEnergyThreads / 32)];
@@ -333,6 +338,8 @@ constexpr int kFinishThreads = 256;
 __global__ void __launch_bounds__(kFinishThreads)
 k_energy_finish(const double *__restrict__ partials, int bps, int batch, double *energies,
                 double *norms, double *unnorm) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ double se[kFinishThreads], sn[kFinishThreads];
     const int b = blockIdx.x;
     const double *p = partials + (size_t)b * bps * 3;
@@ -365,6 +372,8 @@ __global__ void __launch_bounds__(kGradThreads)
 k_grad_finish(const double *__restrict__ part, size_t part_stride, const int *__restrict__ off,
               const int *__restrict__ count, const int *__restrict__ step, int n_params,
               double *grads) {
+    pdl_trigger();
+    pdl_wait();
     __shared__ double sh[kGradThreads];
     const int p = blockIdx.x, b = blockIdx.y;
     const double *src = part + (size_t)b * part_stride + off[p];
@@ -387,12 +396,11 @@ cudaError_t launch_energy(const GroupDesc *groups, int n_groups, const uint32_t 
                           cudaStream_t s) {
     using C = typename EV2<T>::type;
     dim3 grid(bps, batch);
-    k_energy_cols<T><<<grid, kEnergyThreads, 0, s>>>(groups, n_groups, tz,
+    return pdl_launch(k_energy_cols<T>, grid, kEnergyThreads, 0, s, pdl_pays(grid), groups, n_groups, tz,
                                                      reinterpret_cast<const T *>(tc),
                                                      static_cast<const T *>(hdiag), n_qubits,
                                                      static_cast<const C *>(psi), state_stride,
                                                      partials, 0, bps);
-    return cudaGetLastError();
 }
 
 template <typename T>
@@ -402,29 +410,26 @@ cudaError_t launch_apply_h(const GroupDesc *groups, int n_groups, const uint32_t
                            int bps, cudaStream_t s) {
     using C = typename EV2<T>::type;
     dim3 grid(bps, batch);
-    k_apply_h<T><<<grid, kEnergyThreads, 0, s>>>(groups, n_groups, tz,
+    return pdl_launch(k_apply_h<T>, grid, kEnergyThreads, 0, s, pdl_pays(grid), groups, n_groups, tz,
                                                  reinterpret_cast<const T *>(tc),
                                                  static_cast<const T *>(hdiag), n_qubits,
                                                  static_cast<const C *>(psi),
                                                  static_cast<C *>(lam), state_stride, partials);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_energy_finish(const double *partials, int bps, int batch, double *energies,
                                  double *norms, double *unnorm, cudaStream_t s) {
     if (batch <= 0) return cudaSuccess;
-    k_energy_finish<<<batch, kFinishThreads, 0, s>>>(partials, bps, batch, energies, norms,
+    return pdl_launch(k_energy_finish, batch, kFinishThreads, 0, s, pdl_pays(batch), partials, bps, batch, energies, norms,
                                                      unnorm);
-    return cudaGetLastError();
 }
 
 cudaError_t launch_grad_finish(const double *part, size_t part_stride, const int *off,
                                const int *count, const int *step, int n_params, int batch,
                                double *grads, cudaStream_t s) {
     dim3 grid(n_params, batch);
-    k_grad_finish<<<grid, kGradThreads, 0, s>>>(part, part_stride, off, count, step, n_params,
+    return pdl_launch(k_grad_finish, grid, kGradThreads, 0, s, pdl_pays(grid), part, part_stride, off, count, step, n_params,
                                                 grads);
-    return cudaGetLastError();
 }
 
 template cudaError_t launch_energy<float>(const GroupDesc *, int, const uint32_t *, const double *,
@@ -506,6 +511,8 @@ k_energy_win(WinDesc W, const WinGroup *__restrict__ wgroups, const WinTerm *__r
              const uint32_t *__restrict__ hoff, const T *__restrict__ hdiag,
              const typename EV2<T>::type *__restrict__ psi, size_t stride,
              double *__restrict__ partials, int bps_total) {
+    pdl_trigger();
+    pdl_wait();
     using C = typename EV2<T>::type;
     static_assert(kEnergyWinThreads == 512, "pair layout assumes 512 threads");
     constexpr uint32_t size = 1u << K;
@@ -727,6 +734,8 @@ k_apply_h_win(WinDesc W, const WinGroup *__restrict__ wgroups, const WinTerm *__
               const uint32_t *__restrict__ hoff, const T *__restrict__ hdiag,
               const typename EV2<T>::type *__restrict__ psi, typename EV2<T>::type *__restrict__ lam,
               size_t stride, int first, int last, double *__restrict__ partials) {
+    pdl_trigger();
+    pdl_wait();
     using C = typename EV2<T>::type;
     static_assert(kEnergyWinThreads == 512, "pair layout assumes 512 threads");
     constexpr uint32_t size = 1u << K;
@@ -937,10 +946,9 @@ cudaError_t launch_apply_h_win(const WinDesc &W, const WinGroup *wgroups, const 
         if (e != cudaSuccess) return e;
     }
     dim3 grid((unsigned)(1ull << (n_qubits - W.k)), batch);
-    kern<<<grid, kEnergyWinThreads, smem, s>>>(W, wgroups, wterms, hoff, static_cast<const T *>(hdiag),
+    return pdl_launch(kern, grid, kEnergyWinThreads, smem, s, pdl_pays(grid), W, wgroups, wterms, hoff, static_cast<const T *>(hdiag),
                                                static_cast<const C *>(psi), static_cast<C *>(lam),
                                                state_stride, first, last, partials);
-    return cudaGetLastError();
 }
 
 
@@ -961,11 +969,10 @@ cudaError_t launch_energy_win(const WinDesc &W, const WinGroup *wgroups, const W
         if (e != cudaSuccess) return e;
     }
     dim3 grid((unsigned)(1ull << (n_qubits - W.k)), batch);
-    kern<<<grid, kEnergyWinThreads, smem, s>>>(W, wgroups, wterms, hoff,
+    return pdl_launch(kern, grid, kEnergyWinThreads, smem, s, pdl_pays(grid), W, wgroups, wterms, hoff,
                                                static_cast<const T *>(hdiag),
                                                static_cast<const C *>(psi), state_stride,
                                                partials, bps_total);
-    return cudaGetLastError();
 }
 
 // Global-sweep expectation for a subset of groups, writing its block partials
@@ -977,11 +984,10 @@ cudaError_t launch_energy_sub(const GroupDesc *groups, int n_groups, const uint3
                               int bps_total, cudaStream_t s) {
     using C = typename EV2<T>::type;
     dim3 grid(bps, batch);
-    k_energy_cols<T><<<grid, kEnergyThreads, 0, s>>>(groups, n_groups, tz,
+    return pdl_launch(k_energy_cols<T>, grid, kEnergyThreads, 0, s, pdl_pays(grid), groups, n_groups, tz,
                                                      reinterpret_cast<const T *>(tc), nullptr,
                                                      n_qubits, static_cast<const C *>(psi),
                                                      state_stride, partials, block_off, bps_total);
-    return cudaGetLastError();
 }
 
 template cudaError_t launch_apply_h_win<float>(const WinDesc &, const WinGroup *, const WinTerm *,

@@ -21,6 +21,7 @@
 //     dE/dtheta_g = 2 Re <lambda| G_g |psi>,  G_g = T_g - T_g^dag,
 // per pair sgn * (Re conj(lambda_j') psi_j - Re conj(lambda_j) psi_j').
 #include "csum.cuh"
+#include "pdl.cuh"
 #include "vqe_internal.h"
 
 namespace vqe {
@@ -33,6 +34,7 @@ constexpr int kExcMaxHigh = 8;   // k - m <= 8: 256 high-part offsets per pass
 
 template <typename T>
 __global__ void k_exc_stage(const double *__restrict__ params, int total, T *__restrict__ cs) {
+    pdl_trigger();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= total) return;
     double s, c;
@@ -87,17 +89,30 @@ k_exc_pass(ExcPass P, const ExcGate *__restrict__ gates, const uint32_t *__restr
     const int b = blockIdx.y;
     C *Pp = psi + (size_t)b * stride;
     C *Lp = BWD ? lam + (size_t)b * stride : nullptr;
-    uint64_t base = 0;
+    uint64_t base = 0;   // the tile number's bits at the bits of bmask, run by run
     {
         uint32_t bm = P.bmask;
         uint64_t tn = blockIdx.x;
         while (bm) {
-            const int bit = __ffs(bm) - 1;
-            base |= (tn & 1ull) << bit;
-            tn >>= 1;
-            bm &= bm - 1u;
+            const int lo = __ffs(bm) - 1;
+            const uint32_t up = bm >> lo;                       // run of ones from bit 0
+            const int len = up == 0xffffffffu ? 32 : __ffs(~up) - 1;
+            const uint64_t run = (1ull << len) - 1ull;
+            base |= (tn & run) << lo;
+            tn >>= len;
+            bm &= ~(uint32_t)(run << lo);
         }
     }
+    // the plan's tables do not depend on earlier kernels; they are on their way
+    // while the block waits
+    pdl_trigger();
+    static_assert(kExcMaxGates <= kExcThreads && (1 << kExcMaxHigh) <= kExcThreads, "one entry per thread");
+    const uint32_t nh = 1u << (k - m);
+    ExcGate my_gate;
+    uint32_t my_off = 0u;
+    if ((int)tid < ng) my_gate = gates[P.g_begin + tid];
+    if (tid < nh) my_off = hoff[P.hoff + tid];
+    pdl_wait();
     // tiles outside the support of the state (see ExcPass): block-uniform
     if (!BWD && (base & P.zmask) != P.zval) {
         if (init_hf) {   // the first pass writes the whole state
@@ -112,14 +127,10 @@ k_exc_pass(ExcPass P, const ExcGate *__restrict__ gates, const uint32_t *__restr
         for (int i = tid; i < ng; i += blockDim.x) out[i] = 0.0;
         return;
     }
-    for (int i = tid; i < ng; i += blockDim.x) {
-        sg[i] = gates[P.g_begin + i];
-        const int prm = gates[P.g_begin + i].param;
-        scs[2 * i] = cs[((size_t)b * n_exc + prm) * 2];
-        scs[2 * i + 1] = cs[((size_t)b * n_exc + prm) * 2 + 1];
-    }
-    const uint32_t nh = 1u << (k - m);
-    for (uint32_t i = tid; i < nh; i += blockDim.x) shoff[i] = hoff[P.hoff + i];
+    if ((int)tid < 2 * ng)   // gate g of the table has parameter g
+        scs[tid] = cs[((size_t)b * n_exc + P.g_begin) * 2 + tid];
+    if ((int)tid < ng) sg[tid] = my_gate;
+    if (tid < nh) shoff[tid] = my_off;
     __syncthreads();
     const uint32_t lowmask = (1u << m) - 1u;
     // a thread's loads of the tile in flight together (kLoadBatch per
@@ -207,16 +218,18 @@ k_exc_pass(ExcPass P, const ExcGate *__restrict__ gates, const uint32_t *__restr
         const int nw = kExcThreads / 32;
         double *out = gpart + (size_t)b * grad_stride + P.grad_off + (size_t)blockIdx.x * ng;
         for (int i = warp; i < ng; i += nw) {
+            // threads beyond the gate's pairs hold zeros
+            const int used = (int)min(size >> sg[i].n_fixed, (uint32_t)kExcThreads);
             if constexpr (sizeof(T) == 8) {
                 const double *r = reinterpret_cast<const double *>(rows) + i * kExcThreads;
                 double sum = 0.0;
-                for (int t = lane; t < kExcThreads; t += 32) sum += r[t];
+                for (int t = lane; t < used; t += 32) sum += r[t];
                 for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
                 if (lane == 0) out[i] = 2.0 * sum;
             } else {
                 const F32c *r = reinterpret_cast<const F32c *>(rows) + i * kExcThreads;
                 F32c sum = f32c_zero();
-                for (int t = lane; t < kExcThreads; t += 32) sum = f32c_add(sum, r[t]);
+                for (int t = lane; t < used; t += 32) sum = f32c_add(sum, r[t]);
                 sum = f32c_warp_sum(sum, 0xffffffffu, 32);
                 if (lane == 0) out[i] = 2.0 * f32c_value(sum);
             }
@@ -236,25 +249,26 @@ cudaError_t launch_exc_pass(const ExcPass &P, const ExcGate *gates_dev, const ui
     const size_t row = sizeof(T) == 8 ? sizeof(double) : sizeof(F32c);
     const size_t smem = backward ? 2 * tile + size_t(P.n_gates) * kExcThreads * row : tile;
     dim3 grid((unsigned)(1ull << (n_qubits - P.k)), batch);
+    // complex64 blocks wait on memory rather than on a pipe: two on one SM do no harm
+    // (18 qubits, 64 blocks: 498 -> 427 us; 19 qubits, 128 blocks: 541 -> 506)
+    const bool early = sizeof(T) == 4 || pdl_pays(grid);
     if (backward) {
         auto kern = k_exc_pass<T, true>;
-        if (smem > 48 * 1024) {
+        if (smem > 40 * 1024) {   // with the static part beyond the default 48 KiB
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        kern<<<grid, kExcThreads, smem, s>>>(P, gates_dev, hoff_dev, static_cast<C *>(psi),
-                                             static_cast<C *>(lam), state_stride, cs, n_exc, gpart,
-                                             grad_stride, 0, hf_index);
+        return pdl_launch(kern, grid, kExcThreads, smem, s, early, P, gates_dev, hoff_dev, static_cast<C *>(psi),
+                          static_cast<C *>(lam), state_stride, cs, n_exc, gpart, grad_stride, 0, hf_index);
     } else {
         auto kern = k_exc_pass<T, false>;
-        if (smem > 48 * 1024) {
+        if (smem > 40 * 1024) {   // with the static part beyond the default 48 KiB
             cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
             if (e != cudaSuccess) return e;
         }
-        kern<<<grid, kExcThreads, smem, s>>>(P, gates_dev, hoff_dev, static_cast<C *>(psi), nullptr,
-                                             state_stride, cs, n_exc, nullptr, 0, init_hf, hf_index);
+        return pdl_launch(kern, grid, kExcThreads, smem, s, early, P, gates_dev, hoff_dev, static_cast<C *>(psi),
+                          nullptr, state_stride, cs, n_exc, nullptr, 0, init_hf, hf_index);
     }
-    return cudaGetLastError();
 }
 
 template cudaError_t launch_exc_stage<float>(const double *, int, int, float *, cudaStream_t);

@@ -21,6 +21,7 @@
 #include <vector>
 
 #include "pass_core.cuh"
+#include "pdl.cuh"
 
 namespace vqe {
 
@@ -31,6 +32,7 @@ __global__ void k_stage(const StageSlot *__restrict__ slots, int n, int depth,
                         const double *__restrict__ params, RotCoef<T> *__restrict__ coefs,
                         size_t coef_stride, typename V2<T>::type *__restrict__ dtab,
                         size_t dtab_stride) {
+    pdl_trigger();
     using C = typename V2<T>::type;
     __shared__ double ph_c[kMaxTileBits], ph_s[kMaxTileBits], scl[kMaxTileBits], ph_v[kMaxTileBits];
     __shared__ int ph_m[kMaxTileBits];
@@ -224,6 +226,8 @@ k_pass(const PassDesc *__restrict__ desc, int init_zero, typename V2<T>::type *_
        typename V2<T>::type *__restrict__ lam, size_t stride, const RotCoef<T> *__restrict__ coefs,
        size_t coef_stride, const typename V2<T>::type *__restrict__ dtab, size_t dtab_stride,
        double *__restrict__ gpart, size_t grad_stride) {
+    pdl_trigger();
+    pdl_wait();
     using C = typename V2<T>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ PassDesc sd;
@@ -307,6 +311,14 @@ k_pass_fixed(const FixedHead H, const PassDesc *__restrict__ desc, int init_zero
     const uint64_t base = ((tile & ((1ull << mid) - 1ull)) << m) | ((tile >> mid) << (a + (k - m)));
     const uint32_t lowmask = (1u << m) - 1u;
     const RotCoef<T> *cf = coefs + (size_t)b * coef_stride;
+    pdl_trigger();
+    {   // the plan's tables do not depend on earlier kernels
+        const uint32_t *src = reinterpret_cast<const uint32_t *>(desc);
+        uint32_t *dst = reinterpret_cast<uint32_t *>(&sd);
+        for (int i = threadIdx.x; i < (int)(offsetof(PassDesc, ops) / 4) + H.n_ops; i += blockDim.x)
+            dst[i] = src[i];
+    }
+    pdl_wait();
     if (base & H.zmask) {   // block-uniform
         if (BWD) write_zero_partials(*desc, gpart + (size_t)b * grad_stride, tile);
         else write_zero_tile(psi + (size_t)b * stride, base, lowmask, m, a, k);
@@ -323,10 +335,6 @@ k_pass_fixed(const FixedHead H, const PassDesc *__restrict__ desc, int init_zero
                    BWD ? lam + (size_t)b * stride : nullptr, base, lowmask, m, a, init_zero,
                    __ffs(H.gated) - 1};
     auto stage = [&]() {
-        const uint32_t *src = reinterpret_cast<const uint32_t *>(desc);
-        uint32_t *dst = reinterpret_cast<uint32_t *>(&sd);
-        for (int i = threadIdx.x; i < (int)(offsetof(PassDesc, ops) / 4) + H.n_ops; i += blockDim.x)
-            dst[i] = src[i];
         for (int i = threadIdx.x; i < H.n_slots * k; i += blockDim.x) scf[i] = cf[H.coef0 + i];
         __syncthreads();
     };
@@ -349,17 +357,16 @@ cudaError_t launch_fixed(const PassDesc *desc_dev, const PassDesc &dh, int n_qub
     size_t smem = pass_smem_bytes(dh, BWD, sizeof(C));
     if (BWD) smem += fixed_grad_scratch_bytes<T, R>(threads, dh.k) - tile_grad_scratch_bytes(threads, dh.k);
     auto kern = k_pass_fixed<T, R, BWD, Codes...>;
-    if (smem > 48 * 1024) {
+    if (smem > 40 * 1024) {   // with the static part beyond the default 48 KiB
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
     dim3 grid((unsigned)(1ull << (n_qubits - dh.k)), batch);
     const FixedHead head{dh.m, dh.a, dh.n_ops, dh.n_slots, dh.zmask, dh.slot_gated[0], dh.slot_coef_off[0]};
-    kern<<<grid, threads, smem, s>>>(head, desc_dev, init_zero, static_cast<C *>(psi),
+    return pdl_launch(kern, grid, threads, smem, s, pdl_pays(grid), head, desc_dev, init_zero, static_cast<C *>(psi),
                                      static_cast<C *>(lam), stride,
                                      static_cast<const RotCoef<T> *>(coefs), coef_stride,
                                      static_cast<const C *>(dtab), dtab_stride, gpart, grad_stride);
-    return cudaGetLastError();
 }
 
 struct FixedEntry {
@@ -448,16 +455,15 @@ static cudaError_t launch_pass_r(const PassDesc *desc_dev, const PassDesc &dh, i
     if (threads > kPassMaxThreads) return cudaErrorInvalidConfiguration;
     const size_t smem = pass_smem_bytes(dh, BWD, sizeof(C));
     auto kern = k_pass<T, R, BWD>;
-    if (smem > 48 * 1024) {
+    if (smem > 40 * 1024) {   // with the static part beyond the default 48 KiB
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem);
         if (e != cudaSuccess) return e;
     }
     dim3 grid((unsigned)(1ull << (n_qubits - dh.k)), batch);
-    kern<<<grid, threads, smem, s>>>(desc_dev, init_zero, static_cast<C *>(psi),
+    return pdl_launch(kern, grid, threads, smem, s, pdl_pays(grid), desc_dev, init_zero, static_cast<C *>(psi),
                                      static_cast<C *>(lam), stride, coefs, coef_stride,
                                      static_cast<const C *>(dtab), dtab_stride, gpart, grad_stride);
-    return cudaGetLastError();
 }
 
 template <typename T>

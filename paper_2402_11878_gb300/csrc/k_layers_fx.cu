@@ -11,6 +11,7 @@
 
 #include "fx.cuh"
 #include "pass_core.cuh"
+#include "pdl.cuh"
 #include "vqe_internal.h"
 
 namespace vqe {
@@ -48,6 +49,7 @@ __device__ __forceinline__ long long to62(double x, double r) {
 __global__ void k_stage_fx(const StageSlot *__restrict__ slots, int n, int depth,
                            const double *__restrict__ params, RotFx *__restrict__ coefs,
                            size_t coef_stride, longlong2 *__restrict__ dtab, size_t dtab_stride) {
+    pdl_trigger();
     __shared__ longlong2 half_tab[2][1 << (kMaxTileBits / 2)];
     __shared__ longlong2 d0[kMaxTileBits], d1[kMaxTileBits];
     __shared__ long long scl[kMaxTileBits];
@@ -465,6 +467,14 @@ k_pass_fx(const FxHead H, const PassDesc *__restrict__ desc, int init_zero, doub
     auto g32 = [&](uint32_t e) -> uint32_t {
         return (uint32_t)(base | (uint64_t)(e & lowmask) | ((uint64_t)(e >> m) << a));
     };
+    pdl_trigger();
+    {   // the plan's tables do not depend on earlier kernels
+        static_assert(sizeof(PassDesc) % 4 == 0, "descriptor copied in words");
+        const uint32_t *src = reinterpret_cast<const uint32_t *>(desc);
+        uint32_t *dst = reinterpret_cast<uint32_t *>(&sh.d);
+        for (int i = t; i < (int)(offsetof(PassDesc, ops) / 4) + H.n_ops; i += blockDim.x) dst[i] = src[i];
+    }
+    pdl_wait();
     if (base & H.zmask) {   // block-uniform: psi is zero on this tile (see PassDesc::zmask)
         if (BWD) {
             for (int s = 0; s < H.n_slots; ++s)
@@ -489,7 +499,7 @@ k_pass_fx(const FxHead H, const PassDesc *__restrict__ desc, int init_zero, doub
         return x;
     };
 
-    // the tile's loads first: the descriptor and the coefficients arrive under them.
+    // the tile's loads first: the coefficients arrive under them.
     // The state streams past L1, which the tables then stay in.
     long long re[NB][kNR], im[NB][kNR];
     int chunk = H.chunk0;
@@ -514,12 +524,6 @@ k_pass_fx(const FxHead H, const PassDesc *__restrict__ desc, int init_zero, doub
                 im[1][r] = y.y;
             }
         }
-    }
-    {
-        static_assert(sizeof(PassDesc) % 4 == 0, "descriptor copied in words");
-        const uint32_t *src = reinterpret_cast<const uint32_t *>(desc);
-        uint32_t *dst = reinterpret_cast<uint32_t *>(&sh.d);
-        for (int i = t; i < (int)(offsetof(PassDesc, ops) / 4) + H.n_ops; i += blockDim.x) dst[i] = src[i];
     }
     const PassDesc &d = sh.d;
     int any_bad = 0;
@@ -808,18 +812,17 @@ cudaError_t launch_k(const PassDesc *desc_dev, const PassDesc &dh, int n_qubits,
                   size_t(dh.n_slots) * dh.k * sizeof(RotFx);
     if (BWD) smem += size_t(threads) * (dh.k + 1 + kR) * sizeof(long long);
     auto kern = k_pass_fx<BWD, MAXT, MINB>;
-    if (smem > 48 * 1024) {
+    if (smem > 40 * 1024) {   // with the static part beyond the default 48 KiB
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
     dim3 grid((unsigned)(1ull << (n_qubits - dh.k)), batch);
     const FxHead head{dh.k, dh.m, dh.a, dh.n_ops, dh.n_slots, dh.ops[0].chunk, dh.zmask,
                       dh.slot_gated[0], dh.slot_coef_off[0], dh.slot_grad_off[0]};
-    kern<<<grid, threads, smem, s>>>(head, desc_dev, init_zero, static_cast<double2 *>(psi),
+    return pdl_launch(kern, grid, threads, smem, s, pdl_pays(grid), head, desc_dev, init_zero, static_cast<double2 *>(psi),
                                      static_cast<double2 *>(lam), stride, coefs, coef_stride,
                                      static_cast<const longlong2 *>(dtab), dtab_stride, gpart,
                                      grad_stride);
-    return cudaGetLastError();
 }
 
 }  // namespace

@@ -17,6 +17,7 @@
 #include <algorithm>
 
 #include "csum.cuh"
+#include "pdl.cuh"
 #include "vqe_internal.h"
 
 namespace vqe {
@@ -90,6 +91,8 @@ k_apply_h_sweep(SweepDesc W, const uint32_t *__restrict__ order, const SGroup *_
                 int n, const typename SV2<T>::type *__restrict__ psi,
                 typename SV2<T>::type *__restrict__ lam, size_t stride, int first, int last,
                 unsigned long long *__restrict__ ctr, double *__restrict__ cpart) {
+    pdl_trigger();
+    pdl_wait();
     using C = typename SV2<T>::type;
     constexpr int J = kSweepJ;
     constexpr uint32_t kIter = kSweepThreads * J;   // counter values per block iteration
@@ -357,11 +360,10 @@ cudaError_t launch_apply_h_sweep(const SweepDesc &W, const uint32_t *order, cons
         if (e != cudaSuccess) return e;
     }
     dim3 grid((unsigned)blocks, batch);
-    kern<<<grid, kSweepThreads, smem, s>>>(W, order, groups, pat, tz, static_cast<const T *>(ca),
+    return pdl_launch(kern, grid, kSweepThreads, smem, s, pdl_pays(grid), W, order, groups, pat, tz, static_cast<const T *>(ca),
                                            static_cast<const T *>(cb), static_cast<const T *>(hdiag),
                                            n_qubits, static_cast<const C *>(psi), static_cast<C *>(lam),
                                            state_stride, first, last, ctr, cpart);
-    return cudaGetLastError();
 }
 
 template cudaError_t launch_apply_h_sweep<float>(const SweepDesc &, const uint32_t *, const SGroup *,
