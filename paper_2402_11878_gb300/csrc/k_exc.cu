@@ -8,13 +8,34 @@
 // rotation
 //     psi_j  <- cos t psi_j  - sgn sin t psi_j'
 //     psi_j' <- cos t psi_j' + sgn sin t psi_j,   sgn = (-1)^(sign0 + popc(j & smask)),
-// and leaves every other amplitude alone.  A pass stages a tile of 2^k
-// amplitudes in shared memory (its low m bits are a contiguous run of the
-// state, its other k - m bits the modes of its gates) and applies a run of
-// consecutive gates whose modes lie in the tile, one barrier per gate, with
-// one HBM read and write of the state per pass.  The sign factors into a
+// and leaves every other amplitude alone.  A pass stages tiles of 2^k amplitudes
+// in shared memory (the low m tile bits are a contiguous run of the state, the
+// other k - m the modes of its gates) and applies a run of consecutive gates
+// whose modes lie in the tile, one barrier per gate.  The sign factors into a
 // per-tile part (the sign mask's bits outside the tile, fixed by the tile's
 // base) and a per-element parity over the tile bits.
+//
+// Excitations keep the number of electrons, so every amplitude whose index does
+// not have n_elec ones is zero for good.  Inside a tile the live amplitudes are
+// the tile words with n_elec - popc(base) ones: at most binomial(11, 5) = 462 of
+// 2048 (FP64) or 924 of 4096.  Shared memory holds just this class, in the order
+// of a constant table of the words sorted by popcount; a gate's live pairs are a
+// class of the words of its free bits; elements that no gate of the pass pairs
+// are not read or written.  lambda = H psi is needed, and kept up, in the sector
+// alone, because psi is zero elsewhere and the gates do not leave it.
+// At 28 qubits and half filling 15 % of the amplitudes are live; before, a whole
+// tile was read, rotated (64 FP64-pipe cycles per warp instruction) and written
+// back: 118 excitations in FP64, forward 59.1 -> 16.0 ms and backward 176.6 ->
+// 33.7 ms, complex64 at 27 qubits 13.0 -> 4.7 and 27.5 -> 8.1 ms.  What bounds
+// it now is the latency of a tile (two table look-ups, the load, a barrier per
+// gate), hidden by nine or more blocks per SM, and the memory's access size: the
+// scattered elements move in 32-byte sectors.
+//
+// FP64 gives a pair two lanes, one per component: half the FP64 instructions per
+// warp where the 35 pairs of a double (11 tile bits, 5 electrons) are all there
+// is.  All launches start before their predecessor has ended: what precedes the
+// first load of a state (gates, offsets, class words, places) is done by then
+// (FP64 at 17 qubits, 64 blocks: forward 212 -> 112 us).
 //
 // The backward (adjoint) pass un-applies the gates in reverse on psi and
 // lambda = H psi and, before un-applying gate g, takes
@@ -22,6 +43,7 @@
 // per pair sgn * (Re conj(lambda_j') psi_j - Re conj(lambda_j) psi_j').
 #include "csum.cuh"
 #include "pdl.cuh"
+#include "sector.cuh"
 #include "vqe_internal.h"
 
 namespace vqe {
@@ -30,7 +52,9 @@ template <typename T> struct XV2;
 template <> struct XV2<float> { using type = float2; };
 template <> struct XV2<double> { using type = double2; };
 
-constexpr int kExcMaxHigh = 8;   // k - m <= 8: 256 high-part offsets per pass
+constexpr int kExcMaxHigh = 7;   // k - m <= 7: 128 high-part offsets per pass
+constexpr int kExcWide = 256;             // threads of a block of a grid that leaves the chip room
+constexpr uint64_t kExcWideBlocks = 1024;
 
 template <typename T>
 __global__ void k_exc_stage(const double *__restrict__ params, int total, T *__restrict__ cs) {
@@ -51,13 +75,25 @@ cudaError_t launch_exc_stage(const double *params, int n_exc, int batch, T *cs, 
     return cudaGetLastError();
 }
 
-// f with a zero bit inserted at each tile position fixed[0..nf) (increasing).
-__device__ __forceinline__ uint32_t spread_fixed(uint32_t f, const uint8_t *fixed, int nf) {
-    for (int i = 0; i < nf; ++i) {
-        const int b = fixed[i];
-        f = ((f >> b) << (b + 1)) | (f & ((1u << b) - 1u));
+// A gate of the pass as the tile's threads use it.
+struct TileGate {
+    uint32_t amask, flip;    // flip = amask | cmask
+    uint32_t smask_t, sign;  // sign of the tile's base included
+    uint32_t fixed, n_fixed; // four tile bits, a byte each
+    uint32_t word, pairs;    // its live pairs' free bits: kClass.word[word ...]
+};
+
+// Places of both elements of live pair f of a gate, and the pair's sign (bit 31).
+__device__ __forceinline__ uint32_t locate(const TileGate &G, uint32_t f, uint32_t at) {
+    uint32_t e = kClass.word[G.word + f];
+    uint32_t fx = G.fixed;
+    for (uint32_t i = 0; i < G.n_fixed; ++i, fx >>= 8) {   // zero bits at the gate's modes
+        const uint32_t low = (1u << (fx & 31u)) - 1u;
+        e += e & ~low;
     }
-    return f;
+    e |= G.amask;
+    return kClass.place[at + e] | (uint32_t)kClass.place[at + (e ^ G.flip)] << 15 |
+           (G.sign ^ (__popc(e & G.smask_t) & 1u)) << 31;
 }
 
 __device__ __forceinline__ double xflip(double v, uint32_t s) {
@@ -67,167 +103,230 @@ __device__ __forceinline__ float xflip(float v, uint32_t s) {
     return __int_as_float(__float_as_int(v) ^ (int)(s << 31));
 }
 
-template <typename T, bool BWD>
-__global__ void __launch_bounds__(kExcThreads)
+template <typename T, bool BWD, int TH>
+__global__ void __launch_bounds__(TH)
 k_exc_pass(ExcPass P, const ExcGate *__restrict__ gates, const uint32_t *__restrict__ hoff,
            typename XV2<T>::type *__restrict__ psi, typename XV2<T>::type *__restrict__ lam,
            size_t stride, const T *__restrict__ cs, int n_exc, double *__restrict__ gpart,
-           size_t grad_stride, int init_hf, uint64_t hf) {
+           size_t grad_stride, int init_hf, uint64_t hf, int room) {
     using C = typename XV2<T>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ ExcGate sg[kExcMaxGates];
+    __shared__ TileGate sg[kExcMaxGates];
     __shared__ T scs[2 * kExcMaxGates];
     __shared__ uint32_t shoff[1 << kExcMaxHigh];
     const int k = P.k, m = P.m, ng = P.n_gates;
-    const uint32_t size = 1u << k;
+    const uint32_t size = 1u << k, at = size - 1u;
     const uint32_t tid = threadIdx.x;
-    C *sp = reinterpret_cast<C *>(smem_raw);
-    C *sl = BWD ? sp + size : nullptr;
-    // backward: per-thread gradient partials, one row of kExcThreads per gate
+    C *sp = reinterpret_cast<C *>(smem_raw);   // the live elements of the tile
+    C *sl = BWD ? sp + room : nullptr;
+    // backward: per-thread gradient partials, one row of TH per gate
     // (FP64 values, or compensated FP32 pairs in the FP32 kernel)
-    unsigned char *rows = reinterpret_cast<unsigned char *>(sp + (BWD ? 2 * size : size));
+    unsigned char *rows = reinterpret_cast<unsigned char *>(sp + (BWD ? 2 * room : room));
     const int b = blockIdx.y;
     C *Pp = psi + (size_t)b * stride;
     C *Lp = BWD ? lam + (size_t)b * stride : nullptr;
     uint64_t base = 0;   // the tile number's bits at the bits of bmask, run by run
     {
         uint32_t bm = P.bmask;
-        uint64_t tn = blockIdx.x;
+        uint64_t t = blockIdx.x;
         while (bm) {
             const int lo = __ffs(bm) - 1;
-            const uint32_t up = bm >> lo;                       // run of ones from bit 0
+            const uint32_t up = bm >> lo;
             const int len = up == 0xffffffffu ? 32 : __ffs(~up) - 1;
             const uint64_t run = (1ull << len) - 1ull;
-            base |= (tn & run) << lo;
-            tn >>= len;
+            base |= (t & run) << lo;
+            t >>= len;
             bm &= ~(uint32_t)(run << lo);
         }
     }
     // the plan's tables do not depend on earlier kernels; they are on their way
     // while the block waits
     pdl_trigger();
-    static_assert(kExcMaxGates <= kExcThreads && (1 << kExcMaxHigh) <= kExcThreads, "one entry per thread");
-    const uint32_t nh = 1u << (k - m);
-    ExcGate my_gate;
-    uint32_t my_off = 0u;
-    if ((int)tid < ng) my_gate = gates[P.g_begin + tid];
-    if (tid < nh) my_off = hoff[P.hoff + tid];
+    static_assert(2 * kExcMaxGates <= TH, "one entry per thread");
+    const uint32_t lowmask = (1u << m) - 1u;
+    const int left = __popcll(hf) - __popcll(base);   // electrons in the tile's modes
+    const bool live = left >= 0 && left <= k &&
+                      (BWD ? (base & P.bzmask) == P.bzval : (base & P.zmask) == P.zval);   // block-uniform
+    constexpr int kPer = (sizeof(T) == 8 ? 512 : 1024) / TH;   // C(11,5) = 462, C(12,6) = 924 live ones
+    constexpr uint32_t kSplit = sizeof(T) == 8 ? 2 : 1;   // lanes per pair; FP64: one per component
+    constexpr uint32_t kNone = ~0u;
+    uint32_t at_g[kPer];     // where this thread's elements of the class lie in the state
+    uint32_t mine = 0u;      // which of them the pass moves
+    uint32_t nxt = 0u;       // the next gate's first pair, found while this one's is computed
+    if (live) {
+        if ((int)tid < ng) {
+            const ExcGate my = gates[P.g_begin + tid];
+            TileGate &G = sg[tid];
+            G.amask = my.amask;
+            G.flip = my.amask | my.cmask;
+            G.smask_t = my.smask_t;
+            G.sign = (uint32_t)((__popcll(base & (uint64_t)my.smask_g) + my.sign0) & 1);
+            G.fixed = my.fixed[0] | my.fixed[1] << 8 | my.fixed[2] << 16 | (uint32_t)my.fixed[3] << 24;
+            G.n_fixed = my.n_fixed;
+            const int nb = k - my.n_fixed, p = left - my.n_fixed / 2;
+            const bool some = p >= 0 && p <= nb;
+            G.word = some ? (1u << nb) - 1u + kClass.begin[nb][p] : 0u;
+            G.pairs = some ? kClass.begin[nb][p + 1] - kClass.begin[nb][p] : 0u;
+        }
+        for (uint32_t i = tid; i < (1u << (k - m)); i += TH) shoff[i] = hoff[P.hoff + i];
+        const uint32_t first = kClass.begin[k][left], n_live = kClass.begin[k][left + 1] - first;
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            const uint32_t j = tid + u * TH;
+            at_g[u] = j < n_live ? kClass.word[at + first + j] : kNone;
+        }
+        __syncthreads();
+        // only elements that a gate pairs are read and written
+#pragma unroll
+        for (int u = 0; u < kPer; ++u) {
+            const uint32_t e = at_g[u];
+            if (e == kNone) continue;
+            bool used = !BWD && init_hf;
+            for (int i = 0; i < ng; ++i) {
+                const uint32_t v = e & sg[i].flip;
+                used |= v == sg[i].amask || (v ^ sg[i].flip) == sg[i].amask;
+            }
+            mine |= (uint32_t)used << u;
+            at_g[u] = (uint32_t)base | (e & lowmask) | shoff[e >> m];
+        }
+        const TileGate &G = sg[BWD ? ng - 1 : 0];
+        if (tid / kSplit < G.pairs) nxt = locate(G, tid / kSplit, at);
+    }
     pdl_wait();
-    // tiles outside the support of the state (see ExcPass): block-uniform
-    if (!BWD && (base & P.zmask) != P.zval) {
-        if (init_hf) {   // the first pass writes the whole state
-            const uint32_t lowmask = (1u << m) - 1u;
-            for (uint32_t e = tid; e < size; e += blockDim.x)
+    if (!live) {
+        if (BWD) {
+            double *out = gpart + (size_t)b * grad_stride + P.grad_off + (size_t)blockIdx.x * ng;
+            for (int i = tid; i < ng; i += TH) out[i] = 0.0;
+        } else if (init_hf) {   // the first pass writes the whole state
+            for (uint32_t e = tid; e < size; e += TH)
                 Pp[base | (e & lowmask) | hoff[P.hoff + (e >> m)]] = C{};
         }
         return;
     }
-    if (BWD && (base & P.bzmask) != P.bzval) {
-        double *out = gpart + (size_t)b * grad_stride + P.grad_off + (size_t)blockIdx.x * ng;
-        for (int i = tid; i < ng; i += blockDim.x) out[i] = 0.0;
-        return;
-    }
+    const T *my_cs = cs + (size_t)b * n_exc * 2;
     if ((int)tid < 2 * ng)   // gate g of the table has parameter g
-        scs[tid] = cs[((size_t)b * n_exc + P.g_begin) * 2 + tid];
-    if ((int)tid < ng) sg[tid] = my_gate;
-    if (tid < nh) shoff[tid] = my_off;
-    __syncthreads();
-    const uint32_t lowmask = (1u << m) - 1u;
-    // a thread's loads of the tile in flight together (kLoadBatch per
-    // buffer), then their shared-memory stores
-    constexpr int kLoadBatch = 8;
-    for (uint32_t e0 = tid; e0 < size; e0 += kLoadBatch * blockDim.x) {
-        C x[kLoadBatch], l[kLoadBatch];
+        scs[tid] = my_cs[2 * P.g_begin + tid];
+    T one = T(1);
+    if (!BWD && init_hf && base == (hf & P.bmask)) {
+        // an angle that is not a number shows in the energy, also where its
+        // gate has no pair in the sector
+        int bad = 0;
+        for (int i = tid; i < n_exc; i += TH) bad |= !isfinite(my_cs[2 * i]);
+        if (__syncthreads_or(bad)) one = T(NAN);
+    }
+    {
+        C x[kPer], l[kPer];
 #pragma unroll
-        for (int u = 0; u < kLoadBatch; ++u) {
-            const uint32_t e = e0 + u * blockDim.x;
-            if (e >= size) break;
-            const uint64_t g = base | (e & lowmask) | shoff[e >> m];
-            if (init_hf) {
-                x[u].x = (g == hf) ? T(1) : T(0);
+        for (int u = 0; u < kPer; ++u) {
+            if (!((mine >> u) & 1u)) continue;
+            if (!BWD && init_hf) {
+                x[u].x = (at_g[u] == (uint32_t)hf) ? one : T(0);
                 x[u].y = T(0);
             } else {
-                x[u] = Pp[g];
+                x[u] = Pp[at_g[u]];
+                if (BWD) l[u] = Lp[at_g[u]];
             }
-            if (BWD) l[u] = Lp[g];
         }
 #pragma unroll
-        for (int u = 0; u < kLoadBatch; ++u) {
-            const uint32_t e = e0 + u * blockDim.x;
-            if (e >= size) break;
-            sp[e] = x[u];
-            if (BWD) sl[e] = l[u];
+        for (int u = 0; u < kPer; ++u) {
+            if (!((mine >> u) & 1u)) continue;
+            sp[tid + u * TH] = x[u];
+            if (BWD) sl[tid + u * TH] = l[u];
         }
     }
     __syncthreads();
     for (int ii = 0; ii < ng; ++ii) {
         const int i = BWD ? ng - 1 - ii : ii;
-        const ExcGate &G = sg[i];
+        const TileGate &G = sg[i];
         const T c = scs[2 * i], s = scs[2 * i + 1];
-        const uint32_t sb = (uint32_t)((__popcll(base & (uint64_t)G.smask_g) + G.sign0) & 1);
-        const uint32_t npairs = size >> G.n_fixed;
-        const uint32_t flip = G.amask | G.cmask;
+        const uint32_t count = G.pairs * kSplit;
+        uint32_t loc = nxt;
+        if (ii + 1 < ng) {
+            const TileGate &N = sg[BWD ? i - 1 : i + 1];
+            if (tid / kSplit < N.pairs) nxt = locate(N, tid / kSplit, at);
+        }
         double gd = 0.0;
         F32c gf = f32c_zero();
-        for (uint32_t f = tid; f < npairs; f += blockDim.x) {
-            const uint32_t e = spread_fixed(f, G.fixed, G.n_fixed) | G.amask;
-            const uint32_t e2 = e ^ flip;
-            const uint32_t par = sb ^ (__popc(e & G.smask_t) & 1u);
+        for (uint32_t f = tid; f < count; f += TH) {
+            if (f != tid) loc = locate(G, f / kSplit, at);
+            const uint32_t i1 = loc & 0x7fffu, i2 = (loc >> 15) & 0x7fffu, par = loc >> 31;
             const T ss = xflip(s, par);
-            const C x = sp[e], y = sp[e2];
-            C nx, ny;
-            if (!BWD) {
-                nx.x = fma(c, x.x, -ss * y.x);
-                nx.y = fma(c, x.y, -ss * y.y);
-                ny.x = fma(c, y.x, ss * x.x);
-                ny.y = fma(c, y.y, ss * x.y);
+            if constexpr (sizeof(T) == 8) {
+                double *p1 = reinterpret_cast<double *>(sp + i1) + (tid & 1u);
+                double *p2 = reinterpret_cast<double *>(sp + i2) + (tid & 1u);
+                const double x = *p1, y = *p2;
+                if (!BWD) {
+                    *p1 = fma(c, x, -ss * y);
+                    *p2 = fma(c, y, ss * x);
+                } else {
+                    double *q1 = reinterpret_cast<double *>(sl + i1) + (tid & 1u);
+                    double *q2 = reinterpret_cast<double *>(sl + i2) + (tid & 1u);
+                    const double lx = *q1, ly = *q2;
+                    gd += xflip(fma(ly, x, -(lx * y)), par);
+                    *p1 = fma(c, x, ss * y);
+                    *p2 = fma(c, y, -ss * x);
+                    *q1 = fma(c, lx, ss * ly);
+                    *q2 = fma(c, ly, -ss * lx);
+                }
             } else {
-                const C lx = sl[e], ly = sl[e2];
-                const T dg = xflip(fma(ly.x, x.x, fma(ly.y, x.y, -fma(lx.x, y.x, lx.y * y.y))), par);
-                if constexpr (sizeof(T) == 8) gd += dg;
-                else f32c_add(gf, dg);
-                nx.x = fma(c, x.x, ss * y.x);
-                nx.y = fma(c, x.y, ss * y.y);
-                ny.x = fma(c, y.x, -ss * x.x);
-                ny.y = fma(c, y.y, -ss * x.y);
-                C mx, my;
-                mx.x = fma(c, lx.x, ss * ly.x);
-                mx.y = fma(c, lx.y, ss * ly.y);
-                my.x = fma(c, ly.x, -ss * lx.x);
-                my.y = fma(c, ly.y, -ss * lx.y);
-                sl[e] = mx;
-                sl[e2] = my;
+                const C x = sp[i1], y = sp[i2];
+                C nx, ny;
+                if (!BWD) {
+                    nx.x = fma(c, x.x, -ss * y.x);
+                    nx.y = fma(c, x.y, -ss * y.y);
+                    ny.x = fma(c, y.x, ss * x.x);
+                    ny.y = fma(c, y.y, ss * x.y);
+                } else {
+                    const C lx = sl[i1], ly = sl[i2];
+                    f32c_add(gf, xflip(fma(ly.x, x.x, fma(ly.y, x.y, -fma(lx.x, y.x, lx.y * y.y))), par));
+                    nx.x = fma(c, x.x, ss * y.x);
+                    nx.y = fma(c, x.y, ss * y.y);
+                    ny.x = fma(c, y.x, -ss * x.x);
+                    ny.y = fma(c, y.y, -ss * x.y);
+                    C mx, my;
+                    mx.x = fma(c, lx.x, ss * ly.x);
+                    mx.y = fma(c, lx.y, ss * ly.y);
+                    my.x = fma(c, ly.x, -ss * lx.x);
+                    my.y = fma(c, ly.y, -ss * lx.y);
+                    sl[i1] = mx;
+                    sl[i2] = my;
+                }
+                sp[i1] = nx;
+                sp[i2] = ny;
             }
-            sp[e] = nx;
-            sp[e2] = ny;
         }
         if constexpr (BWD) {
-            if constexpr (sizeof(T) == 8) reinterpret_cast<double *>(rows)[i * kExcThreads + tid] = gd;
-            else reinterpret_cast<F32c *>(rows)[i * kExcThreads + tid] = gf;
+            if constexpr (sizeof(T) == 8) reinterpret_cast<double *>(rows)[i * TH + tid] = gd;
+            else reinterpret_cast<F32c *>(rows)[i * TH + tid] = gf;
         }
         __syncthreads();   // the next gate's pairs touch other threads' elements
     }
-    for (uint32_t e = tid; e < size; e += blockDim.x) {
-        const uint64_t g = base | (e & lowmask) | shoff[e >> m];
-        Pp[g] = sp[e];
-        if (BWD) Lp[g] = sl[e];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        if (!((mine >> u) & 1u)) continue;
+        const uint32_t j = tid + u * TH;
+        Pp[at_g[u]] = sp[j];
+        if (BWD) Lp[at_g[u]] = sl[j];
     }
+    if (!BWD && init_hf)   // the first pass writes the whole state
+        for (uint32_t e = tid; e < size; e += TH)
+            if (__popc(e) != left) Pp[base | (e & lowmask) | shoff[e >> m]] = C{};
     if constexpr (BWD) {
         // each warp sums whole rows in a fixed order (bitwise reproducible)
-        const int warp = tid >> 5, lane = tid & 31;
-        const int nw = kExcThreads / 32;
         double *out = gpart + (size_t)b * grad_stride + P.grad_off + (size_t)blockIdx.x * ng;
+        const int warp = tid >> 5, lane = tid & 31;
+        const int nw = TH / 32;
         for (int i = warp; i < ng; i += nw) {
             // threads beyond the gate's pairs hold zeros
-            const int used = (int)min(size >> sg[i].n_fixed, (uint32_t)kExcThreads);
+            const int used = (int)min(sg[i].pairs * kSplit, (uint32_t)TH);
             if constexpr (sizeof(T) == 8) {
-                const double *r = reinterpret_cast<const double *>(rows) + i * kExcThreads;
+                const double *r = reinterpret_cast<const double *>(rows) + i * TH;
                 double sum = 0.0;
                 for (int t = lane; t < used; t += 32) sum += r[t];
                 for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
                 if (lane == 0) out[i] = 2.0 * sum;
             } else {
-                const F32c *r = reinterpret_cast<const F32c *>(rows) + i * kExcThreads;
+                const F32c *r = reinterpret_cast<const F32c *>(rows) + i * TH;
                 F32c sum = f32c_zero();
                 for (int t = lane; t < used; t += 32) sum = f32c_add(sum, r[t]);
                 sum = f32c_warp_sum(sum, 0xffffffffu, 32);
@@ -243,32 +342,25 @@ cudaError_t launch_exc_pass(const ExcPass &P, const ExcGate *gates_dev, const ui
                             const T *cs, int n_exc, double *gpart, size_t grad_stride,
                             bool backward, int init_hf, uint64_t hf_index, cudaStream_t s) {
     using C = typename XV2<T>::type;
-    if (P.k - P.m > kExcMaxHigh || P.n_gates > kExcMaxGates || P.n_gates < 1 || P.k > n_qubits)
-        return cudaErrorInvalidValue;
-    const size_t tile = (size_t(1) << P.k) * sizeof(C);
+    const dim3 grid(1u << (n_qubits - P.k), batch);
+    int room = 1;   // the largest class: binomial(k, k / 2)
+    for (int i = 1; i <= P.k / 2; ++i) room = room * (P.k + 1 - i) / i;
+    if (P.k > (sizeof(T) == 8 ? 11 : 12)) return cudaErrorInvalidValue;
     const size_t row = sizeof(T) == 8 ? sizeof(double) : sizeof(F32c);
-    const size_t smem = backward ? 2 * tile + size_t(P.n_gates) * kExcThreads * row : tile;
-    dim3 grid((unsigned)(1ull << (n_qubits - P.k)), batch);
-    // complex64 blocks wait on memory rather than on a pipe: two on one SM do no harm
-    // (18 qubits, 64 blocks: 498 -> 427 us; 19 qubits, 128 blocks: 541 -> 506)
-    const bool early = sizeof(T) == 4 || pdl_pays(grid);
-    if (backward) {
-        auto kern = k_exc_pass<T, true>;
-        if (smem > 40 * 1024) {   // with the static part beyond the default 48 KiB
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
-        return pdl_launch(kern, grid, kExcThreads, smem, s, early, P, gates_dev, hoff_dev, static_cast<C *>(psi),
-                          static_cast<C *>(lam), state_stride, cs, n_exc, gpart, grad_stride, 0, hf_index);
-    } else {
-        auto kern = k_exc_pass<T, false>;
-        if (smem > 40 * 1024) {   // with the static part beyond the default 48 KiB
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
-        return pdl_launch(kern, grid, kExcThreads, smem, s, early, P, gates_dev, hoff_dev, static_cast<C *>(psi),
-                          nullptr, state_stride, cs, n_exc, nullptr, 0, init_hf, hf_index);
-    }
+    // 256 threads where a grid leaves the chip room, for a shorter chain per gate;
+    // 128 beyond, for more tiles per SM.  FP64, forward + backward of 100
+    // excitations, 128 / 256 threads: 14 qubits (8 blocks) 302 / 270 us, 20 (512)
+    // 574 / 565, 21 (1024) 822 / 798, 22 (2048) 1139 / 1150, 24 3.02 / 3.41 ms;
+    // complex64: 18 (64) 316 / 260 us, 22 (1024) 595 / 564, 24 1.48 / 1.60 ms.
+    const int th = uint64_t(grid.x) * grid.y <= kExcWideBlocks ? kExcWide : kExcThreads;
+    const size_t smem = room * sizeof(C) * (backward ? 2 : 1) + (backward ? size_t(P.n_gates) * th * row : 0);
+    auto launch = [&](auto kern) {
+        return pdl_launch(kern, grid, th, smem, s, true, P, gates_dev, hoff_dev, static_cast<C *>(psi),
+                          static_cast<C *>(lam), state_stride, cs, n_exc, gpart, grad_stride, init_hf, hf_index,
+                          room);
+    };
+    if (th == kExcWide) return backward ? launch(k_exc_pass<T, true, kExcWide>) : launch(k_exc_pass<T, false, kExcWide>);
+    return backward ? launch(k_exc_pass<T, true, kExcThreads>) : launch(k_exc_pass<T, false, kExcThreads>);
 }
 
 template cudaError_t launch_exc_stage<float>(const double *, int, int, float *, cudaStream_t);

@@ -21,9 +21,9 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 
 // Where it pays, by the number of blocks (152 SMs; a gradient in us, plain
 // against early launch).  Small grids: the gaps between kernels count (14 qubits,
-// 8 blocks: 588 -> 550 FP64, pc 561 -> 457; 16 qubits, 32 blocks: pc 647 -> 536).
+// 8 blocks: 588 -> 550 FP64).
 // Large ones: blocks of the next kernel take the places that the last wave frees
-// (22 qubits: 5921 -> 5821, pc 4253 -> 4017, complex64 1327 -> 1215).  In between the
+// (22 qubits: 5921 -> 5821, complex64 1327 -> 1215).  In between the
 // early blocks double up on some SMs while others stay empty (18 qubits, 128
 // blocks: 677 -> 837; 19 qubits, 256 blocks: 905 -> 933).
 inline bool pdl_pays(dim3 grid) {

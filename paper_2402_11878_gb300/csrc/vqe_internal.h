@@ -108,7 +108,7 @@ struct StageSlot {
 // whose modes all lie in the tile.
 
 constexpr int kExcMaxGates = 16;      // gates of one pass
-constexpr int kExcThreads = 256;
+constexpr int kExcThreads = 128;     // threads of a block (twice as many in small grids)
 
 struct ExcGate {
     uint32_t amask, cmask;   // tile bits annihilated / created by T
