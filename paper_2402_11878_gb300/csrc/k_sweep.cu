@@ -18,6 +18,7 @@
 
 #include "csum.cuh"
 #include "pdl.cuh"
+#include "sector.cuh"
 #include "vqe_internal.h"
 
 namespace vqe {
@@ -83,14 +84,24 @@ __device__ __forceinline__ void sweep_block_sum_c(F32c a, F32c b, float *sh, dou
 }
 
 // FP64: three blocks of 256 threads per SM (<= 85 registers), FP32 four.
-template <typename T>
+//
+// SECTOR: psi is zero outside the index words with n_elec ones and lambda is
+// wanted there alone (the excitation ansatz).  A chunk's counter values share
+// all but their low bits, and the bit order only moves bits, so the chunk's live
+// states are one class of equal popcount; its words come from the class table.
+// Other elements of lambda are left as they are.  28 qubits FP64, half filling,
+// 43 groups: 29.1 ms for the whole state (bound by the FP64 pipe), 8.8 for the
+// 15 % in the sector; there the gathers' latency counts (16.6 with one state's
+// gather after the other, inside the vote), so the J states' are issued together
+// as in complex64.  complex64 at 27 qubits: 3.75 -> 1.03 ms.
+template <typename T, bool SECTOR>
 __global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 3 : 4)
 k_apply_h_sweep(SweepDesc W, const uint32_t *__restrict__ order, const SGroup *__restrict__ groups,
                 const uint32_t *__restrict__ pat, const uint32_t *__restrict__ tz,
                 const T *__restrict__ ca, const T *__restrict__ cb, const T *__restrict__ hdiag,
                 int n, const typename SV2<T>::type *__restrict__ psi,
                 typename SV2<T>::type *__restrict__ lam, size_t stride, int first, int last,
-                unsigned long long *__restrict__ ctr, double *__restrict__ cpart) {
+                int n_elec, unsigned long long *__restrict__ ctr, double *__restrict__ cpart) {
     pdl_trigger();
     pdl_wait();
     using C = typename SV2<T>::type;
@@ -139,15 +150,31 @@ k_apply_h_sweep(SweepDesc W, const uint32_t *__restrict__ order, const SGroup *_
         if (chunk >= nchunks) break;
         double dacc = 0.0, dnrm = 0.0;
         F32c facc = f32c_zero(), fnrm = f32c_zero();
-        for (uint32_t it = 0; it < kSweepChunk / kIter; ++it) {
-            const uint64_t s0 = chunk * kSweepChunk + (uint64_t)it * kIter + threadIdx.x;
+        uint32_t n_live = kSweepChunk, word = 0u;
+        if (SECTOR) {
+            static_assert(kSweepChunk == 1 << kClassBits, "a chunk's low bits are a word of the table");
+            const int nb = n < kClassBits ? n : kClassBits;
+            const int left = n_elec - __popcll(chunk);   // ones among the chunk's low bits
+            const bool some = left >= 0 && left <= nb;
+            word = some ? (1u << nb) - 1u + kClass.begin[nb][left] : 0u;
+            n_live = some ? kClass.begin[nb][left + 1] - kClass.begin[nb][left] : 0u;
+        }
+        for (uint32_t it = 0; it * kIter < n_live; ++it) {
+            const uint32_t i0 = it * kIter + threadIdx.x;
             uint32_t a[J];
             bool ok[J];
             C lv[J];
 #pragma unroll
             for (int j = 0; j < J; ++j) {
-                const uint64_t s = s0 + (uint64_t)j * kSweepThreads;
-                ok[j] = s < dim;
+                const uint32_t i = i0 + j * kSweepThreads;
+                uint64_t s = chunk * kSweepChunk;
+                if (SECTOR) {
+                    ok[j] = i < n_live;
+                    s |= ok[j] ? kClass.word[word + i] : 0u;
+                } else {
+                    s |= i;
+                    ok[j] = s < dim;
+                }
                 const uint32_t ss = (uint32_t)(ok[j] ? s : 0u);
                 a[j] = sord[ss & 255u] | sord[256 + ((ss >> 8) & 255u)] |
                        sord[512 + ((ss >> 16) & 255u)] | sord[768 + (ss >> 24)];
@@ -236,7 +263,7 @@ k_apply_h_sweep(SweepDesc W, const uint32_t *__restrict__ order, const SGroup *_
                         }
                     }
                 }
-                if constexpr (sizeof(T) == 8) {
+                if constexpr (sizeof(T) == 8 && !SECTOR) {
                     // FP64 (bound by the FP64 pipe): the gather and the
                     // multiply-adds of a state inside a warp-uniform branch.
                     // The patterns of X bits above the lanes' bits are
@@ -260,7 +287,10 @@ k_apply_h_sweep(SweepDesc W, const uint32_t *__restrict__ order, const SGroup *_
                 } else {
                     C p[J];
 #pragma unroll
-                    for (int j = 0; j < J; ++j) p[j] = nz[j] ? P[a[j] ^ x] : C{T(0), T(0)};
+                    for (int j = 0; j < J; ++j) {
+                        if (SECTOR) nz[j] = nz[j] && ok[j];
+                        p[j] = nz[j] ? P[a[j] ^ x] : C{T(0), T(0)};
+                    }
                     // complex64 (issue-bound): the gathers of the J states
                     // issued together, the multiply-adds after a warp vote
                     // (which the compiler may turn into a select)
@@ -322,20 +352,19 @@ size_t sweep_smem_bytes(const SweepDesc &W, size_t real_bytes) {
 // Resident blocks per SM of the sweep kernel with `smem` bytes of dynamic
 // shared memory: the grid must be resident at once, so that all threads of
 // a state traverse the counter together.
-int sweep_blocks_per_sm(int elem_bytes, size_t smem) {
+int sweep_blocks_per_sm(int elem_bytes, size_t smem, bool sector) {
+    const void *kern = elem_bytes == 16
+        ? (sector ? (const void *)k_apply_h_sweep<double, true> : (const void *)k_apply_h_sweep<double, false>)
+        : (sector ? (const void *)k_apply_h_sweep<float, true> : (const void *)k_apply_h_sweep<float, false>);
     int occ = 0;
     if (smem > 48 * 1024) {
-        cudaError_t e = elem_bytes == 16
-            ? cudaFuncSetAttribute(k_apply_h_sweep<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)
-            : cudaFuncSetAttribute(k_apply_h_sweep<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return 1;
         }
     }
-    cudaError_t e = elem_bytes == 16
-        ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_apply_h_sweep<double>, kSweepThreads, smem)
-        : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_apply_h_sweep<float>, kSweepThreads, smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kSweepThreads, smem);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return 1;
@@ -348,13 +377,13 @@ cudaError_t launch_apply_h_sweep(const SweepDesc &W, const uint32_t *order, cons
                                  const uint32_t *pat, const uint32_t *tz, const void *ca,
                                  const void *cb, const void *hdiag, int n_qubits, int batch,
                                  const void *psi, void *lam, size_t state_stride, int first,
-                                 int last, unsigned long long *ctr, double *cpart, int blocks,
-                                 cudaStream_t s) {
+                                 int last, int n_elec, unsigned long long *ctr, double *cpart,
+                                 int blocks, cudaStream_t s) {
     using C = typename SV2<T>::type;
     if (W.t_count > kSweepMaxTerms || W.g_end - W.g_begin > kSweepMaxGroups || W.n_pat > kSweepMaxPat)
         return cudaErrorInvalidValue;
     const size_t smem = sweep_smem_bytes(W, sizeof(T));
-    auto kern = k_apply_h_sweep<T>;
+    auto kern = n_elec >= 0 ? k_apply_h_sweep<T, true> : k_apply_h_sweep<T, false>;
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -363,18 +392,18 @@ cudaError_t launch_apply_h_sweep(const SweepDesc &W, const uint32_t *order, cons
     return pdl_launch(kern, grid, kSweepThreads, smem, s, pdl_pays(grid), W, order, groups, pat, tz, static_cast<const T *>(ca),
                                            static_cast<const T *>(cb), static_cast<const T *>(hdiag),
                                            n_qubits, static_cast<const C *>(psi), static_cast<C *>(lam),
-                                           state_stride, first, last, ctr, cpart);
+                                           state_stride, first, last, n_elec, ctr, cpart);
 }
 
 template cudaError_t launch_apply_h_sweep<float>(const SweepDesc &, const uint32_t *, const SGroup *,
                                                  const uint32_t *, const uint32_t *, const void *,
                                                  const void *, const void *, int, int, const void *,
-                                                 void *, size_t, int, int, unsigned long long *,
+                                                 void *, size_t, int, int, int, unsigned long long *,
                                                  double *, int, cudaStream_t);
 template cudaError_t launch_apply_h_sweep<double>(const SweepDesc &, const uint32_t *, const SGroup *,
                                                   const uint32_t *, const uint32_t *, const void *,
                                                   const void *, const void *, int, int, const void *,
-                                                  void *, size_t, int, int, unsigned long long *,
+                                                  void *, size_t, int, int, int, unsigned long long *,
                                                   double *, int, cudaStream_t);
 
 }  // namespace vqe

@@ -1839,6 +1839,7 @@ template <typename T>
 vqe_status run_apply_h(vqe_ctx *h, int B, void *psi, void *lam, double *E) {
     cudaStream_t s = h->stream;
     const size_t N = h->state_elems();
+    const int sector = h->ansatz == 1 ? h->n_elec : -1;   // lambda is wanted where psi can be nonzero
     const int mk_h = prof_begin(h, 2);
     const bool windows = h->hd.apply_form == 1;
     const uint64_t atiles = windows ? (uint64_t(1) << (h->n - h->hd.wins[0].k)) : 0;
@@ -1857,7 +1858,7 @@ vqe_status run_apply_h(vqe_ctx *h, int B, void *psi, void *lam, double *E) {
         size_t smem = 0;
         for (const SweepDesc &W : h->hd.sweeps)
             smem = std::max(smem, sweep_smem_bytes(W, h->prec == VQE_C128 ? 8 : 4));
-        const int occ = sweep_blocks_per_sm(h->prec == VQE_C128 ? 16 : 8, smem);
+        const int occ = sweep_blocks_per_sm(h->prec == VQE_C128 ? 16 : 8, smem, sector >= 0);
         const int blocks = int(std::max<uint64_t>(1, std::min<uint64_t>(nchunks, uint64_t(h->sms) * occ / B)));
         auto *ctr = static_cast<unsigned long long *>(h->d_sctr.p);
         for (int w = 0; w < ns; ++w) {
@@ -1867,7 +1868,7 @@ vqe_status run_apply_h(vqe_ctx *h, int B, void *psi, void *lam, double *E) {
                                                 static_cast<const uint32_t *>(h->hd.d_spat.p),
                                                 static_cast<const uint32_t *>(h->hd.d_stz.p),
                                                 h->hd.d_sta.p, h->hd.d_stb.p, h->hd.hdiag(), h->n, B,
-                                                psi, lam, N, w == 0 ? 1 : 0, w == ns - 1 ? 1 : 0,
+                                                psi, lam, N, w == 0 ? 1 : 0, w == ns - 1 ? 1 : 0, sector,
                                                 ctr + size_t(w) * B, static_cast<double *>(h->d_epart.p),
                                                 blocks, s));
             h->stats.kernel_launches++;

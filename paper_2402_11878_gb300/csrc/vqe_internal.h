@@ -346,16 +346,17 @@ cudaError_t launch_apply_h_win(const WinDesc &W, const WinGroup *wgroups, const 
 // `ctr` holds one zeroed counter per state for this launch.  `order` points
 // at the sweep's 1024-entry bit-order table; terms, groups and patterns are
 // the whole plan's arrays (the sweep's ranges are in W); coefficients are T.
-// `blocks` blocks per state.
+// `blocks` blocks per state.  With n_elec >= 0 psi is zero outside the indexes of
+// n_elec ones and only those elements of lambda are computed.
 template <typename T>
 cudaError_t launch_apply_h_sweep(const SweepDesc &W, const uint32_t *order, const SGroup *groups,
                                  const uint32_t *pat, const uint32_t *tz, const void *ca,
                                  const void *cb, const void *hdiag, int n_qubits, int batch,
                                  const void *psi, void *lam, size_t state_stride, int first,
-                                 int last, unsigned long long *ctr, double *cpart, int blocks,
+                                 int last, int n_elec, unsigned long long *ctr, double *cpart, int blocks,
                                  cudaStream_t s);
 size_t sweep_smem_bytes(const SweepDesc &W, size_t real_bytes);
-int sweep_blocks_per_sm(int elem_bytes, size_t smem);
+int sweep_blocks_per_sm(int elem_bytes, size_t smem, bool sector);
 // Tile bits (log2 of elements) of the windowed expectation for a precision:
 // 512 threads hold 2^(kWinBits - 9) elements each.
 constexpr int win_tile_bits(bool c128) { return c128 ? 12 : 13; }

@@ -57,6 +57,25 @@ def test_fillings(pkg, oracle_mod, prec, n, ne):
     eng.close()
 
 
+@pytest.mark.parametrize("prec", ["c128", "c64"])
+@pytest.mark.parametrize("n,ne,batch", [(11, 4, 1), (12, 0, 1), (12, 6, 3), (13, 12, 1), (14, 7, 1), (15, 15, 2), (16, 5, 1)])
+def test_sweep_over_the_sector(pkg, oracle_mod, prec, n, ne, batch):
+    """lambda = H psi by sweeps over the sector's states (chunks of 2^12
+    counter values: one that is not full, one, several)."""
+    exc, H = _any_excitations(n, 30, 3 * n + ne), _random_hamiltonian(n, 30, 7 * n)
+    P = np.random.default_rng(n).uniform(-3, 3, (batch, len(exc)))
+    eng = pkg.Engine.particle_conserving(n, ne, exc, prec)
+    eng.set_hamiltonian(H.x, H.z, H.c)
+    assert eng.set_apply_mode(2) == 2
+    G, E = eng.gradient_batch(P)
+    for b in range(batch):
+        g_ref, E_ref = oracle_mod.pc_gradient_adjoint(n, ne, exc, P[b], H.x, H.z, H.c)
+        assert abs(E[b] - E_ref) <= (1e-11 if prec == "c128" else 1e-5) * H.sum_abs()
+        scale = max(1.0, float(np.max(np.abs(g_ref))))
+        assert np.max(np.abs(G[b] - g_ref)) <= (1e-10 if prec == "c128" else 1e-4) * scale
+    eng.close()
+
+
 @pytest.mark.parametrize("prec,batch", [("c128", 160), ("c64", 300)])
 def test_block_widths(pkg, prec, batch):
     n = 14
