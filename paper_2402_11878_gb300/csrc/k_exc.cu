@@ -21,21 +21,27 @@
 // 2048 (FP64) or 924 of 4096.  Shared memory holds just this class, in the order
 // of a constant table of the words sorted by popcount; a gate's live pairs are a
 // class of the words of its free bits; elements that no gate of the pass pairs
-// are not read or written.  lambda = H psi is needed, and kept up, in the sector
-// alone, because psi is zero elsewhere and the gates do not leave it.
-// At 28 qubits and half filling 15 % of the amplitudes are live; before, a whole
-// tile was read, rotated (64 FP64-pipe cycles per warp instruction) and written
-// back: 118 excitations in FP64, forward 59.1 -> 16.0 ms and backward 176.6 ->
-// 33.7 ms, complex64 at 27 qubits 13.0 -> 4.7 and 27.5 -> 8.1 ms.  What bounds
-// it now is the latency of a tile (two table look-ups, the load, a barrier per
-// gate), hidden by nine or more blocks per SM, and the memory's access size: the
-// scattered elements move in 32-byte sectors.
+// are not read or written.  Where every gate also keeps the electrons of one
+// spin's modes, elements with another number of those are left out too.
+// lambda = H psi is needed, and kept up, in the sector alone, because psi is zero
+// elsewhere and the gates do not leave it.
 //
+// At 28 qubits and half filling 15 % of the amplitudes have the right number of
+// ones, 4.4 % the right spins.  118 excitations in FP64, forward / backward:
+// whole tiles 59.1 / 176.6 ms, the number sector 16.0 / 33.5, with the spins
+// 14.7 / 22.2; complex64 at 27 qubits 13.0 / 27.5, 4.7 / 8.0, 4.5 / 5.9 ms.
+//
+// Before the wait for the kernel before, a warp per gate lists the gate's live
+// pairs (their places in shared memory, from the table), so that a gate is one
+// list entry, the rotation and a barrier (FP64, 14 qubits, 60 excitations: forward
+// 66 -> 48 us, backward 93 -> 73, against looking the places up at the gate).
 // FP64 gives a pair two lanes, one per component: half the FP64 instructions per
-// warp where the 35 pairs of a double (11 tile bits, 5 electrons) are all there
-// is.  All launches start before their predecessor has ended: what precedes the
-// first load of a state (gates, offsets, class words, places) is done by then
-// (FP64 at 17 qubits, 64 blocks: forward 212 -> 112 us).
+// warp where the 35 pairs of a double (11 tile bits, 5 electrons) are all there is.
+//
+// What bounds it now: at small sizes the chain of launch, staging and one
+// barrier per gate; at large ones the latency of a tile (nine or more blocks per
+// SM hide it) and the memory's 32-byte sectors, of which the scattered elements
+// fill a half.
 //
 // The backward (adjoint) pass un-applies the gates in reverse on psi and
 // lambda = H psi and, before un-applying gate g, takes
@@ -54,7 +60,7 @@ template <> struct XV2<double> { using type = double2; };
 
 constexpr int kExcMaxHigh = 7;   // k - m <= 7: 128 high-part offsets per pass
 constexpr int kExcWide = 256;             // threads of a block of a grid that leaves the chip room
-constexpr uint64_t kExcWideBlocks = 1024;
+constexpr uint64_t kExcWideBlocks = 608;   // four per SM
 
 template <typename T>
 __global__ void k_exc_stage(const double *__restrict__ params, int total, T *__restrict__ cs) {
@@ -83,8 +89,9 @@ struct TileGate {
     uint32_t word, pairs;    // its live pairs' free bits: kClass.word[word ...]
 };
 
-// Places of both elements of live pair f of a gate, and the pair's sign (bit 31).
-__device__ __forceinline__ uint32_t locate(const TileGate &G, uint32_t f, uint32_t at) {
+// Places of both elements of pair f of a gate, whether it is dead for its spins
+// (bit 30) and its sign (bit 31).
+__device__ __forceinline__ uint32_t locate(const TileGate &G, uint32_t f, uint32_t at, uint32_t up, int up_left) {
     uint32_t e = kClass.word[G.word + f];
     uint32_t fx = G.fixed;
     for (uint32_t i = 0; i < G.n_fixed; ++i, fx >>= 8) {   // zero bits at the gate's modes
@@ -93,6 +100,7 @@ __device__ __forceinline__ uint32_t locate(const TileGate &G, uint32_t f, uint32
     }
     e |= G.amask;
     return kClass.place[at + e] | (uint32_t)kClass.place[at + (e ^ G.flip)] << 15 |
+           (uint32_t)(__popc(e & up) != up_left) << 30 |
            (G.sign ^ (__popc(e & G.smask_t) & 1u)) << 31;
 }
 
@@ -108,7 +116,7 @@ __global__ void __launch_bounds__(TH)
 k_exc_pass(ExcPass P, const ExcGate *__restrict__ gates, const uint32_t *__restrict__ hoff,
            typename XV2<T>::type *__restrict__ psi, typename XV2<T>::type *__restrict__ lam,
            size_t stride, const T *__restrict__ cs, int n_exc, double *__restrict__ gpart,
-           size_t grad_stride, int init_hf, uint64_t hf, int room) {
+           size_t grad_stride, int init_hf, uint64_t hf, uint32_t spin, int room, int span) {
     using C = typename XV2<T>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ TileGate sg[kExcMaxGates];
@@ -122,6 +130,8 @@ k_exc_pass(ExcPass P, const ExcGate *__restrict__ gates, const uint32_t *__restr
     // backward: per-thread gradient partials, one row of TH per gate
     // (FP64 values, or compensated FP32 pairs in the FP32 kernel)
     unsigned char *rows = reinterpret_cast<unsigned char *>(sp + (BWD ? 2 * room : room));
+    // the gates' live pairs (locate), `span` words each
+    uint32_t *list = reinterpret_cast<uint32_t *>(rows + (BWD ? (size_t)ng * TH * 8 : 0));
     const int b = blockIdx.y;
     C *Pp = psi + (size_t)b * stride;
     C *Lp = BWD ? lam + (size_t)b * stride : nullptr;
@@ -145,14 +155,18 @@ k_exc_pass(ExcPass P, const ExcGate *__restrict__ gates, const uint32_t *__restr
     static_assert(2 * kExcMaxGates <= TH, "one entry per thread");
     const uint32_t lowmask = (1u << m) - 1u;
     const int left = __popcll(hf) - __popcll(base);   // electrons in the tile's modes
-    const bool live = left >= 0 && left <= k &&
+    // and those of them in the modes of `spin`, of which the tile has n_up
+    const int up_left = __popc((uint32_t)hf & spin) - __popc((uint32_t)base & spin);
+    const int n_up = __popc(spin & ~P.bmask);
+    const bool live = left >= 0 && left <= k && up_left >= 0 && up_left <= n_up &&
+                      left - up_left >= 0 && left - up_left <= k - n_up &&
                       (BWD ? (base & P.bzmask) == P.bzval : (base & P.zmask) == P.zval);   // block-uniform
     constexpr int kPer = (sizeof(T) == 8 ? 512 : 1024) / TH;   // C(11,5) = 462, C(12,6) = 924 live ones
     constexpr uint32_t kSplit = sizeof(T) == 8 ? 2 : 1;   // lanes per pair; FP64: one per component
     constexpr uint32_t kNone = ~0u;
     uint32_t at_g[kPer];     // where this thread's elements of the class lie in the state
     uint32_t mine = 0u;      // which of them the pass moves
-    uint32_t nxt = 0u;       // the next gate's first pair, found while this one's is computed
+    uint32_t up = 0u;        // the modes of `spin` among the tile bits
     if (live) {
         if ((int)tid < ng) {
             const ExcGate my = gates[P.g_begin + tid];
@@ -176,6 +190,11 @@ k_exc_pass(ExcPass P, const ExcGate *__restrict__ gates, const uint32_t *__restr
             at_g[u] = j < n_live ? kClass.word[at + first + j] : kNone;
         }
         __syncthreads();
+        {
+            const uint32_t lane = tid & 31u;
+            const bool in = (int)lane < k - m && (shoff[1u << lane] & spin) != 0u;
+            up = (spin & lowmask) | __ballot_sync(0xffffffffu, in) << m;
+        }
         // only elements that a gate pairs are read and written
 #pragma unroll
         for (int u = 0; u < kPer; ++u) {
@@ -186,11 +205,23 @@ k_exc_pass(ExcPass P, const ExcGate *__restrict__ gates, const uint32_t *__restr
                 const uint32_t v = e & sg[i].flip;
                 used |= v == sg[i].amask || (v ^ sg[i].flip) == sg[i].amask;
             }
+            used = used && ((!BWD && init_hf) || __popc(e & up) == up_left);
             mine |= (uint32_t)used << u;
             at_g[u] = (uint32_t)base | (e & lowmask) | shoff[e >> m];
         }
-        const TileGate &G = sg[BWD ? ng - 1 : 0];
-        if (tid / kSplit < G.pairs) nxt = locate(G, tid / kSplit, at);
+        // the gates' lists of live pairs, a gate per warp
+        for (int i = tid >> 5; i < ng; i += TH / 32) {
+            const uint32_t pairs = sg[i].pairs, lane = tid & 31u;
+            uint32_t n = 0;
+            for (uint32_t f = lane; f - lane < pairs; f += 32) {
+                const uint32_t loc = f < pairs ? locate(sg[i], f, at, up, up_left) : 1u << 30;
+                const bool ok = ((loc >> 30) & 1u) == 0u;
+                const uint32_t votes = __ballot_sync(0xffffffffu, ok);
+                if (ok) list[i * span + n + __popc(votes & ((1u << lane) - 1u))] = loc;
+                n += __popc(votes);
+            }
+            if (lane == 0) sg[i].pairs = n;
+        }
     }
     pdl_wait();
     if (!live) {
@@ -240,15 +271,10 @@ k_exc_pass(ExcPass P, const ExcGate *__restrict__ gates, const uint32_t *__restr
         const TileGate &G = sg[i];
         const T c = scs[2 * i], s = scs[2 * i + 1];
         const uint32_t count = G.pairs * kSplit;
-        uint32_t loc = nxt;
-        if (ii + 1 < ng) {
-            const TileGate &N = sg[BWD ? i - 1 : i + 1];
-            if (tid / kSplit < N.pairs) nxt = locate(N, tid / kSplit, at);
-        }
         double gd = 0.0;
         F32c gf = f32c_zero();
         for (uint32_t f = tid; f < count; f += TH) {
-            if (f != tid) loc = locate(G, f / kSplit, at);
+            const uint32_t loc = list[i * span + f / kSplit];
             const uint32_t i1 = loc & 0x7fffu, i2 = (loc >> 15) & 0x7fffu, par = loc >> 31;
             const T ss = xflip(s, par);
             if constexpr (sizeof(T) == 8) {
@@ -340,7 +366,7 @@ template <typename T>
 cudaError_t launch_exc_pass(const ExcPass &P, const ExcGate *gates_dev, const uint32_t *hoff_dev,
                             int n_qubits, int batch, void *psi, void *lam, size_t state_stride,
                             const T *cs, int n_exc, double *gpart, size_t grad_stride,
-                            bool backward, int init_hf, uint64_t hf_index, cudaStream_t s) {
+                            bool backward, int init_hf, uint64_t hf_index, uint32_t spin, cudaStream_t s) {
     using C = typename XV2<T>::type;
     const dim3 grid(1u << (n_qubits - P.k), batch);
     int room = 1;   // the largest class: binomial(k, k / 2)
@@ -349,15 +375,22 @@ cudaError_t launch_exc_pass(const ExcPass &P, const ExcGate *gates_dev, const ui
     const size_t row = sizeof(T) == 8 ? sizeof(double) : sizeof(F32c);
     // 256 threads where a grid leaves the chip room, for a shorter chain per gate;
     // 128 beyond, for more tiles per SM.  FP64, forward + backward of 100
-    // excitations, 128 / 256 threads: 14 qubits (8 blocks) 302 / 270 us, 20 (512)
-    // 574 / 565, 21 (1024) 822 / 798, 22 (2048) 1139 / 1150, 24 3.02 / 3.41 ms;
-    // complex64: 18 (64) 316 / 260 us, 22 (1024) 595 / 564, 24 1.48 / 1.60 ms.
+    // excitations, 128 / 256 threads: 14 qubits (8 blocks) 200 / 184 us, 18 (128)
+    // 304 / 242, 20 (512) 390 / 327, 21 (1024) 471 / 578; complex64: 18 (64) 183 /
+    // 160 us, 21 (512) 293 / 304, 22 (1024) 409 / 547.
     const int th = uint64_t(grid.x) * grid.y <= kExcWideBlocks ? kExcWide : kExcThreads;
-    const size_t smem = room * sizeof(C) * (backward ? 2 : 1) + (backward ? size_t(P.n_gates) * th * row : 0);
+    int span = 1;   // the most pairs: a single's, binomial(k - 2, (k - 2) / 2)
+    for (int i = 1; i <= (P.k - 2) / 2; ++i) span = span * (P.k - 1 - i) / i;
+    const size_t smem = room * sizeof(C) * (backward ? 2 : 1) +
+                        P.n_gates * ((backward ? th * row : 0) + span * sizeof(uint32_t));
     auto launch = [&](auto kern) {
+        if (smem > 40 * 1024) {   // with the static part beyond the default 48 KiB
+            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+            if (e != cudaSuccess) return e;
+        }
         return pdl_launch(kern, grid, th, smem, s, true, P, gates_dev, hoff_dev, static_cast<C *>(psi),
                           static_cast<C *>(lam), state_stride, cs, n_exc, gpart, grad_stride, init_hf, hf_index,
-                          room);
+                          spin, room, span);
     };
     if (th == kExcWide) return backward ? launch(k_exc_pass<T, true, kExcWide>) : launch(k_exc_pass<T, false, kExcWide>);
     return backward ? launch(k_exc_pass<T, true, kExcThreads>) : launch(k_exc_pass<T, false, kExcThreads>);
@@ -367,9 +400,9 @@ template cudaError_t launch_exc_stage<float>(const double *, int, int, float *, 
 template cudaError_t launch_exc_stage<double>(const double *, int, int, double *, cudaStream_t);
 template cudaError_t launch_exc_pass<float>(const ExcPass &, const ExcGate *, const uint32_t *, int,
                                             int, void *, void *, size_t, const float *, int,
-                                            double *, size_t, bool, int, uint64_t, cudaStream_t);
+                                            double *, size_t, bool, int, uint64_t, uint32_t, cudaStream_t);
 template cudaError_t launch_exc_pass<double>(const ExcPass &, const ExcGate *, const uint32_t *, int,
                                              int, void *, void *, size_t, const double *, int,
-                                             double *, size_t, bool, int, uint64_t, cudaStream_t);
+                                             double *, size_t, bool, int, uint64_t, uint32_t, cudaStream_t);
 
 }  // namespace vqe

@@ -143,6 +143,7 @@ struct vqe_ctx {
     uint64_t hf_index = 0;
     std::vector<int> exc;                // 4 per excitation, in the order of application
     std::vector<ExcPass> pc_passes;
+    uint32_t pc_spin = 0;
     DevBuf d_pc_gates, d_pc_hoff;
     int pc_k = 0;
 
@@ -766,6 +767,23 @@ bool make_pc_plan(int n, vqe_precision prec, const std::vector<int> &exc, uint64
     return true;
 }
 
+// Modes whose electron number every excitation keeps: one spin's, where they
+// alternate (mode = 2 site + spin) or fill the lower half; 0 if neither is kept.
+uint32_t conserved_spin(int n, const std::vector<int> &exc) {
+    const uint32_t nmask = n >= 32 ? 0xffffffffu : (1u << n) - 1u;
+    for (uint32_t mask : {0x55555555u & nmask, (1u << (n / 2)) - 1u}) {
+        bool kept = true;
+        for (size_t j = 0; j + 3 < exc.size() && kept; j += 4) {
+            int moved = 0;
+            for (int u = 0; u < 4; ++u)
+                if (exc[j + u] >= 0 && ((mask >> exc[j + u]) & 1u)) moved += u < 2 ? 1 : -1;
+            kept = moved == 0;
+        }
+        if (kept) return mask;
+    }
+    return 0u;
+}
+
 vqe_status build_pc_plan(vqe_ctx *h) {
     PcHostPlan pp;
     std::string err;
@@ -778,6 +796,7 @@ vqe_status build_pc_plan(vqe_ctx *h) {
     if ((st = upload(h, P.d_gcnt, pp.gcnt, "grad map")) != VQE_OK) return st;
     if ((st = upload(h, P.d_gstep, pp.gstep, "grad map")) != VQE_OK) return st;
     h->pc_passes = pp.passes;
+    h->pc_spin = conserved_spin(h->n, h->exc);
     h->pc_k = pp.k;
     for (int w = 0; w < 2; ++w) {
         h->plan[w].fwd.clear();
@@ -1732,7 +1751,7 @@ vqe_status run_forward_pc(vqe_ctx *h, const double *params_dev, int B, void *psi
         VQE_CUDA(h, launch_exc_pass<T>(h->pc_passes[p], static_cast<const ExcGate *>(h->d_pc_gates.p),
                                        static_cast<const uint32_t *>(h->d_pc_hoff.p), h->n, B, psi,
                                        nullptr, h->state_elems(), cs, K, nullptr, 0, false,
-                                       p == 0 ? 1 : 0, h->hf_index, h->stream));
+                                       p == 0 ? 1 : 0, h->hf_index, h->pc_spin, h->stream));
         h->stats.kernel_launches++;
     }
     prof_end(h, mk, int(h->pc_passes.size()));
@@ -1749,7 +1768,7 @@ vqe_status run_backward_pc(vqe_ctx *h, int B, void *psi, void *lam) {
         VQE_CUDA(h, launch_exc_pass<T>(h->pc_passes[p], static_cast<const ExcGate *>(h->d_pc_gates.p),
                                        static_cast<const uint32_t *>(h->d_pc_hoff.p), h->n, B, psi,
                                        lam, h->state_elems(), cs, K, gpart, h->plan[1].grad_stride,
-                                       true, 0, h->hf_index, h->stream));
+                                       true, 0, h->hf_index, h->pc_spin, h->stream));
         h->stats.kernel_launches++;
     }
     prof_end(h, mk, int(h->pc_passes.size()));

@@ -139,11 +139,13 @@ struct ExcPass {
 template <typename T>
 cudaError_t launch_exc_stage(const double *params, int n_exc, int batch, T *cs, cudaStream_t s);
 
+// `spin`: modes that every gate of the ansatz leaves with as many electrons as it
+// found (one spin's modes; 0 if there are none such).
 template <typename T>
 cudaError_t launch_exc_pass(const ExcPass &P, const ExcGate *gates_dev, const uint32_t *hoff_dev,
                             int n_qubits, int batch, void *psi, void *lam, size_t state_stride,
                             const T *cs, int n_exc, double *gpart, size_t grad_stride,
-                            bool backward, int init_hf, uint64_t hf_index, cudaStream_t s);
+                            bool backward, int init_hf, uint64_t hf_index, uint32_t spin, cudaStream_t s);
 
 // ---------------------------------------------------------------- Hamiltonian
 //

@@ -1,7 +1,7 @@
 """The excitation passes hold only the amplitudes of the n_elec sector that a
 pass's gates pair: fillings from empty to full, excitations without a pair in
 the sector, Hamiltonians that leave the sector, both block widths (a grid of
-more than 1024 blocks takes the narrow one) and an angle that is not a number.
+more than 608 blocks takes the narrow one) and an angle that is not a number.
 
 Tolerances as in test_gpu_pc.py; the two block widths add the same terms in
 another order: FP64 1e-13 of the gradient's largest entry, complex64
@@ -54,6 +54,35 @@ def test_fillings(pkg, oracle_mod, prec, n, ne):
     assert abs(E - E_ref) <= (1e-11 if prec == "c128" else 1e-5) * H.sum_abs()
     scale = max(1.0, float(np.max(np.abs(g_ref))))
     assert np.max(np.abs(g - g_ref)) <= (1e-10 if prec == "c128" else 1e-4) * scale
+    eng.close()
+
+
+@pytest.mark.parametrize("prec", ["c128", "c64"])
+@pytest.mark.parametrize("order", ["alternating", "halves"])
+@pytest.mark.parametrize("n,ne", [(8, 3), (13, 7), (14, 2), (15, 8)])
+def test_spins_kept_apart(pkg, oracle_mod, prec, order, n, ne):
+    """Excitations that keep each spin's electrons, under both mode orders;
+    the Hamiltonian keeps neither."""
+    rng = np.random.default_rng(17 * n + ne)
+    up = np.arange(0, n, 2) if order == "alternating" else np.arange(n // 2)
+    down = np.setdiff1d(np.arange(n), up)
+    exc = []
+    for j in range(36):
+        a, b = rng.permutation(up), rng.permutation(down)
+        exc.append([[a[0], -1, a[1], -1], [b[0], -1, b[1], -1], [a[0], b[0], a[1], b[1]],
+                    [a[0], b[0], b[1], a[1]], [*a[:4]] if len(a) > 3 else [a[0], -1, a[2], -1]][j % 5])
+    exc, H = np.array(exc, dtype=np.int32), _random_hamiltonian(n, 30, n)
+    th = rng.uniform(-3, 3, len(exc))
+    eng = pkg.Engine.particle_conserving(n, ne, exc, prec)
+    eng.set_hamiltonian(H.x, H.z, H.c)
+    g, E = eng.gradient(th)
+    g_ref, E_ref = oracle_mod.pc_gradient_adjoint(n, ne, exc, th, H.x, H.z, H.c)
+    assert abs(E - E_ref) <= (1e-11 if prec == "c128" else 1e-5) * H.sum_abs()
+    scale = max(1.0, float(np.max(np.abs(g_ref))))
+    assert np.max(np.abs(g - g_ref)) <= (1e-10 if prec == "c128" else 1e-4) * scale
+    eng.apply_ansatz(th)
+    ref = oracle_mod.pc_ansatz_state(n, ne, exc, th)
+    assert np.max(np.abs(eng.get_state() - ref)) <= (1e-12 if prec == "c128" else 2e-6)
     eng.close()
 
 
