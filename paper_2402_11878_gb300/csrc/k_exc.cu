@@ -378,7 +378,12 @@ cudaError_t launch_exc_pass(const ExcPass &P, const ExcGate *gates_dev, const ui
     // excitations, 128 / 256 threads: 14 qubits (8 blocks) 200 / 184 us, 18 (128)
     // 304 / 242, 20 (512) 390 / 327, 21 (1024) 471 / 578; complex64: 18 (64) 183 /
     // 160 us, 21 (512) 293 / 304, 22 (1024) 409 / 547.
-    const int th = uint64_t(grid.x) * grid.y <= kExcWideBlocks ? kExcWide : kExcThreads;
+    // FP64 forward has half the rows to move and no partials: 64 threads from 2048
+    // blocks on (22 qubits 276 -> 232 us, 24 789 -> 709, 28 14.7 -> 12.7 ms; at 1024
+    // blocks 163 -> 192 us, and backward and complex64 are slower with 64).
+    const uint64_t blocks = uint64_t(grid.x) * grid.y;
+    const bool small = sizeof(T) == 8 && !backward && blocks >= 2048;
+    const int th = small ? 64 : blocks <= kExcWideBlocks ? kExcWide : kExcThreads;
     int span = 1;   // the most pairs: a single's, binomial(k - 2, (k - 2) / 2)
     for (int i = 1; i <= (P.k - 2) / 2; ++i) span = span * (P.k - 1 - i) / i;
     const size_t smem = room * sizeof(C) * (backward ? 2 : 1) +
@@ -393,6 +398,8 @@ cudaError_t launch_exc_pass(const ExcPass &P, const ExcGate *gates_dev, const ui
                           spin, room, span);
     };
     if (th == kExcWide) return backward ? launch(k_exc_pass<T, true, kExcWide>) : launch(k_exc_pass<T, false, kExcWide>);
+    if constexpr (sizeof(T) == 8)
+        if (small) return launch(k_exc_pass<T, false, 64>);
     return backward ? launch(k_exc_pass<T, true, kExcThreads>) : launch(k_exc_pass<T, false, kExcThreads>);
 }
 

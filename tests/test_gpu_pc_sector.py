@@ -1,9 +1,9 @@
 """The excitation passes hold only the amplitudes of the n_elec sector that a
 pass's gates pair: fillings from empty to full, excitations without a pair in
-the sector, Hamiltonians that leave the sector, both block widths (a grid of
-more than 608 blocks takes the narrow one) and an angle that is not a number.
+the sector, Hamiltonians that leave the sector, the block widths (a grid of more
+than 608 blocks takes a narrower one, FP64 forward again from 2048) and an angle that is not a number.
 
-Tolerances as in test_gpu_pc.py; the two block widths add the same terms in
+Tolerances as in test_gpu_pc.py; the block widths add the same terms in
 another order: FP64 1e-13 of the gradient's largest entry, complex64
 (compensated FP32 partials, 2^-46 of the sum of the terms' magnitudes) 1e-9.
 """
@@ -105,7 +105,7 @@ def test_sweep_over_the_sector(pkg, oracle_mod, prec, n, ne, batch):
     eng.close()
 
 
-@pytest.mark.parametrize("prec,batch", [("c128", 160), ("c64", 300)])
+@pytest.mark.parametrize("prec,batch", [("c128", 160), ("c128", 300), ("c64", 300)])
 def test_block_widths(pkg, prec, batch):
     n = 14
     exc, H = vi.excitations(n, 6, 8, 24, seed=2), vi.hubbard_1d(7, 1.0, 4.0)
