@@ -24,6 +24,7 @@ from __future__ import annotations
 
 import argparse
 import json
+import math
 import os
 import platform
 import statistics
@@ -50,10 +51,10 @@ FP64_UNITS_PEAK = 152 * 2 * 2 * 2.070e9 / 1e12   # SMs x DFMA/clk/SM x 2 flop x 
 # DRAM read + write bytes of the FP64 backward pass kernel per byte it must
 # move (psi and lambda read and written per live tile), from an ncu capture
 # of its three launch shapes at 24 qubits on the 4x3 lattice (dram__bytes
-# read + write: 3.119 GB against 3.221 GB); the per-tile traffic of these
+# read + write: 3.049 GB against 3.221 GB); the per-tile traffic of these
 # passes does not depend on the qubit count.  None once the kernel changes,
 # until it is captured again.
-BWD_TRAFFIC_PER_ALGORITHMIC_BYTE = 3119003392 / 3221225472
+BWD_TRAFFIC_PER_ALGORITHMIC_BYTE = 3049170432 / 3221225472
 
 
 # ---------------------------------------------------------------- work models
@@ -454,19 +455,23 @@ def run_gpu(args, world, rank, local, pg):
                             "tflops": fl_b / (bwd_ms / 1e3) / 1e12,
                             "hbm_gbs": by_b / (bwd_ms / 1e3) / 1e9},
     }
-    achieved = fl_b / (bwd_ms / 1e3) / 1e12
-    roofline = {"bound": "alu", "achieved": achieved, "peak": fp64_peak, "unit": "TFLOP/s",
-                "frac": achieved / fp64_peak,
+    # The backward passes run in 64-bit fixed point: bound by the issue of
+    # integer instructions, so their fraction is given of the memory's rate; the
+    # FP64 multiply-add rate, which the same work in FP64 cannot exceed, beside it.
+    achieved = by_b / (bwd_ms / 1e3) / 1e9
+    roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
+                "frac": achieved / hbm_peak if hbm_peak else None,
                 "traffic": (by_b / bwd_launches * BWD_TRAFFIC_PER_ALGORITHMIC_BYTE
                             if BWD_TRAFFIC_PER_ALGORITHMIC_BYTE else None),
-                "kernel": "k_pass_fixed<double,3,bwd> (adjoint backward tile passes)",
-                "peak_source": ("measured FP64 FMA rate of this GPU (vqe_measure_fma_peak, "
-                                "independent FMA chains on every SM, CUDA events); unit count x "
-                                f"max clock gives {FP64_UNITS_PEAK:.4g}"),
+                "kernel": "k_pass_fx<bwd> (adjoint backward tile passes, 64-bit block fixed point)",
+                "peak_source": "measured HBM copy bandwidth",
+                "algorithmic_tflops": fl_b / (bwd_ms / 1e3) / 1e12, "fp64_fma_peak_tflops": fp64_peak,
+                "fp64_fma_peak_source": ("measured FP64 FMA rate of this GPU (vqe_measure_fma_peak, "
+                                         "independent FMA chains on every SM, CUDA events); unit count x "
+                                         f"max clock gives {FP64_UNITS_PEAK:.4g}"),
                 "algorithmic_flops_per_launch": fl_b / bwd_launches,
                 "mean_launch_ms": bwd_ms / bwd_launches,
                 "share_of_step": bwd_ms / (ms / steps),
-                "hbm_gbs_moved": by_b / (bwd_ms / 1e3) / 1e9, "hbm_peak_gbs": hbm_peak,
                 # the memory view of the whole evaluation: (6D + 2) state
                 # sweeps of b N bytes at the algorithmic minimum (forward read
                 # + write per layer, lambda written, backward psi and lambda
@@ -744,25 +749,18 @@ def run_workload(name: str, args):
             npass = eng.stats()["ansatz_passes"]
             f_ms = pr["forward_passes"]["ms"] / reps
             b_ms = pr["backward_passes"]["ms"] / reps
-            # bytes the passes must move: one read and write of every tile in
-            # the support of the state (the first pass writes the rest as zeros)
-            from paper_2402_11878_gb300 import plans
-            pl = plans.pc_plan(n, prec, exc, ne)
-            by_f = by_b = 0.0
-            for i, Pp in enumerate(pl["passes"]):
-                tile = st * (1 << Pp.k)
-                tiles = 1 << (n - Pp.k)
-                live_f = 1 << (bin(Pp.bmask).count("1") - bin(Pp.zmask).count("1"))
-                live_b = 1 << (bin(Pp.bmask).count("1") - bin(Pp.bzmask).count("1"))
-                by_f += tile * (2 * live_f + (tiles - live_f if i == 0 else 0))
-                by_b += tile * 4 * live_b
+            # amplitudes that can differ from zero (both spins' electrons are
+            # kept), once read and written per pass and buffer: an upper bound
+            # of what the passes need, which move only what their gates pair
+            sector = st * math.comb(n // 2, ne // 2) ** 2
+            by_f, by_b = npass * 2 * sector, npass * 4 * sector
             out[prec] = {"evals_per_s": 1e3 / ms, "ms_per_eval": ms, "energy": float(E[0]),
                          "passes": npass, "apply_form": tune["apply_form"],
                          "forward_ms": f_ms, "apply_h_ms": pr["apply_h"]["ms"] / reps,
                          "backward_ms": b_ms,
-                         "forward_hbm_gbs": by_f / (f_ms / 1e3) / 1e9,
-                         "backward_hbm_gbs": by_b / (b_ms / 1e3) / 1e9,
-                         "support_fraction": by_b / (npass * 4 * st * float(1 << n)),
+                         "forward_sector_gbs": by_f / (f_ms / 1e3) / 1e9,
+                         "backward_sector_gbs": by_b / (b_ms / 1e3) / 1e9,
+                         "sector_fraction": sector / (st * float(1 << n)),
                          "grad_inf": float(G.abs().max())}
             g = G[0].cpu().numpy().copy()
             if prec == "c128":

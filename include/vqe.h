@@ -31,7 +31,14 @@
  *     back to back.
  *   - Energies are <psi|H|psi>/<psi|psi> (Eq. 7); gradients are of the
  *     unnormalised <psi|H|psi> (equal for the unitary circuit).
- *   - Precision: VQE_C128 computes everything in FP64.  VQE_C64 keeps the
+ *   - Precision: VQE_C128 keeps the state in FP64 and computes in FP64, but for
+ *     the passes of the layered ansatz with reg_bits 3 (the default): these
+ *     turn a tile of up to 2^12 amplitudes into 64-bit fixed point with one
+ *     exponent per tile and back.  Their error is relative to the tile's norm,
+ *     not to each amplitude: below that of FP64 arithmetic for states and
+ *     gradients (root mean square 5.8e-16 against 8.8e-16, 1.1e-15 against
+ *     2.1e-15), while an amplitude 2^-50 times smaller than its tile's norm
+ *     keeps few significant bits.  VQE_C64 keeps the
  *     state in complex64 and does gate arithmetic in FP32, and accumulates
  *     energies, norms and gradients in FP64.
  *

@@ -29,7 +29,7 @@
 // At 28 qubits and half filling 15 % of the amplitudes have the right number of
 // ones, 4.4 % the right spins.  118 excitations in FP64, forward / backward:
 // whole tiles 59.1 / 176.6 ms, the number sector 16.0 / 33.5, with the spins
-// 14.7 / 22.2; complex64 at 27 qubits 13.0 / 27.5, 4.7 / 8.0, 4.5 / 5.9 ms.
+// 12.7 / 22.2; complex64 at 27 qubits 13.0 / 27.5, 4.7 / 8.0, 4.5 / 5.9 ms.
 //
 // Before the wait for the kernel before, a warp per gate lists the gate's live
 // pairs (their places in shared memory, from the table), so that a gate is one

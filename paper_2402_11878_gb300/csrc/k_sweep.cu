@@ -91,9 +91,10 @@ __device__ __forceinline__ void sweep_block_sum_c(F32c a, F32c b, float *sh, dou
 // states are one class of equal popcount; its words come from the class table.
 // Other elements of lambda are left as they are.  28 qubits FP64, half filling,
 // 43 groups: 29.1 ms for the whole state (bound by the FP64 pipe), 8.8 for the
-// 15 % in the sector; there the gathers' latency counts (16.6 with one state's
-// gather after the other, inside the vote), so the J states' are issued together
-// as in complex64.  complex64 at 27 qubits: 3.75 -> 1.03 ms.
+// 15 % in the sector, again bound by the FP64 pipe (94 % busy at 24 qubits: a warp
+// of sector states mixes every group's patterns, so none skips its multiply-adds).
+// The J states' gathers are issued together, as in complex64: 16.6 ms with one
+// after the other inside the vote.  complex64 at 27 qubits: 3.75 -> 1.03 ms.
 template <typename T, bool SECTOR>
 __global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 3 : 4)
 k_apply_h_sweep(SweepDesc W, const uint32_t *__restrict__ order, const SGroup *__restrict__ groups,
