@@ -36,7 +36,9 @@ def sources():
 
 
 def _deps_mtime() -> float:
-    files = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(INCLUDE, "*.h"))
+    files = sources()
+    for pattern in (os.path.join(CSRC, "*.h"), os.path.join(CSRC, "*.cuh"), os.path.join(INCLUDE, "*.h")):
+        files += glob.glob(pattern)
     return max(os.path.getmtime(f) for f in files)
 
 
