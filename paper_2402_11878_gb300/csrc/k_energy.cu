@@ -112,8 +112,8 @@ template <typename T>
 __global__ void __launch_bounds__(kEnergyThreads)
 k_energy_cols(const GroupDesc *__restrict__ groups, int n_groups, const uint32_t *__restrict__ tz,
               const T *__restrict__ tc, const T *__restrict__ hdiag, int n,
-              const typename EV2<T>::type *__restrict__ psi, size_t stride,
-              double *__restrict__ partials, int block_off, int bps_total) {
+              const typename EV2<T>::type *psi, size_t stride,
+              double *partials, int block_off, int bps_total) {
     pdl_trigger();
     pdl_wait();
     using C = typename EV2<T>::type;
@@ -222,8 +222,8 @@ template <typename T>
 __global__ void __launch_bounds__(kEnergyThreads)
 k_apply_h(const GroupDesc *__restrict__ groups, int n_groups, const uint32_t *__restrict__ tz,
           const T *__restrict__ tc, const T *__restrict__ hdiag, int n,
-          const typename EV2<T>::type *__restrict__ psi, typename EV2<T>::type *__restrict__ lam,
-          size_t stride, double *__restrict__ partials) {
+          const typename EV2<T>::type *psi, typename EV2<T>::type *lam,
+          size_t stride, double *partials) {
     pdl_trigger();
     pdl_wait();
     using C = typename EV2<T>::type;
@@ -280,6 +280,9 @@ k_apply_h(const GroupDesc *__restrict__ groups, int n_groups, const uint32_t *__
                 }
             }
         }
+        C xj[J];   // loaded together, before the first store
+#pragma unroll
+        for (int j = 0; j < J; ++j) xj[j] = P[i[j]];
 #pragma unroll
         for (int j = 0; j < J; ++j) {
             if (!ok[j]) continue;
@@ -287,7 +290,7 @@ k_apply_h(const GroupDesc *__restrict__ groups, int n_groups, const uint32_t *__
             out.x = lr[j];
             out.y = li[j];
             L[i[j]] = out;
-            const C x = P[i[j]];
+            const C x = xj[j];
             acc += (double)fma(x.x, lr[j], x.y * li[j]);
             nrm += (double)fma(x.x, x.x, x.y * x.y);
         }
@@ -336,7 +339,7 @@ template cudaError_t launch_build_hdiag<double>(const uint32_t *, const double *
 // partials, then a fixed-order tree over the block (bitwise reproducible).
 constexpr int kFinishThreads = 256;
 __global__ void __launch_bounds__(kFinishThreads)
-k_energy_finish(const double *__restrict__ partials, int bps, int batch, double *energies,
+k_energy_finish(const double *partials, int bps, int batch, double *energies,
                 double *norms, double *unnorm) {
     pdl_trigger();
     pdl_wait();
@@ -369,7 +372,7 @@ k_energy_finish(const double *__restrict__ partials, int bps, int batch, double 
 // fixed-order tree over the block (bitwise reproducible).
 constexpr int kGradThreads = 128;
 __global__ void __launch_bounds__(kGradThreads)
-k_grad_finish(const double *__restrict__ part, size_t part_stride, const int *__restrict__ off,
+k_grad_finish(const double *part, size_t part_stride, const int *__restrict__ off,
               const int *__restrict__ count, const int *__restrict__ step, int n_params,
               double *grads) {
     pdl_trigger();
@@ -509,8 +512,8 @@ template <typename T, int K, bool RUNS>
 __global__ void __launch_bounds__(kEnergyWinThreads, 2)
 k_energy_win(WinDesc W, const WinGroup *__restrict__ wgroups, const WinTerm *__restrict__ wterms,
              const uint32_t *__restrict__ hoff, const T *__restrict__ hdiag,
-             const typename EV2<T>::type *__restrict__ psi, size_t stride,
-             double *__restrict__ partials, int bps_total) {
+             const typename EV2<T>::type *psi, size_t stride,
+             double *partials, int bps_total) {
     pdl_trigger();
     pdl_wait();
     using C = typename EV2<T>::type;
@@ -732,8 +735,8 @@ template <typename T, int K, bool RUNS>
 __global__ void __launch_bounds__(kEnergyWinThreads, 1)
 k_apply_h_win(WinDesc W, const WinGroup *__restrict__ wgroups, const WinTerm *__restrict__ wterms,
               const uint32_t *__restrict__ hoff, const T *__restrict__ hdiag,
-              const typename EV2<T>::type *__restrict__ psi, typename EV2<T>::type *__restrict__ lam,
-              size_t stride, int first, int last, double *__restrict__ partials) {
+              const typename EV2<T>::type *psi, typename EV2<T>::type *lam,
+              size_t stride, int first, int last, double *partials) {
     pdl_trigger();
     pdl_wait();
     using C = typename EV2<T>::type;

@@ -114,8 +114,8 @@ __device__ __forceinline__ float xflip(float v, uint32_t s) {
 template <typename T, bool BWD, int TH>
 __global__ void __launch_bounds__(TH)
 k_exc_pass(ExcPass P, const ExcGate *__restrict__ gates, const uint32_t *__restrict__ hoff,
-           typename XV2<T>::type *__restrict__ psi, typename XV2<T>::type *__restrict__ lam,
-           size_t stride, const T *__restrict__ cs, int n_exc, double *__restrict__ gpart,
+           typename XV2<T>::type *psi, typename XV2<T>::type *lam,
+           size_t stride, const T *cs, int n_exc, double *gpart,
            size_t grad_stride, int init_hf, uint64_t hf, uint32_t spin, int room, int span) {
     using C = typename XV2<T>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -140,7 +140,7 @@ struct GridEnv {
     int init_zero;
     int t0;         // lowest gated tile bit: the tables have no index bits below it
     __device__ RotCoef<T> coef(int slot, int bit) const { return cf[slot * d->k + bit]; }
-    __device__ C diag(int slot, uint32_t e) const { return __ldg(dt + d->slot_dtab_off[slot] + (e >> t0)); }
+    __device__ C diag(int slot, uint32_t e) const { return chain_load(dt + d->slot_dtab_off[slot] + (e >> t0)); }
     __device__ void grad(int slot, int bit, int comp, double v) const {
         gout[d->slot_grad_off[slot] + tile * (uint64_t)(2 * d->k) + bit * 2 + comp] = v;
     }
@@ -150,7 +150,7 @@ struct GridEnv {
 // memory, so the op interpreter reads them with shared-memory loads.
 template <typename T>
 __device__ __forceinline__ void stage_pass(const PassDesc *__restrict__ desc,
-                                           const RotCoef<T> *__restrict__ cf, PassDesc *sd,
+                                           const RotCoef<T> *cf, PassDesc *sd,
                                            RotCoef<T> *scf) {
     static_assert(sizeof(PassDesc) % 4 == 0, "descriptor copied in words");
     const uint32_t *src = reinterpret_cast<const uint32_t *>(desc);
@@ -222,10 +222,10 @@ __device__ __forceinline__ void write_product_tile(const PassDesc &d, const RotC
 // SM (<= 64 registers); backward passes hold two.
 template <typename T, int R, bool BWD>
 __global__ void __launch_bounds__(kPassMaxThreads, (BWD || R > 4) ? 1 : 2)
-k_pass(const PassDesc *__restrict__ desc, int init_zero, typename V2<T>::type *__restrict__ psi,
-       typename V2<T>::type *__restrict__ lam, size_t stride, const RotCoef<T> *__restrict__ coefs,
-       size_t coef_stride, const typename V2<T>::type *__restrict__ dtab, size_t dtab_stride,
-       double *__restrict__ gpart, size_t grad_stride) {
+k_pass(const PassDesc *__restrict__ desc, int init_zero, typename V2<T>::type *psi,
+       typename V2<T>::type *lam, size_t stride, const RotCoef<T> *coefs,
+       size_t coef_stride, const typename V2<T>::type *dtab, size_t dtab_stride,
+       double *gpart, size_t grad_stride) {
     pdl_trigger();
     pdl_wait();
     using C = typename V2<T>::type;
@@ -289,10 +289,10 @@ struct FixedHead {
 template <typename T, int R, bool BWD, int... Codes>
 __global__ void __launch_bounds__(kPassMaxThreads, (BWD || R > 4) ? 1 : 2)
 k_pass_fixed(const FixedHead H, const PassDesc *__restrict__ desc, int init_zero,
-             typename V2<T>::type *__restrict__ psi, typename V2<T>::type *__restrict__ lam,
-             size_t stride, const RotCoef<T> *__restrict__ coefs, size_t coef_stride,
-             const typename V2<T>::type *__restrict__ dtab, size_t dtab_stride,
-             double *__restrict__ gpart, size_t grad_stride) {
+             typename V2<T>::type *psi, typename V2<T>::type *lam,
+             size_t stride, const RotCoef<T> *coefs, size_t coef_stride,
+             const typename V2<T>::type *dtab, size_t dtab_stride,
+             double *gpart, size_t grad_stride) {
     using C = typename V2<T>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ PassDesc sd;

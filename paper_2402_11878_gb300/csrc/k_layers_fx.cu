@@ -438,10 +438,10 @@ __device__ __forceinline__ void write_product_tile_fx(const PassDesc &d, const R
 // 24.7 ms, gradient at 13 qubits (depth 6) 706 -> 513 us.
 template <bool BWD, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB)
-k_pass_fx(const FxHead H, const PassDesc *__restrict__ desc, int init_zero, double2 *__restrict__ psi,
-          double2 *__restrict__ lam, size_t stride, const RotFx *__restrict__ coefs,
-          size_t coef_stride, const longlong2 *__restrict__ dtab, size_t dtab_stride,
-          double *__restrict__ gpart, size_t grad_stride) {
+k_pass_fx(const FxHead H, const PassDesc *__restrict__ desc, int init_zero, double2 *psi,
+          double2 *lam, size_t stride, const RotFx *coefs,
+          size_t coef_stride, const longlong2 *dtab, size_t dtab_stride,
+          double *gpart, size_t grad_stride) {
     constexpr int NB = BWD ? 2 : 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ FxShared sh;
@@ -660,7 +660,7 @@ k_pass_fx(const FxHead H, const PassDesc *__restrict__ desc, int init_zero, doub
             FxWide ua[BWD ? kNR : 1];
 #pragma unroll
             for (int r = 0; r < kNR; ++r) {
-                const longlong2 e = __ldg(tab + ((e0 ^ ((uint32_t)r << chunk)) >> t0));
+                const longlong2 e = chain_load(tab + ((e0 ^ ((uint32_t)r << chunk)) >> t0));
                 // signs by complement: one unit of 2^-63 off
                 const long long sg = -(long long)((sm >> r) & 1u);
                 const long long dre = e.x ^ sg, dim = e.y ^ sg, dng = e.y ^ ~sg;

@@ -100,9 +100,9 @@ __global__ void __launch_bounds__(kSweepThreads, sizeof(T) == 8 ? 3 : 4)
 k_apply_h_sweep(SweepDesc W, const uint32_t *__restrict__ order, const SGroup *__restrict__ groups,
                 const uint32_t *__restrict__ pat, const uint32_t *__restrict__ tz,
                 const T *__restrict__ ca, const T *__restrict__ cb, const T *__restrict__ hdiag,
-                int n, const typename SV2<T>::type *__restrict__ psi,
-                typename SV2<T>::type *__restrict__ lam, size_t stride, int first, int last,
-                int n_elec, unsigned long long *__restrict__ ctr, double *__restrict__ cpart) {
+                int n, const typename SV2<T>::type *psi,
+                typename SV2<T>::type *lam, size_t stride, int first, int last,
+                int n_elec, unsigned long long *ctr, double *cpart) {
     pdl_trigger();
     pdl_wait();
     using C = typename SV2<T>::type;
@@ -309,12 +309,17 @@ k_apply_h_sweep(SweepDesc W, const uint32_t *__restrict__ order, const SGroup *_
                     }
                 }
             }
+            C own[J];   // loaded together, before the first store
+            if (last) {
+#pragma unroll
+                for (int j = 0; j < J; ++j) own[j] = P[a[j]];
+            }
 #pragma unroll
             for (int j = 0; j < J; ++j) {
                 if (!ok[j]) continue;
                 L[a[j]] = lv[j];
                 if (last) {
-                    const C x = P[a[j]];
+                    const C x = own[j];
                     const T e = fma(x.x, lv[j].x, x.y * lv[j].y);
                     const T q = fma(x.x, x.x, x.y * x.y);
                     if constexpr (sizeof(T) == 4) {

@@ -8,6 +8,14 @@
 // and before it exits, so a kernel never completes before its predecessor; the
 // first kernel of an evaluation is launched plainly (full order after whatever
 // the stream holds).
+//
+// The data of the chain (states, staged coefficients and tables, partials) change
+// while a kernel launched early is already running.  A pointer to them is
+// therefore neither __restrict__ nor read through the read-only path (__ldg,
+// ld.global.nc): both promise data that stay the same for the kernel's lifetime,
+// so the compiler may move such a load above the wait, and the wait does not order
+// it.  Plain loads after pdl_wait(), __ldcg or chain_load() are ordered.  Tables of
+// the plan and of the Hamiltonian, which no kernel of a chain writes, may be both.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -18,6 +26,11 @@ namespace vqe {
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // Returns when the kernel before has completed and its writes are visible.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// A table that an earlier kernel of the chain staged, kept in L1.  (For the
+// diagonal tables of the ansatz passes: as fast as __ldg.)
+template <class C>
+__device__ __forceinline__ C chain_load(const C *p) { return __ldca(p); }
 
 // Where it pays, by the number of blocks (152 SMs; a gradient in us, plain
 // against early launch).  Small grids: the gaps between kernels count (14 qubits,
