@@ -396,10 +396,10 @@ template <typename T>
 cudaError_t launch_energy(const GroupDesc *groups, int n_groups, const uint32_t *tz,
                           const double *tc, const void *hdiag, int n_qubits, int batch,
                           const void *psi, size_t state_stride, double *partials, int bps,
-                          cudaStream_t s) {
+                          bool early, cudaStream_t s) {
     using C = typename EV2<T>::type;
     dim3 grid(bps, batch);
-    return pdl_launch(k_energy_cols<T>, grid, kEnergyThreads, 0, s, pdl_pays(grid), groups, n_groups, tz,
+    return pdl_launch(k_energy_cols<T>, grid, kEnergyThreads, 0, s, early && pdl_pays(grid), groups, n_groups, tz,
                                                      reinterpret_cast<const T *>(tc),
                                                      static_cast<const T *>(hdiag), n_qubits,
                                                      static_cast<const C *>(psi), state_stride,
@@ -437,10 +437,10 @@ cudaError_t launch_grad_finish(const double *part, size_t part_stride, const int
 
 template cudaError_t launch_energy<float>(const GroupDesc *, int, const uint32_t *, const double *,
                                           const void *, int, int, const void *, size_t, double *,
-                                          int, cudaStream_t);
+                                          int, bool, cudaStream_t);
 template cudaError_t launch_energy<double>(const GroupDesc *, int, const uint32_t *,
                                            const double *, const void *, int, int, const void *,
-                                           size_t, double *, int, cudaStream_t);
+                                           size_t, double *, int, bool, cudaStream_t);
 template cudaError_t launch_apply_h<float>(const GroupDesc *, int, const uint32_t *,
                                            const double *, const void *, int, int, const void *,
                                            void *, size_t, double *, int, cudaStream_t);
@@ -959,7 +959,7 @@ template <typename T>
 cudaError_t launch_energy_win(const WinDesc &W, const WinGroup *wgroups, const WinTerm *wterms,
                               const uint32_t *hoff, const void *hdiag, int n_qubits, int batch,
                               const void *psi, size_t state_stride, double *partials,
-                              int bps_total, cudaStream_t s) {
+                              int bps_total, bool early, cudaStream_t s) {
     using C = typename EV2<T>::type;
     const size_t smem = win_smem_bytes(W, sizeof(C));
     auto kern = W.any_runs
@@ -972,7 +972,7 @@ cudaError_t launch_energy_win(const WinDesc &W, const WinGroup *wgroups, const W
         if (e != cudaSuccess) return e;
     }
     dim3 grid((unsigned)(1ull << (n_qubits - W.k)), batch);
-    return pdl_launch(kern, grid, kEnergyWinThreads, smem, s, pdl_pays(grid), W, wgroups, wterms, hoff,
+    return pdl_launch(kern, grid, kEnergyWinThreads, smem, s, early && pdl_pays(grid), W, wgroups, wterms, hoff,
                                                static_cast<const T *>(hdiag),
                                                static_cast<const C *>(psi), state_stride,
                                                partials, bps_total);
@@ -1003,10 +1003,10 @@ template cudaError_t launch_apply_h_win<double>(const WinDesc &, const WinGroup 
                                                 cudaStream_t);
 template cudaError_t launch_energy_win<float>(const WinDesc &, const WinGroup *, const WinTerm *,
                                               const uint32_t *, const void *, int, int,
-                                              const void *, size_t, double *, int, cudaStream_t);
+                                              const void *, size_t, double *, int, bool, cudaStream_t);
 template cudaError_t launch_energy_win<double>(const WinDesc &, const WinGroup *, const WinTerm *,
                                                const uint32_t *, const void *, int, int,
-                                               const void *, size_t, double *, int, cudaStream_t);
+                                               const void *, size_t, double *, int, bool, cudaStream_t);
 template cudaError_t launch_energy_sub<float>(const GroupDesc *, int, const uint32_t *,
                                               const double *, int, int, const void *, size_t,
                                               double *, int, int, int, cudaStream_t);

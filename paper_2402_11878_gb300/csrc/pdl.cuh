@@ -6,8 +6,8 @@
 // Rules that keep the chain ordered: every block of a kernel launched this way
 // calls pdl_wait() before it reads or writes anything an earlier kernel touches
 // and before it exits, so a kernel never completes before its predecessor; the
-// first kernel of an evaluation is launched plainly (full order after whatever
-// the stream holds).
+// first kernel of a call is launched plainly (full order after whatever the stream
+// holds: the wait covers the kernel before, not one that this one overtook).
 //
 // The data of the chain (states, staged coefficients and tables, partials) change
 // while a kernel launched early is already running.  A pointer to them is

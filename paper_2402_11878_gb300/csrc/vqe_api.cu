@@ -1801,9 +1801,11 @@ vqe_status run_forward(vqe_ctx *h, int which, const double *params_dev, int B, v
     return VQE_OK;
 }
 
+// `chained`: follows the circuit's kernels of the same call, else its first kernel
+// is the call's first.
 template <typename T>
 vqe_status run_energy(vqe_ctx *h, int B, const void *psi, double *energies, double *norms,
-                      double *unnorm) {
+                      double *unnorm, bool chained) {
     if (!h->hd.wins.empty() && uint64_t(h->hd.win_tiles / int(h->hd.wins.size())) * B >= uint64_t(2 * h->sms)) {
         const int bps_wide = h->hd.n_wide ? blocks_per_state(h, B) : 0;
         const int bps_total = h->hd.win_tiles + bps_wide;
@@ -1816,7 +1818,8 @@ vqe_status run_energy(vqe_ctx *h, int B, const void *psi, double *energies, doub
                                              static_cast<const WinTerm *>(h->hd.d_wterms.p),
                                              static_cast<const uint32_t *>(h->hd.d_whoff.p),
                                              h->hd.hdiag(), h->n, B, psi, h->state_elems(), part,
-                                             bps_total, h->stream));
+                                             bps_total, chained, h->stream));
+            chained = true;
             h->stats.kernel_launches++;
         }
         if (h->hd.n_wide) {
@@ -1838,7 +1841,7 @@ vqe_status run_energy(vqe_ctx *h, int B, const void *psi, double *energies, doub
                                  static_cast<const uint32_t *>(h->hd.d_tz.p),
                                  static_cast<const double *>(h->hd.d_tc.p), h->hd.hdiag(), h->n, B, psi,
                                  h->state_elems(), static_cast<double *>(h->d_epart.p), bps,
-                                 h->stream));
+                                 chained, h->stream));
     prof_end(h, mk, 1);
     VQE_CUDA(h, launch_energy_finish(static_cast<double *>(h->d_epart.p), bps, B, energies, norms,
                                      unnorm, h->stream));
@@ -1850,7 +1853,7 @@ template <typename T>
 vqe_status energy_chunk(vqe_ctx *h, const double *params_dev, int B, double *E, double *nrm) {
     vqe_status st = run_forward<T>(h, 0, params_dev, B, h->ws);
     if (st != VQE_OK) return st;
-    return run_energy<T>(h, B, h->ws, E, nrm, nullptr);
+    return run_energy<T>(h, B, h->ws, E, nrm, nullptr, true);
 }
 
 // lambda = H psi for B states with the fused energy E = Re<psi|lambda>/<psi|psi>.
@@ -1979,7 +1982,7 @@ vqe_status pergate_chunk(vqe_ctx *h, const double *params_dev, int B, double *E,
             h->stats.kernel_launches++;
         }
     }
-    return run_energy<T>(h, B, h->ws, E, nrm, nullptr);
+    return run_energy<T>(h, B, h->ws, E, nrm, nullptr, true);
 }
 
 enum class Job { Energy, Gradient, PerGate };
@@ -2277,8 +2280,8 @@ vqe_status vqe_energy(vqe_handle h, double *energy, double *norm) {
     vqe_status st = ensure_scratch(h, 1);
     if (st != VQE_OK) return st;
     double *out = static_cast<double *>(h->d_out.p);
-    st = h->prec == VQE_C128 ? run_energy<double>(h, 1, h->ws, out, out + 1, nullptr)
-                             : run_energy<float>(h, 1, h->ws, out, out + 1, nullptr);
+    st = h->prec == VQE_C128 ? run_energy<double>(h, 1, h->ws, out, out + 1, nullptr, false)
+                             : run_energy<float>(h, 1, h->ws, out, out + 1, nullptr, false);
     if (st != VQE_OK) return st;
     double host[2];
     VQE_CUDA(h, cudaMemcpyAsync(host, out, sizeof(host), cudaMemcpyDeviceToHost, h->stream));

@@ -290,7 +290,8 @@ struct SGroup {
 };
 
 // ---------------------------------------------------------------- launchers
-// Each returns cudaGetLastError() after queueing.
+// Each returns cudaGetLastError() after queueing.  `early` = false: the kernel is
+// the first of its call and starts after all that the stream holds (pdl.cuh).
 
 template <typename T>
 cudaError_t launch_stage(const StageSlot *slots_dev, int n_slots, int n_qubits, int depth,
@@ -320,7 +321,7 @@ template <typename T>
 cudaError_t launch_energy(const GroupDesc *groups, int n_groups, const uint32_t *tz,
                           const double *tc, const void *hdiag, int n_qubits, int batch,
                           const void *psi, size_t state_stride, double *partials,
-                          int blocks_per_state, cudaStream_t s);
+                          int blocks_per_state, bool early, cudaStream_t s);
 
 template <typename T>
 cudaError_t launch_apply_h(const GroupDesc *groups, int n_groups, const uint32_t *tz,
@@ -332,7 +333,7 @@ template <typename T>
 cudaError_t launch_energy_win(const WinDesc &W, const WinGroup *wgroups, const WinTerm *wterms,
                               const uint32_t *hoff, const void *hdiag, int n_qubits, int batch,
                               const void *psi, size_t state_stride, double *partials,
-                              int bps_total, cudaStream_t s);
+                              int bps_total, bool early, cudaStream_t s);
 // Windowed apply-H over windows planned with each group's terms ordered by
 // their pattern over a thread's elements: `first` writes lambda, later windows
 // add to it; the `last` window writes block partials (Re<psi|lambda>, norm)

@@ -1,0 +1,70 @@
+"""What the host queues, seen through a CUDA runtime that records it (fake_cudart.cpp)."""
+import ctypes
+import glob
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+import vqe_inputs as vi
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def fake_lib(tmp_path_factory):
+    from paper_2402_11878_gb300 import build
+    objs = sorted(glob.glob(os.path.join(build.OBJ_DIR, "*.cu.o")))
+    built = build.build(force=len(objs) != len(build.sources()))
+    objs = [os.path.join(build.OBJ_DIR, os.path.basename(s) + ".o") for s in build.sources()]
+    out = str(tmp_path_factory.mktemp("fake") / "libvqe_fake.so")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build._nvcc()))), "include")
+    subprocess.run(["g++", "-shared", "-fPIC", "-O1", "-std=c++17", "-Wl,-Bsymbolic", "-I", cuda, "-o", out,
+                    os.path.join(HERE, "fake_cudart.cpp")] + objs, check=True)
+    assert built
+    return out
+
+
+@pytest.fixture
+def runtime(fake_lib, monkeypatch):
+    from paper_2402_11878_gb300 import binding
+    monkeypatch.setattr(binding, "LIB_PATH", fake_lib)
+    monkeypatch.setattr(binding, "_lib", None)
+    lib = ctypes.CDLL(fake_lib)
+    lib.fake_record.restype = ctypes.c_char_p
+
+    class Runtime:
+        engine = binding.Engine
+
+        def reset(self, static_bytes=1024):
+            lib.fake_reset(static_bytes)
+
+        def events(self, kind):
+            rows = [line.split() for line in lib.fake_record().decode().splitlines()]
+            return [r[1:] for r in rows if r[0] == kind]
+
+    r = Runtime()
+    r.reset()
+    return r
+
+
+@pytest.mark.parametrize("n", [8, 13, 22])
+@pytest.mark.parametrize("ansatz", ["hea", "pc"])
+@pytest.mark.parametrize("precision", ["c64", "c128"])
+@pytest.mark.parametrize("ham", ["chain", "random"])
+def test_the_first_kernel_of_a_call_is_launched_plainly(runtime, n, ansatz, precision, ham):
+    if ansatz == "pc":
+        eng = runtime.engine.particle_conserving(n, n // 2, vi.excitations(n, n // 2, 2, 6, seed=1), precision)
+    else:
+        eng = runtime.engine(n, 2, precision)
+    h = vi.hubbard_1d(n // 2, 1.0, 4.0) if ham == "chain" else vi.random_pauli_sum(n, 2 * n, 3)
+    eng.set_hamiltonian(h.x, h.z, h.c)
+    p = np.zeros(eng.n_params)
+    eng.apply_ansatz(p)
+    calls = [lambda: eng.apply_ansatz(p), eng.energy, lambda: eng.gradient(p), lambda: eng.energy_batch(p)]
+    for call in calls:
+        runtime.reset()
+        call()
+        kinds = [e[2] for e in runtime.events("launch")]
+        assert kinds[0] == "plain" and len(kinds) >= 2
