@@ -32,13 +32,18 @@
  *   - Energies are <psi|H|psi>/<psi|psi> (Eq. 7); gradients are of the
  *     unnormalised <psi|H|psi> (equal for the unitary circuit).
  *   - Precision: VQE_C128 keeps the state in FP64 and computes in FP64, but for
- *     the passes of the layered ansatz with reg_bits 3 (the default): these
- *     turn a tile of up to 2^12 amplitudes into 64-bit fixed point with one
- *     exponent per tile and back.  Their error is relative to the tile's norm,
- *     not to each amplitude: below that of FP64 arithmetic for states and
- *     gradients (root mean square 5.8e-16 against 8.8e-16, 1.1e-15 against
- *     2.1e-15), while an amplitude 2^-50 times smaller than its tile's norm
- *     keeps few significant bits.  VQE_C64 keeps the
+ *     the passes of the layered ansatz with reg_bits 3 (the default) where the
+ *     angles are generic.  Such a pass turns a tile of up to 2^12 amplitudes
+ *     into 64-bit fixed point with one exponent per tile and back: every
+ *     operation errs by about one unit of 2^-61 of the tile's norm, whatever the
+ *     size of the single amplitude (an FP64 operation by 2^-53 of the amplitude).
+ *     It is used, per state and pass, where no amplitude of a tile lies further
+ *     than 2^-8 below the largest by its angles: the product over the tile's
+ *     qubits of the largest |tan| over the layers of theta/2, from the nearest
+ *     multiple of pi/2, is above 2^-8.  Uniform angles are there from about six
+ *     layers on; circuits of one or two layers, or of small angles, stay in FP64
+ *     and keep every amplitude to FP64's own relative precision.  Any other
+ *     reg_bits always computes in FP64.  VQE_C64 keeps the
  *     state in complex64 and does gate arithmetic in FP32, and accumulates
  *     energies, norms and gradients in FP64.
  *
@@ -133,7 +138,8 @@ vqe_status vqe_bind_workspace(vqe_handle h, void *dev_ptr, size_t bytes);
  * Rejected (VQE_ERR_ARG) if a pass would need more than 512 threads or
  * 227 KiB of shared memory.  Rebuilds the plans; the state of
  * vqe_apply_ansatz is discarded.  Results do not depend on the plan beyond
- * floating-point rounding order. */
+ * rounding: its order, and with reg_bits 3 in C128 its unit where passes run in
+ * fixed point (see Precision above). */
 vqe_status vqe_set_plan_options(vqe_handle h, int tile_bits_max, int run_bits, int reg_bits);
 
 /* Form of lambda = H psi in gradient evaluations (the adjoint's apply-H):

@@ -25,6 +25,7 @@ template <typename T>
 struct BatchEnv {
     using C = typename V2<T>::type;
     static constexpr int kLoad = 0;
+    static constexpr bool kRows = false;
     const PassDesc *d;
     const RotCoef<T> *coef_s;   // shared: all slots of the instance (plan's coef offsets)
     const C *lo_s;              // shared: per plan slot, 2^kl low half-table entries

@@ -6,12 +6,15 @@
 // (backward) flushes runs on it.  The arithmetic is that of fx.cuh: doubles in
 // global memory, 64-bit integers in registers and shared memory.  One compiled
 // body serves every program: the 3 register bits of a round are the same code
-// wherever the round's chunk lies, only the addresses depend on it.
+// wherever the round's chunk lies, only the addresses depend on it.  A state whose
+// angles spread a tile's amplitudes too far for one exponent (kFxMaxSpread) goes
+// through the same launch in FP64 (WideEnv).
 #include <cstddef>
 
 #include "fx.cuh"
 #include "pass_core.cuh"
 #include "pdl.cuh"
+#include "stage.cuh"
 #include "vqe_internal.h"
 
 namespace vqe {
@@ -40,6 +43,40 @@ __device__ __forceinline__ long long to62(double x, double r) {
     return __double2ll_rn(x * 0x1p62) + __double2ll_rn(x * r * 0x1p62);
 }
 
+// Bits by which the amplitudes of a tile of the slot's pass spread (fx.cuh): per
+// qubit of the tile the layers' largest tangent, 16 threads each.  The same for every
+// slot of a pass, bit for bit.  A qubit that no layer turns leaves exact zeros.
+__device__ __forceinline__ float tile_spread(const StageSlot &S, int n, int depth, const double *pr) {
+    __shared__ float bits[kMaxTileBits];
+    static_assert(kMaxTileBits <= 16, "16 threads per tile bit");
+    const int j = threadIdx.x >> 4, t0 = S.tile_bit[0];   // the tile's ungated bits are qubits 0 .. t0 - 1
+    if (j < S.k) {
+        const int q = j < t0 ? j : S.qubit[j - t0];
+        double w = 0.0;
+        for (int l = threadIdx.x & 15; l < depth; l += 16) {
+            const double th = pr[((size_t)l * n + q) * 2];
+            const double turns = rint(th * 0.31830988618379067);   // 1 / pi
+            const double d = fma(-turns, 1.2246467991473532e-16, fma(-turns, 3.141592653589793, th));
+            w = fmax(w, fabs(d));   // an angle that is not a number does not count
+        }
+        float bit = w == 0.0 ? 0.f : w < 1e-30 ? 100.f : -log2f(tanf(fminf((float)(0.5 * w), 0.78539816f)));
+        const unsigned group = 0xffffu << (threadIdx.x & 16u);
+        for (int o = 8; o > 0; o >>= 1) {
+            const double ow = __shfl_xor_sync(group, w, o);
+            const float ob = __shfl_xor_sync(group, bit, o);
+            if (ow > w) {
+                w = ow;
+                bit = ob;
+            }
+        }
+        if ((threadIdx.x & 15u) == 0) bits[j] = fmaxf(bit, 0.f);
+    }
+    __syncthreads();
+    float sum = 0.f;
+    for (int i = 0; i < S.k; ++i) sum += bits[i];
+    return sum;
+}
+
 // One block per slot and state: coefficients, gradient scales and shift
 // schedule of the slot's gated bits, and the slot's diagonal table
 //   d[l] = 2^S sigma prod_j (phase and quarter-turn sign of bit j of l),
@@ -60,6 +97,11 @@ __global__ void k_stage_fx(const StageSlot *__restrict__ slots, int n, int depth
     const StageSlot S = slots[blockIdx.x];
     const int b = blockIdx.y;
     const double *pr = params + (size_t)b * (2 * (size_t)n * depth);
+    if (tile_spread(S, n, depth, pr) > kFxMaxSpread) {   // the pass stays in FP64
+        stage_slot<double>(S, n, pr, reinterpret_cast<RotWide *>(coefs + (size_t)b * coef_stride + S.coef_off),
+                           reinterpret_cast<double2 *>(dtab + (size_t)b * dtab_stride + S.dtab_off));
+        return;
+    }
     if (threadIdx.x < (unsigned)S.n_gated) {
         const int j = threadIdx.x;
         const int q = S.qubit[j];
@@ -99,7 +141,7 @@ __global__ void k_stage_fx(const StageSlot *__restrict__ slots, int n, int depth
         rot[j].tl = fx_lo(T);
         rot[j].th = fx_hi(T);
         rot[j].meta = ((turns & 1) ? kFxFlip : 0u) | (half_turn ? kFx45 : 0u) | (bad ? kFxBad : 0u);
-        rot[j].spare = 0;
+        rot[j].wide = 0;
         double sp, cp;
         sincos(0.5 * phi, &sp, &cp);
         const double c2 = cp * cp, c2e = fma(cp, cp, -c2), s2 = sp * sp, s2e = fma(sp, sp, -s2);
@@ -426,6 +468,38 @@ __device__ __forceinline__ void write_product_tile_fx(const PassDesc &d, const R
     }
 }
 
+// A pass in FP64, for run_tile: bound by the FP64 pipe.  24 qubits, depth 8, energy /
+// gradient: normal angles of deviation 0.1 in FP64 13.4 / 54.5 ms (54.5 with a row of
+// partials per bit, 61.9 with a warp sum per gate), uniform angles in fixed point 6.7
+// / 22.5.  Asking which it is costs the fixed-point passes 0.7 % forward (20 qubits,
+// 64 energies: 24.51 -> 24.71 ms) and nothing backward (28 qubits: 394.4 -> 394.2).
+struct WideEnv {
+    using C = double2;
+    static constexpr int kLoad = 1;
+    static constexpr bool kRows = true;
+    const PassDesc *d;
+    const RotWide *cf;
+    const double2 *dt;
+    double *gout;
+    uint64_t gslot;
+    double2 *P, *L;
+    int init_zero;
+    int t0;
+    __device__ RotCoef<double> coef(int slot, int bit) const {
+        const RotWide &r = cf[slot * d->k + bit];
+        return RotCoef<double>{r.v, r.gs, r.mode};
+    }
+    __device__ C diag(int slot, uint32_t e) const { return chain_load(dt + d->slot_dtab_off[slot] + (e >> t0)); }
+    __device__ void grad(int slot, int bit, int comp, double v) const { gout[slot * gslot + bit * 2 + comp] = v; }
+};
+
+// Forward inlined, backward called: neither then takes registers from the
+// fixed-point path (a call reserves some, which the forward's 64 cannot spare).
+__device__ __noinline__ void wide_backward(const PassDesc &d, int n_ops, uint64_t base, double2 *buf, double *gsh,
+                                           uint32_t size, WideEnv &env) {
+    run_tile<double, kR, true>(d, d.ops, n_ops, base, buf, buf + size, gsh, env);
+}
+
 // One CTA per (tile, state).  A tile's phases (load, conversion, diagonal,
 // gates, exchanges, store) use different pipes, so what counts beside the
 // instructions (backward 760, forward 330 per amplitude in a slot of 7 gates) is
@@ -526,9 +600,10 @@ k_pass_fx(const FxHead H, const PassDesc *__restrict__ desc, int init_zero, doub
         }
     }
     const PassDesc &d = sh.d;
-    int any_bad = 0;
+    int any_bad = 0, wide = 0;
     {
         const RotFx *src = coefs + (size_t)b * coef_stride + H.coef0;
+        if constexpr (!BWD) wide = chain_load(&src[t0].wide);   // (backward has no register to spare)
         for (int i = t; i < H.n_slots * k; i += blockDim.x) {
             const RotFx c = src[i];
             scf[i] = c;
@@ -536,6 +611,14 @@ k_pass_fx(const FxHead H, const PassDesc *__restrict__ desc, int init_zero, doub
         }
     }
     any_bad = __syncthreads_or(any_bad);
+    if (BWD ? scf[t0].wide : wide) {   // block-uniform
+        WideEnv env{&d, reinterpret_cast<const RotWide *>(scf), reinterpret_cast<const double2 *>(dt), gout, gslot,
+                    P, L, init_zero, t0};
+        double2 *buf = reinterpret_cast<double2 *>(sbuf);
+        if constexpr (BWD) wide_backward(d, H.n_ops, base, buf, reinterpret_cast<double *>(rows), size, env);
+        else run_tile<double, kR, false>(d, d.ops, H.n_ops, base, buf, nullptr, nullptr, env);
+        return;
+    }
     for (int s = t; s < H.n_slots; s += blockDim.x) {
         uint32_t f = 0u;
         for (int j = t0; j < k; ++j)

@@ -20,6 +20,9 @@
 //        1 = the state in global memory (members P, L and init_zero: start from
 //        |0...0>), 0 = that where the member `direct` is set, else `buf`/`lbuf`
 //        in plain order; the last round writes to the same place
+//   static constexpr bool kRows   (backward) gradient partials of a slot: one row per
+//        bit and thread in the scratch (nthr * (k + 1 + R) values), summed at the
+//        flush, instead of a sum over the warp at every gate
 #pragma once
 
 #include <type_traits>
@@ -191,7 +194,7 @@ __device__ __forceinline__ void run_tile(const PassDesc &d, const PassOp *ops, i
     bool direct = true;
     if constexpr (Env::kLoad == 0) direct = env.direct;
 
-    int chunk = -1;
+    int chunk = -1, diag_chunk = 0;
     bool first_exchange = true;
     for (int oi = 0; oi < n_ops; ++oi) {
         const PassOp op = ops[oi];
@@ -263,18 +266,19 @@ __device__ __forceinline__ void run_tile(const PassDesc &d, const PassOp *ops, i
                             gt = fma(-l0.x, p1.x, gt);
                             gt = fma(-l0.y, p1.y, gt);
                         }
-                        // warp sum: FP64, or compensated FP32 pairs (FP64 adds
-                        // are scarce on this GPU), then FP64 per warp
-                        double dgt;
-                        if constexpr (sizeof(T) == 4) {
-                            dgt = f32c_value(f32c_warp_sum(F32c{gt * rc.gs, 0.f}, wmask, wlanes));
+                        if constexpr (Env::kRows) {
+                            reinterpret_cast<T *>(gsh)[(chunk + j) * nthr + t] = gt;   // gs at the flush
+                        } else if constexpr (sizeof(T) == 4) {
+                            // warp sum in compensated FP32 pairs (FP64 adds are
+                            // scarce on this GPU), then FP64 per warp
+                            const double dgt = f32c_value(f32c_warp_sum(F32c{gt * rc.gs, 0.f}, wmask, wlanes));
+                            if (lane == 0) gsh[(warp * k + chunk + j) * 2 + 0] = dgt;
                         } else {
                             T wgt = gt * rc.gs;
                             for (int o = wlanes >> 1; o > 0; o >>= 1)
                                 wgt += __shfl_xor_sync(wmask, wgt, o);
-                            dgt = (double)wgt;
+                            if (lane == 0) gsh[(warp * k + chunk + j) * 2 + 0] = (double)wgt;
                         }
-                        if (lane == 0) gsh[(warp * k + chunk + j) * 2 + 0] = dgt;
                     }
                 }
                 if (!active) continue;
@@ -363,32 +367,50 @@ __device__ __forceinline__ void run_tile(const PassDesc &d, const PassOp *ops, i
                 // for every gated bit q of the slot, taken before the diagonal is
                 // undone (where the buffers hold the exact states).
                 T u[NR];
-                T tot = T(0);
 #pragma unroll
-                for (int r = 0; r < NR; ++r) {
-                    u[r] = fma(w[r].x, v[r].y, -w[r].y * v[r].x);
-                    tot += u[r];
-                }
-                const uint32_t gated = d.slot_gated[op.slot];
-                const uint32_t e0 = elem_of(t, 0, chunk, R);
-                for (int q = 0; q < k; ++q) {
-                    if (!((gated >> q) & 1u)) continue;
-                    T gq;
-                    if (q >= chunk && q < chunk + R) {
-                        gq = T(0);
+                for (int r = 0; r < NR; ++r) u[r] = fma(w[r].x, v[r].y, -w[r].y * v[r].x);
+                if constexpr (Env::kRows) {
+                    // the thread's total (row k) and its signed sums over the chunk's
+                    // bits (rows k + 1 + j), in one butterfly
+                    T *rows = reinterpret_cast<T *>(gsh);
+                    diag_chunk = chunk;
 #pragma unroll
-                        for (int r = 0; r < NR; ++r) gq += ((r >> (q - chunk)) & 1) ? -u[r] : u[r];
-                    } else {
-                        gq = ((e0 >> q) & 1u) ? -tot : tot;
+                    for (int j = 0; j < R; ++j) {
+                        T dsum = T(0);
+#pragma unroll
+                        for (int c = 0; c < (NR >> (j + 1)); ++c) {
+                            const T x0 = u[2 * c], x1 = u[2 * c + 1];
+                            dsum += x0 - x1;
+                            u[c] = x0 + x1;
+                        }
+                        rows[(k + 1 + j) * nthr + t] = dsum;
                     }
-                    double dg;
-                    if constexpr (sizeof(T) == 4) {
-                        dg = f32c_value(f32c_warp_sum(F32c{gq, 0.f}, wmask, wlanes));
-                    } else {
-                        for (int o = wlanes >> 1; o > 0; o >>= 1) gq += __shfl_xor_sync(wmask, gq, o);
-                        dg = (double)gq;
+                    rows[k * nthr + t] = u[0];
+                } else {
+                    T tot = T(0);
+#pragma unroll
+                    for (int r = 0; r < NR; ++r) tot += u[r];
+                    const uint32_t gated = d.slot_gated[op.slot];
+                    const uint32_t e0 = elem_of(t, 0, chunk, R);
+                    for (int q = 0; q < k; ++q) {
+                        if (!((gated >> q) & 1u)) continue;
+                        T gq;
+                        if (q >= chunk && q < chunk + R) {
+                            gq = T(0);
+#pragma unroll
+                            for (int r = 0; r < NR; ++r) gq += ((r >> (q - chunk)) & 1) ? -u[r] : u[r];
+                        } else {
+                            gq = ((e0 >> q) & 1u) ? -tot : tot;
+                        }
+                        double dg;
+                        if constexpr (sizeof(T) == 4) {
+                            dg = f32c_value(f32c_warp_sum(F32c{gq, 0.f}, wmask, wlanes));
+                        } else {
+                            for (int o = wlanes >> 1; o > 0; o >>= 1) gq += __shfl_xor_sync(wmask, gq, o);
+                            dg = (double)gq;
+                        }
+                        if (lane == 0) gsh[(warp * k + q) * 2 + 1] = dg;
                     }
-                    if (lane == 0) gsh[(warp * k + q) * 2 + 1] = dg;
                 }
             }
             if (active) {
@@ -453,13 +475,30 @@ __device__ __forceinline__ void run_tile(const PassDesc &d, const PassOp *ops, i
             __syncthreads();
             const uint32_t gated = d.slot_gated[op.slot];
             const int used_warps = (int)((nthr + 31) >> 5);
-            // one thread per total, the warps in order (one thread for all of them
-            // kept the block waiting for 2 k times the warps dependent FP64 adds)
-            for (int idx = threadIdx.x; idx < 2 * k; idx += blockDim.x) {
-                if (!((gated >> (idx >> 1)) & 1u)) continue;
-                double s = 0.0;
-                for (int wi = 0; wi < used_warps; ++wi) s += gsh[wi * 2 * k + idx];
-                env.grad(op.slot, idx >> 1, idx & 1, s);
+            if constexpr (Env::kRows) {
+                // a warp per row; phi of a bit outside the chunk: the total row with
+                // the sign of the thread's element
+                for (int idx = warp; idx < 2 * k; idx += nwarps) {
+                    const int q = idx >> 1, dp = diag_chunk;
+                    if (!((gated >> q) & 1u)) continue;
+                    const bool theta = (idx & 1) == 0, in_chunk = q >= dp && q < dp + R;
+                    const T *src = reinterpret_cast<const T *>(gsh) +
+                                   (theta ? q : in_chunk ? k + 1 + q - dp : k) * nthr;
+                    T sum = T(0);
+                    for (uint32_t tt = lane; tt < nthr; tt += 32)
+                        sum += !theta && !in_chunk ? flip_sign(src[tt], (elem_of(tt, 0, dp, R) >> q) & 1u) : src[tt];
+                    for (int o = wlanes >> 1; o > 0; o >>= 1) sum += __shfl_xor_sync(wmask, sum, o);
+                    if (lane == 0) env.grad(op.slot, q, idx & 1, theta ? sum * env.coef(op.slot, q).gs : sum);
+                }
+            } else {
+                // one thread per total, the warps in order (one thread for all of them
+                // kept the block waiting for 2 k times the warps dependent FP64 adds)
+                for (int idx = threadIdx.x; idx < 2 * k; idx += blockDim.x) {
+                    if (!((gated >> (idx >> 1)) & 1u)) continue;
+                    double s = 0.0;
+                    for (int wi = 0; wi < used_warps; ++wi) s += gsh[wi * 2 * k + idx];
+                    env.grad(op.slot, idx >> 1, idx & 1, s);
+                }
             }
             __syncthreads();
         }

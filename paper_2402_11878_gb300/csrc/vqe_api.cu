@@ -119,7 +119,7 @@ struct vqe_ctx {
         std::vector<PassDesc> fwd, bwd;
         DevBuf d_fwd, d_bwd, d_stage, d_goff, d_gcnt, d_gstep;
         int n_stage = 0;
-        bool fx = false;   // FP64 passes in block fixed point (k_layers_fx.cu)
+        bool fx = false;   // FP64 passes that may run in block fixed point (k_layers_fx.cu)
         size_t coef_stride = 0, dtab_stride = 0, grad_stride = 0;
         void release() {
             for (DevBuf *b : {&d_fwd, &d_bwd, &d_stage, &d_goff, &d_gcnt, &d_gstep}) b->release();
