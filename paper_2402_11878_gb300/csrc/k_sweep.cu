@@ -363,7 +363,7 @@ int sweep_blocks_per_sm(int elem_bytes, size_t smem, bool sector) {
         ? (sector ? (const void *)k_apply_h_sweep<double, true> : (const void *)k_apply_h_sweep<double, false>)
         : (sector ? (const void *)k_apply_h_sweep<float, true> : (const void *)k_apply_h_sweep<float, false>);
     int occ = 0;
-    if (smem > 48 * 1024) {
+    if (smem > 40 * 1024) {   // with the static part beyond the default 48 KiB
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) {
             cudaGetLastError();
@@ -390,7 +390,7 @@ cudaError_t launch_apply_h_sweep(const SweepDesc &W, const uint32_t *order, cons
         return cudaErrorInvalidValue;
     const size_t smem = sweep_smem_bytes(W, sizeof(T));
     auto kern = n_elec >= 0 ? k_apply_h_sweep<T, true> : k_apply_h_sweep<T, false>;
-    if (smem > 48 * 1024) {
+    if (smem > 40 * 1024) {   // with the static part beyond the default 48 KiB
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }

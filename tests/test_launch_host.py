@@ -68,3 +68,22 @@ def test_the_first_kernel_of_a_call_is_launched_plainly(runtime, n, ansatz, prec
         call()
         kinds = [e[2] for e in runtime.events("launch")]
         assert kinds[0] == "plain" and len(kinds) >= 2
+
+
+def _one_wide_group(n, n_terms):
+    """One X mask of six bits, which the sweeps keep term by term: 20 bytes of
+    tables per FP64 term and 4132 beside them."""
+    z = np.arange(n_terms, dtype=np.uint64) << np.uint64(6)     # no Y: every term real
+    return np.full(n_terms, 0b111111, dtype=np.uint64), z, np.linspace(0.1, 1.0, n_terms)
+
+
+@pytest.mark.parametrize("n_terms", [2244, 2245, 2251, 2252])
+def test_sweep_tables_about_48_kib(runtime, n_terms):
+    """48 KiB hold the tables and the kernel's static 136 bytes, not the tables alone."""
+    eng = runtime.engine(18, 1, "c128")
+    eng.set_hamiltonian(*_one_wide_group(18, n_terms))
+    assert eng.set_apply_mode(2) == 2
+    runtime.reset(static_bytes=136)
+    eng.gradient(np.zeros(eng.n_params))
+    sizes = [int(e[1]) for e in runtime.events("launch") if "k_apply_h_sweep" in e[0]]
+    assert sizes == [4132 + 20 * n_terms]
