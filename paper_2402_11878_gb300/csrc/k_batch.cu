@@ -16,6 +16,7 @@
 // of 20.8.
 #include "batch_internal.h"
 #include "pass_core.cuh"
+#include "smem_limit.h"
 
 namespace vqe {
 
@@ -296,8 +297,7 @@ cudaError_t launch_batch(const BatchArgs &args, bool r4, int grid, size_t smem, 
     } else if (r4) {
         return cudaErrorInvalidValue;   // FP64 plans keep R <= 3 (tiles of at most 2^12)
     }
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
+    if (const cudaError_t e = allow_smem((const void *)kern, smem); e != cudaSuccess) return e;
     kern<<<grid, kBatchThreads, smem, s>>>(args);
     return cudaGetLastError();
 }

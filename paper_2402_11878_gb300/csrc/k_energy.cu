@@ -16,6 +16,7 @@
 
 #include "csum.cuh"
 #include "pdl.cuh"
+#include "smem_limit.h"
 #include "vqe_internal.h"
 
 namespace vqe {
@@ -944,10 +945,7 @@ cudaError_t launch_apply_h_win(const WinDesc &W, const WinGroup *wgroups, const 
         : (W.k == 13 ? k_apply_h_win<T, 13, false> : (W.k == 12 ? k_apply_h_win<T, 12, false> : nullptr));
     if (!kern || W.t_count > kWinMaxTerms || W.g_end - W.g_begin > kWinMaxGroups)
         return cudaErrorInvalidValue;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem((const void *)kern, smem); e != cudaSuccess) return e;
     dim3 grid((unsigned)(1ull << (n_qubits - W.k)), batch);
     return pdl_launch(kern, grid, kEnergyWinThreads, smem, s, pdl_pays(grid), W, wgroups, wterms, hoff, static_cast<const T *>(hdiag),
                                                static_cast<const C *>(psi), static_cast<C *>(lam),
@@ -967,10 +965,7 @@ cudaError_t launch_energy_win(const WinDesc &W, const WinGroup *wgroups, const W
         : (W.k == 13 ? k_energy_win<T, 13, false> : (W.k == 12 ? k_energy_win<T, 12, false> : nullptr));
     if (!kern || W.t_count > kWinMaxTerms || W.g_end - W.g_begin > kWinMaxGroups)
         return cudaErrorInvalidValue;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem((const void *)kern, smem); e != cudaSuccess) return e;
     dim3 grid((unsigned)(1ull << (n_qubits - W.k)), batch);
     return pdl_launch(kern, grid, kEnergyWinThreads, smem, s, early && pdl_pays(grid), W, wgroups, wterms, hoff,
                                                static_cast<const T *>(hdiag),

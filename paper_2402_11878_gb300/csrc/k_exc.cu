@@ -50,6 +50,7 @@
 #include "csum.cuh"
 #include "pdl.cuh"
 #include "sector.cuh"
+#include "smem_limit.h"
 #include "vqe_internal.h"
 
 namespace vqe {
@@ -389,10 +390,7 @@ cudaError_t launch_exc_pass(const ExcPass &P, const ExcGate *gates_dev, const ui
     const size_t smem = room * sizeof(C) * (backward ? 2 : 1) +
                         P.n_gates * ((backward ? th * row : 0) + span * sizeof(uint32_t));
     auto launch = [&](auto kern) {
-        if (smem > 40 * 1024) {   // with the static part beyond the default 48 KiB
-            cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
+        if (const cudaError_t e = allow_smem((const void *)kern, smem); e != cudaSuccess) return e;
         return pdl_launch(kern, grid, th, smem, s, true, P, gates_dev, hoff_dev, static_cast<C *>(psi),
                           static_cast<C *>(lam), state_stride, cs, n_exc, gpart, grad_stride, init_hf, hf_index,
                           spin, room, span);

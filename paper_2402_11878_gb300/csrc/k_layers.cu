@@ -22,6 +22,7 @@
 
 #include "pass_core.cuh"
 #include "pdl.cuh"
+#include "smem_limit.h"
 #include "stage.cuh"
 
 namespace vqe {
@@ -292,10 +293,7 @@ cudaError_t launch_fixed(const PassDesc *desc_dev, const PassDesc &dh, int n_qub
     size_t smem = pass_smem_bytes(dh, BWD, sizeof(C));
     if (BWD) smem += fixed_grad_scratch_bytes<T, R>(threads, dh.k) - tile_grad_scratch_bytes(threads, dh.k);
     auto kern = k_pass_fixed<T, R, BWD, Codes...>;
-    if (smem > 40 * 1024) {   // with the static part beyond the default 48 KiB
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem((const void *)kern, smem); e != cudaSuccess) return e;
     dim3 grid((unsigned)(1ull << (n_qubits - dh.k)), batch);
     const FixedHead head{dh.m, dh.a, dh.n_ops, dh.n_slots, dh.zmask, dh.slot_gated[0], dh.slot_coef_off[0]};
     return pdl_launch(kern, grid, threads, smem, s, pdl_pays(grid), head, desc_dev, init_zero, static_cast<C *>(psi),
@@ -390,11 +388,7 @@ static cudaError_t launch_pass_r(const PassDesc *desc_dev, const PassDesc &dh, i
     if (threads > kPassMaxThreads) return cudaErrorInvalidConfiguration;
     const size_t smem = pass_smem_bytes(dh, BWD, sizeof(C));
     auto kern = k_pass<T, R, BWD>;
-    if (smem > 40 * 1024) {   // with the static part beyond the default 48 KiB
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem((const void *)kern, smem); e != cudaSuccess) return e;
     dim3 grid((unsigned)(1ull << (n_qubits - dh.k)), batch);
     return pdl_launch(kern, grid, threads, smem, s, pdl_pays(grid), desc_dev, init_zero, static_cast<C *>(psi),
                                      static_cast<C *>(lam), stride, coefs, coef_stride,

@@ -14,6 +14,7 @@
 #include "fx.cuh"
 #include "pass_core.cuh"
 #include "pdl.cuh"
+#include "smem_limit.h"
 #include "stage.cuh"
 #include "vqe_internal.h"
 
@@ -895,10 +896,7 @@ cudaError_t launch_k(const PassDesc *desc_dev, const PassDesc &dh, int n_qubits,
                   size_t(dh.n_slots) * dh.k * sizeof(RotFx);
     if (BWD) smem += size_t(threads) * (dh.k + 1 + kR) * sizeof(long long);
     auto kern = k_pass_fx<BWD, MAXT, MINB>;
-    if (smem > 40 * 1024) {   // with the static part beyond the default 48 KiB
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem((const void *)kern, smem); e != cudaSuccess) return e;
     dim3 grid((unsigned)(1ull << (n_qubits - dh.k)), batch);
     const FxHead head{dh.k, dh.m, dh.a, dh.n_ops, dh.n_slots, dh.ops[0].chunk, dh.zmask,
                       dh.slot_gated[0], dh.slot_coef_off[0], dh.slot_grad_off[0]};

@@ -19,6 +19,7 @@
 #include "csum.cuh"
 #include "pdl.cuh"
 #include "sector.cuh"
+#include "smem_limit.h"
 #include "vqe_internal.h"
 
 namespace vqe {
@@ -363,12 +364,9 @@ int sweep_blocks_per_sm(int elem_bytes, size_t smem, bool sector) {
         ? (sector ? (const void *)k_apply_h_sweep<double, true> : (const void *)k_apply_h_sweep<double, false>)
         : (sector ? (const void *)k_apply_h_sweep<float, true> : (const void *)k_apply_h_sweep<float, false>);
     int occ = 0;
-    if (smem > 40 * 1024) {   // with the static part beyond the default 48 KiB
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) {
-            cudaGetLastError();
-            return 1;
-        }
+    if (allow_smem(kern, smem) != cudaSuccess) {
+        cudaGetLastError();
+        return 1;
     }
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, kSweepThreads, smem);
     if (e != cudaSuccess) {
@@ -390,10 +388,7 @@ cudaError_t launch_apply_h_sweep(const SweepDesc &W, const uint32_t *order, cons
         return cudaErrorInvalidValue;
     const size_t smem = sweep_smem_bytes(W, sizeof(T));
     auto kern = n_elec >= 0 ? k_apply_h_sweep<T, true> : k_apply_h_sweep<T, false>;
-    if (smem > 40 * 1024) {   // with the static part beyond the default 48 KiB
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    if (const cudaError_t e = allow_smem((const void *)kern, smem); e != cudaSuccess) return e;
     dim3 grid((unsigned)blocks, batch);
     return pdl_launch(kern, grid, kSweepThreads, smem, s, pdl_pays(grid), W, order, groups, pat, tz, static_cast<const T *>(ca),
                                            static_cast<const T *>(cb), static_cast<const T *>(hdiag),

@@ -87,3 +87,33 @@ def test_sweep_tables_about_48_kib(runtime, n_terms):
     eng.gradient(np.zeros(eng.n_params))
     sizes = [int(e[1]) for e in runtime.events("launch") if "k_apply_h_sweep" in e[0]]
     assert sizes == [4132 + 20 * n_terms]
+
+
+def test_a_smaller_launch_never_lowers_a_kernels_limit(runtime):
+    """The limit belongs to the process: a thread that lowers it to its own launch's
+    size refuses the larger launch another thread is about to make."""
+    def pc(n, count, precision):
+        return runtime.engine.particle_conserving(n, n // 2, vi.excitations(n, n // 2, count // 7, count, seed=1),
+                                                  precision)
+
+    def hea(n, depth, precision, *options):
+        eng = runtime.engine(n, depth, precision)
+        if options:
+            eng.set_plan_options(*options)
+        return eng
+
+    runtime.reset()
+    for make in (lambda: hea(14, 24, "c128"), lambda: hea(14, 2, "c128"), lambda: hea(14, 3, "c64", 13, 3, 4),
+                 lambda: hea(14, 3, "c64", 12, 3, 3), lambda: hea(14, 3, "c64"), lambda: hea(14, 2, "c128", 12, 2, 4),
+                 lambda: hea(14, 2, "c128", 11, 2, 2), lambda: hea(14, 12, "c128", 12, 2, 3),
+                 lambda: hea(14, 2, "c128", 12, 2, 3), lambda: pc(14, 60, "c128"), lambda: pc(16, 8, "c128"),
+                 lambda: pc(14, 60, "c64"), lambda: pc(16, 8, "c64")):
+        eng = make()
+        h = vi.hubbard_1d(eng.n // 2, 1.0, 4.0)
+        eng.set_hamiltonian(h.x, h.z, h.c)
+        eng.gradient(np.zeros(eng.n_params))
+    limits = {}
+    for name, value in runtime.events("limit"):
+        limits.setdefault(name, set()).add(int(value))
+    assert len(limits) >= 6
+    assert {n: v for n, v in limits.items() if len(v) > 1} == {}
