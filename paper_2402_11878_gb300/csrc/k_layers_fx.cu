@@ -886,6 +886,15 @@ k_pass_fx(const FxHead H, const PassDesc *__restrict__ desc, int init_zero, doub
     }
 }
 
+// What vqe_set_plan_options accepts by the tile buffers alone fits with the rows, the
+// coefficients and the static part: the largest plan is 2^12 amplitudes, 512 threads.
+constexpr int kFxMaxTileBits = kR + 9;
+static_assert(2 * tile_buf_elems(kFxMaxTileBits, 16) * 16 +
+                      (1u << (kFxMaxTileBits - kR)) * (kFxMaxTileBits + 1 + kR) * sizeof(long long) +
+                      kMaxSlots * kFxMaxTileBits * sizeof(RotFx) + sizeof(FxShared) <=
+                  227 * 1024,
+              "the largest fixed-point plan fits the shared memory of a block");
+
 template <bool BWD, int MAXT, int MINB>
 cudaError_t launch_k(const PassDesc *desc_dev, const PassDesc &dh, int n_qubits, int batch, void *psi,
                      void *lam, size_t stride, const RotFx *coefs, size_t coef_stride,
