@@ -809,8 +809,9 @@ __device__ __forceinline__ void run_tile_fixed(const PassDesc &d, const PassOp *
             if constexpr (BWD) {
                 using A = F32c;   // compensated FP32 pairs
                 // stage-2 partials go to the psi tile buffer, free between rounds
-                // (the tile is in registers; the next round exchange starts
-                // with a barrier): 2 KT rows of 33
+                // (the tile is in registers): 2 KT rows of 33.  The next exchange
+                // writes that buffer without a barrier before it: the barrier at
+                // the end of the flush is what keeps warp 0's reads ahead of it
                 static_assert(2 * KT * 33 * sizeof(A) <= (1u << KT) * sizeof(typename V2<T>::type),
                               "partials fit the tile buffer");
                 const PassOp op = ops[i];
@@ -858,7 +859,7 @@ __device__ __forceinline__ void run_tile_fixed(const PassDesc &d, const PassOp *
                         env.grad(op.slot, q, comp, f32c_value(tot));
                     }
                 }
-                __syncthreads();
+                __syncthreads();   // required: see above
             }
         }
     });
