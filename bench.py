@@ -127,6 +127,15 @@ def pass_bytes(n: int, depth: int, prec: str):
     return float(fwd), float(bwd)
 
 
+def excitation_pass_bytes(n: int, n_elec: int, n_pass: int, amp_bytes: float):
+    """HBM bytes that bound the excitation ansatz's forward and backward passes from
+    above: the amplitudes that can differ from zero (both spins' electrons are kept),
+    once read and written per pass and buffer, though a pass moves only those that its
+    gates pair; the first forward pass reads nothing and writes the whole state."""
+    sector = amp_bytes * math.comb(n // 2, n_elec // 2) ** 2
+    return amp_bytes * 2.0 ** n + (n_pass - 1) * 2 * sector, n_pass * 4 * sector
+
+
 def oracle_sweeps(n: int, depth: int, n_terms: int) -> int:
     """State sweeps of one oracle energy + adjoint gradient: the gate-by-gate
     forward (2n rotations and n-1 CZ per layer), the per-term lambda = H psi,
@@ -749,18 +758,14 @@ def run_workload(name: str, args):
             npass = eng.stats()["ansatz_passes"]
             f_ms = pr["forward_passes"]["ms"] / reps
             b_ms = pr["backward_passes"]["ms"] / reps
-            # amplitudes that can differ from zero (both spins' electrons are
-            # kept), once read and written per pass and buffer: an upper bound
-            # of what the passes need, which move only what their gates pair
-            sector = st * math.comb(n // 2, ne // 2) ** 2
-            by_f, by_b = npass * 2 * sector, npass * 4 * sector
+            by_f, by_b = excitation_pass_bytes(n, ne, npass, st)
             out[prec] = {"evals_per_s": 1e3 / ms, "ms_per_eval": ms, "energy": float(E[0]),
                          "passes": npass, "apply_form": tune["apply_form"],
                          "forward_ms": f_ms, "apply_h_ms": pr["apply_h"]["ms"] / reps,
                          "backward_ms": b_ms,
-                         "forward_sector_gbs": by_f / (f_ms / 1e3) / 1e9,
+                         "forward_pass_gbs": by_f / (f_ms / 1e3) / 1e9,
                          "backward_sector_gbs": by_b / (b_ms / 1e3) / 1e9,
-                         "sector_fraction": sector / (st * float(1 << n)),
+                         "sector_fraction": math.comb(n // 2, ne // 2) ** 2 / float(1 << n),
                          "grad_inf": float(G.abs().max())}
             g = G[0].cpu().numpy().copy()
             if prec == "c128":
