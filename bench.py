@@ -47,6 +47,9 @@ WORKLOAD = ("32q FP64 (complex128) 4x4 periodic 2D Fermi-Hubbard (snake order, t
 # the reference arm; each is extrapolated to 32 qubits (see oracle_scale).
 SAMPLE_CPU = (4, 3)
 SAMPLE_REFERENCE = (5, 2)
+# 64-bit fixed-point multiply-adds of the backward passes: 15 clocks each per warp and
+# scheduler, measured with independent chains (7 instructions; csrc/fx.cuh)
+FIXED_POINT_PEAK = 152 * 4 * (32 / 15) * 2 * 2.070e9 / 1e12   # SMs x schedulers x lanes/clk x 2 flop x max clock
 FP64_UNITS_PEAK = 152 * 2 * 2 * 2.070e9 / 1e12   # SMs x DFMA/clk/SM x 2 flop x max SM clock
 # DRAM read + write bytes of the FP64 backward pass kernel per byte it must
 # move (psi and lambda read and written per live tile), from an ncu capture
@@ -464,17 +467,22 @@ def run_gpu(args, world, rank, local, pg):
                             "tflops": fl_b / (bwd_ms / 1e3) / 1e12,
                             "hbm_gbs": by_b / (bwd_ms / 1e3) / 1e9},
     }
-    # The backward passes run in 64-bit fixed point: bound by the issue of
-    # integer instructions, so their fraction is given of the memory's rate; the
-    # FP64 multiply-add rate, which the same work in FP64 cannot exceed, beside it.
-    achieved = by_b / (bwd_ms / 1e3) / 1e9
-    roofline = {"bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
-                "frac": achieved / hbm_peak if hbm_peak else None,
+    # The backward passes run in 64-bit fixed point and are bound by the issue of
+    # integer instructions: their fraction is of the measured rate of the
+    # multiply-adds they are made of.  The FP64 multiply-add rate, which the same work
+    # in FP64 cannot exceed, and the memory's rate stand beside it.
+    achieved = fl_b / (bwd_ms / 1e3) / 1e12
+    hbm = by_b / (bwd_ms / 1e3) / 1e9
+    roofline = {"bound": "alu", "achieved": achieved, "peak": FIXED_POINT_PEAK, "unit": "TFLOP/s",
+                "frac": achieved / FIXED_POINT_PEAK,
+                "hbm_gbs": hbm, "hbm_peak_gbs": hbm_peak, "hbm_frac": hbm / hbm_peak if hbm_peak else None,
                 "traffic": (by_b / bwd_launches * BWD_TRAFFIC_PER_ALGORITHMIC_BYTE
                             if BWD_TRAFFIC_PER_ALGORITHMIC_BYTE else None),
                 "kernel": "k_pass_fx<bwd> (adjoint backward tile passes, 64-bit block fixed point)",
-                "peak_source": "measured HBM copy bandwidth",
-                "algorithmic_tflops": fl_b / (bwd_ms / 1e3) / 1e12, "fp64_fma_peak_tflops": fp64_peak,
+                "peak_source": "64-bit fixed-point multiply-adds, 15 clocks per warp and scheduler (measured), "
+                               "at the maximum clock",
+                "hbm_peak_source": "measured HBM copy bandwidth",
+                "fp64_fma_peak_tflops": fp64_peak,
                 "fp64_fma_peak_source": ("measured FP64 FMA rate of this GPU (vqe_measure_fma_peak, "
                                          "independent FMA chains on every SM, CUDA events); unit count x "
                                          f"max clock gives {FP64_UNITS_PEAK:.4g}"),
@@ -764,7 +772,7 @@ def run_workload(name: str, args):
                          "forward_ms": f_ms, "apply_h_ms": pr["apply_h"]["ms"] / reps,
                          "backward_ms": b_ms,
                          "forward_pass_gbs": by_f / (f_ms / 1e3) / 1e9,
-                         "backward_sector_gbs": by_b / (b_ms / 1e3) / 1e9,
+                         "backward_pass_gbs": by_b / (b_ms / 1e3) / 1e9,
                          "sector_fraction": math.comb(n // 2, ne // 2) ** 2 / float(1 << n),
                          "grad_inf": float(G.abs().max())}
             g = G[0].cpu().numpy().copy()
