@@ -57,7 +57,7 @@ FP64_UNITS_PEAK = 152 * 2 * 2 * 2.070e9 / 1e12   # SMs x DFMA/clk/SM x 2 flop x 
 # read + write: 3.049 GB against 3.221 GB); the per-tile traffic of these
 # passes does not depend on the qubit count.  None once the kernel changes,
 # until it is captured again.
-BWD_TRAFFIC_PER_ALGORITHMIC_BYTE = 3049170432 / 3221225472
+BWD_TRAFFIC_PER_ALGORITHMIC_BYTE = 3049310464 / 3221225472
 
 
 # ---------------------------------------------------------------- work models
@@ -848,7 +848,8 @@ def run_case(name: str, batch: int):
         "fwd24c64": (24, 4, "c64", False, "chain"), "grad24c64": (24, 4, "c64", True, "chain"),
         "fwd26c64": (26, 4, "c64", False, "chain"),
         "mol24c64": (24, 2, "c64", True, "mol"),     # synthetic molecular Hamiltonian, 12 orbitals
-        "lat24c128": (24, 2, "c128", True, "lattice"),   # 4x3 periodic lattice: the 32q model's family
+        "lat24c128": (24, 2, "c128", True, "lattice"),   # 4x3 periodic lattice, passes in FP64 (two layers)
+        "latd24c128": (24, 8, "c128", True, "lattice"),  # the 32q model's family and depth: fixed-point passes
         "lat24c64": (24, 2, "c64", True, "lattice"),
         "rand22c64": (22, 2, "c64", False, "random"),    # random Pauli sum: groups wider than a window
         "pcl24c128": (24, 0, "c128", True, "pc"),        # particle-conserving ansatz, 4x3 lattice

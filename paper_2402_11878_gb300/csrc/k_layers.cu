@@ -320,7 +320,7 @@ struct FixedEntry {
 
 // The pass program shapes of the default FP32 plans (tiles of 2^11 with 16
 // amplitudes per thread: chunks 0, 4, 7), forward and backward.  FP64 plans
-// with 8 amplitudes per thread run in fixed point (k_layers_fx.cu).
+// with 8 amplitudes per thread run in k_layers_fx.cu.
 const std::vector<FixedEntry> &fixed_programs() {
     static const std::vector<FixedEntry> table = {
         VQE_FWD(float, 4, VQE_RD(7), VQE_B, VQE_RD(4), VQE_B, VQE_D, VQE_RD(7)),
@@ -417,7 +417,7 @@ cudaError_t launch_pass(const PassDesc *desc_dev, const PassDesc &dh, int n_qubi
     switch (dh.R) {
         VQE_PASS_CASE(1)
         VQE_PASS_CASE(2)
-        case 3:   // FP64: in fixed point (launch_pass_fx)
+        case 3:   // FP64: launch_pass_fx
             if constexpr (sizeof(T) == 4)
                 return backward ? launch_pass_r<T, 3, true>(desc_dev, dh, n_qubits, batch, psi, lam, stride,
                                                             coefs, coef_stride, dtab, dtab_stride, gpart,

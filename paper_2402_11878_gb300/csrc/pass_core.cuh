@@ -574,7 +574,7 @@ __device__ __forceinline__ void run_tile_fixed(const PassDesc &d, const PassOp *
                                                typename V2<T>::type *lbuf, double *gsh,
                                                Env &env, Stage &&stage) {
     static_assert(Env::kLoad == 1, "direct environment");
-    static_assert(sizeof(T) == 4, "FP64 plans of fixed shape run in fixed point (k_layers_fx.cu)");
+    static_assert(sizeof(T) == 4, "FP64 plans of fixed shape run in k_layers_fx.cu");
     static_assert(!BWD || R == 4, "gradient rows are sized for R = 4");
     using C = typename V2<T>::type;
     constexpr int NR = 1 << R;

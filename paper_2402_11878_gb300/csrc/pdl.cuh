@@ -38,7 +38,9 @@ __device__ __forceinline__ C chain_load(const C *p) { return __ldca(p); }
 // Large ones: blocks of the next kernel take the places that the last wave frees
 // (22 qubits: 5921 -> 5821, complex64 1327 -> 1215).  In between the
 // early blocks double up on some SMs while others stay empty (18 qubits, 128
-// blocks: 677 -> 837; 19 qubits, 256 blocks: 905 -> 933).
+// blocks: 677 -> 837; 19 qubits, 256 blocks: 905 -> 933).  The lines, a quarter of a
+// block and three blocks per SM, lie between those sizes; nothing measured places
+// them closer.
 inline bool pdl_pays(dim3 grid) {
     const unsigned long long blocks = (unsigned long long)grid.x * grid.y;
     return blocks <= 38 || blocks >= 456;

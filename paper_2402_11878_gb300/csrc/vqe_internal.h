@@ -305,8 +305,9 @@ cudaError_t launch_pass(const PassDesc *desc_dev, const PassDesc &desc_host, int
                         size_t dtab_stride, double *grad_part, size_t grad_stride, bool backward,
                         int init_zero, cudaStream_t s);
 
-// The same in block fixed point (k_layers_fx.cu): FP64 plans with 8 amplitudes
-// per thread (R = 3), with their own coefficients and tables in the same buffers.
+// The same for FP64 plans with 8 amplitudes per thread (R = 3; k_layers_fx.cu): in
+// block fixed point or in FP64, as staging finds the angles, with their own
+// coefficients and tables in the same buffers.
 struct RotFx;
 cudaError_t launch_stage_fx(const StageSlot *slots_dev, int n_slots, int n_qubits, int depth,
                             const double *params, int batch, RotFx *coefs, size_t coef_stride,
