@@ -433,42 +433,6 @@ __device__ __forceinline__ long long fx_gate(long long (&re)[BWD ? 2 : 1][kNR],
     return ((hp - hn) << 3) + ((lo + (1ll << 27)) >> 28);
 }
 
-// The first forward pass when it holds one slot: its only nonzero tile (base
-// 0) starts as |0...0>, so element e of the tile is the product of one factor
-// per tile bit, and the slot's table entry and CZ sign at logical index
-// e ^ flips follow.  In FP64: one tile per state.
-__device__ __forceinline__ void write_product_tile_fx(const PassDesc &d, const RotFx *cf,
-                                                      const longlong2 *tab, int t0, uint32_t flips,
-                                                      double2 *P, uint32_t lowmask, int m, int a,
-                                                      int k) {
-    const uint32_t gated = d.slot_gated[0], cz = d.slot_czmask[0];
-    const int slot_shift = gated ? (int)((cf[__ffs(gated) - 1].meta >> kFxSlotShift) & 255u) : 0;
-    const int half = gated ? (int)(cf[__ffs(gated) - 1].meta & kFxHalf) : 0;
-    const double unit = ldexp(1.0, (half ? -62 : -63) - slot_shift);
-    for (uint32_t e = threadIdx.x; e < (1u << k); e += blockDim.x) {
-        double f = unit;
-        bool bad = false;
-        for (int j = 0; j < k; ++j) {
-            const bool bit = (e >> j) & 1u;
-            if (!((gated >> j) & 1u)) {
-                if (bit) f = 0.0;
-                continue;
-            }
-            const RotFx c = cf[j];
-            const double t = ((double)c.th * 0x1p32 + (double)c.tl) * 0x1p-64;
-            if (c.meta & kFx45) f *= bit ? 1.0 + t : 1.0 - t;
-            else if (bit) f *= t;
-            bad |= (c.meta & kFxBad) != 0u;
-        }
-        const uint32_t l = e ^ flips;
-        const uint32_t g = (l & lowmask) | ((l >> m) << a);
-        const longlong2 y = tab[l >> t0];
-        const double s = (__popc(g & (g >> 1) & cz) & 1) ? -f : f;
-        const double nan = __longlong_as_double(0x7ff8000000000000ll);
-        P[g] = bad ? make_double2(nan, nan) : make_double2((double)y.x * s, (double)y.y * s);
-    }
-}
-
 // A pass in FP64, for run_tile: bound by the FP64 pipe.  24 qubits, depth 8, energy /
 // gradient: normal angles of deviation 0.1 in FP64 13.4 / 54.5 ms (54.5 with a row of
 // partials per bit, 61.9 with a warp sum per gate), uniform angles in fixed point 6.7
@@ -616,6 +580,10 @@ k_pass_fx(const FxHead H, const PassDesc *__restrict__ desc, int init_zero, doub
         WideEnv env{&d, reinterpret_cast<const RotWide *>(scf), reinterpret_cast<const double2 *>(dt), gout, gslot,
                     P, L, init_zero, t0};
         double2 *buf = reinterpret_cast<double2 *>(sbuf);
+        if (!BWD && init_zero && H.n_slots == 1) {   // the tile at base 0
+            write_product_tile<double>(d, reinterpret_cast<const RotWide *>(scf), env.dt, P, base, lowmask, m, a, k);
+            return;
+        }
         if constexpr (BWD) wide_backward(d, H.n_ops, base, buf, reinterpret_cast<double *>(rows), size, env);
         else run_tile<double, kR, false>(d, d.ops, H.n_ops, base, buf, nullptr, nullptr, env);
         return;
@@ -627,13 +595,7 @@ k_pass_fx(const FxHead H, const PassDesc *__restrict__ desc, int init_zero, doub
         sh.flip[s] = f;
         sh.half[s] = scf[s * k + t0].meta & kFxHalf;
     }
-    if (!BWD && init_zero) {
-        __syncthreads();
-        if (H.n_slots == 1) {   // the tile at base 0
-            write_product_tile_fx(d, scf, dt + d.slot_dtab_off[0], t0, sh.flip[0], P, lowmask, m, a, k);
-            return;
-        }
-    }
+    if (!BWD && init_zero) __syncthreads();   // other tiles: fx_load_tile's
     const uint32_t nthr = blockDim.x;   // 2^(k - 3)
     const int nwarps = (int)((nthr + 31) >> 5);
     const int warp = t >> 5, lane = t & 31;

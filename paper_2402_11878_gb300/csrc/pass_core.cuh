@@ -105,6 +105,39 @@ __device__ __forceinline__ C cmul_conj(C x, C d) {   // x * conj(d)
     return r;
 }
 
+// The first forward pass when it holds one slot: its only nonzero tile (base
+// 0) starts as |0...0>, so the slot's scaled butterflies give each element
+// the product of one factor per tile bit (|0> -> (1, v) in tan form, (v, 1)
+// in cot form; an ungated bit stays 0), and the slot's diagonal (table entry
+// and CZ sign) follows.  Written straight to global memory, no tile rounds.
+template <typename T, class Row>
+__device__ __forceinline__ void write_product_tile(const PassDesc &d, const Row *cf,
+                                                   const typename V2<T>::type *dt,
+                                                   typename V2<T>::type *P, uint64_t base,
+                                                   uint32_t lowmask, int m, int a, int k) {
+    using C = typename V2<T>::type;
+    const uint32_t gated = d.slot_gated[0], cz = d.slot_czmask[0];
+    const C *tab = dt + d.slot_dtab_off[0];
+    for (uint32_t e = threadIdx.x; e < (1u << k); e += blockDim.x) {
+        const uint64_t g = base | (e & lowmask) | ((uint64_t)(e >> m) << a);
+        T f = T(1);
+        for (int j = 0; j < k; ++j) {
+            const uint32_t bit = (e >> j) & 1u;
+            if (!((gated >> j) & 1u)) {
+                if (bit) f = T(0);
+                continue;
+            }
+            const Row rc = cf[j];
+            if (bit ^ (uint32_t)rc.mode) f *= rc.v;
+        }
+        C y = tab[e >> (__ffs(gated) - 1)];
+        const uint32_t s = __popc((uint32_t)g & ((uint32_t)g >> 1) & cz) & 1u;
+        y.x = flip_sign(y.x * f, s);
+        y.y = flip_sign(y.y * f, s);
+        P[g] = y;
+    }
+}
+
 // Scratch a backward tile program needs besides the tile buffers:
 // nwarps * k * 2 doubles.
 __host__ __device__ inline size_t tile_grad_scratch_bytes(int threads, int k) {
