@@ -422,9 +422,9 @@ cudaError_t launch_apply_h(const GroupDesc *groups, int n_groups, const uint32_t
 }
 
 cudaError_t launch_energy_finish(const double *partials, int bps, int batch, double *energies,
-                                 double *norms, double *unnorm, cudaStream_t s) {
+                                 double *norms, double *unnorm, dim3 before, cudaStream_t s) {
     if (batch <= 0) return cudaSuccess;
-    return pdl_launch(k_energy_finish, batch, kFinishThreads, 0, s, pdl_pays(batch), partials, bps, batch, energies, norms,
+    return pdl_launch(k_energy_finish, batch, kFinishThreads, 0, s, pdl_pays(before) && pdl_pays(batch), partials, bps, batch, energies, norms,
                                                      unnorm);
 }
 

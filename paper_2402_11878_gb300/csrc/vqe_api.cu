@@ -1831,7 +1831,7 @@ vqe_status run_energy(vqe_ctx *h, int B, const void *psi, double *energies, doub
             h->stats.kernel_launches++;
         }
         prof_end(h, mk, int(h->hd.wins.size()) + (h->hd.n_wide ? 1 : 0));
-        VQE_CUDA(h, launch_energy_finish(part, bps_total, B, energies, norms, unnorm, h->stream));
+        VQE_CUDA(h, launch_energy_finish(part, bps_total, B, energies, norms, unnorm, dim3(bps_total, B), h->stream));
         h->stats.kernel_launches++;
         return VQE_OK;
     }
@@ -1844,7 +1844,7 @@ vqe_status run_energy(vqe_ctx *h, int B, const void *psi, double *energies, doub
                                  chained, h->stream));
     prof_end(h, mk, 1);
     VQE_CUDA(h, launch_energy_finish(static_cast<double *>(h->d_epart.p), bps, B, energies, norms,
-                                     unnorm, h->stream));
+                                     unnorm, dim3(bps, B), h->stream));
     h->stats.kernel_launches += 2;
     return VQE_OK;
 }
@@ -1897,7 +1897,7 @@ vqe_status run_apply_h(vqe_ctx *h, int B, void *psi, void *lam, double *E) {
         }
         prof_end(h, mk_h, ns);
         VQE_CUDA(h, launch_energy_finish(static_cast<double *>(h->d_epart.p), int(nchunks), B, E, nullptr,
-                                         nullptr, s));
+                                         nullptr, dim3(blocks, B), s));
         h->stats.kernel_launches++;
     } else if (windows && atiles * B >= uint64_t(2 * h->sms)) {
         // windowed: lambda accumulated window by window; the last window's
@@ -1917,7 +1917,7 @@ vqe_status run_apply_h(vqe_ctx *h, int B, void *psi, void *lam, double *E) {
         }
         prof_end(h, mk_h, nw);
         VQE_CUDA(h, launch_energy_finish(static_cast<double *>(h->d_epart.p), bps_w, B, E, nullptr,
-                                         nullptr, s));
+                                         nullptr, dim3(bps_w, B), s));
         h->stats.kernel_launches++;
     } else {
         const int bps = blocks_per_state(h, B);
@@ -1927,7 +1927,7 @@ vqe_status run_apply_h(vqe_ctx *h, int B, void *psi, void *lam, double *E) {
                                       psi, lam, N, static_cast<double *>(h->d_epart.p), bps, s));
         prof_end(h, mk_h, 1);
         VQE_CUDA(h, launch_energy_finish(static_cast<double *>(h->d_epart.p), bps, B, E, nullptr,
-                                         nullptr, s));
+                                         nullptr, dim3(bps, B), s));
         h->stats.kernel_launches += 2;
     }
     return VQE_OK;

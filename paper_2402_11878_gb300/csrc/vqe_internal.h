@@ -377,8 +377,11 @@ cudaError_t launch_energy_sub(const GroupDesc *groups, int n_groups, const uint3
                               size_t state_stride, double *partials, int bps, int block_off,
                               int bps_total, cudaStream_t s);
 
+// `before`: the grid whose partials these are.  What follows a reduction of a few
+// blocks that starts early starts beside that grid: where it leaves only some SMs
+// free, the blocks that follow would double up on them (see pdl_pays).
 cudaError_t launch_energy_finish(const double *partials, int blocks_per_state, int batch,
-                                 double *energies, double *norms, double *unnorm,
+                                 double *energies, double *norms, double *unnorm, dim3 before,
                                  cudaStream_t s);
 
 // Gradient reduction: param p of state b sums `count` partials at

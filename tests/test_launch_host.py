@@ -117,3 +117,19 @@ def test_a_smaller_launch_never_lowers_a_kernels_limit(runtime):
         limits.setdefault(name, set()).add(int(value))
     assert len(limits) >= 6
     assert {n: v for n, v in limits.items() if len(v) > 1} == {}
+
+
+@pytest.mark.parametrize("n,kind", [(14, "early"), (15, "plain"), (16, "plain"), (17, "plain"), (18, "early")])
+def test_passes_do_not_start_beside_a_grid_that_leaves_some_sms(runtime, n, kind):
+    """apply-H of a general Pauli sum has 2^(n - 9) blocks (152 SMs): the passes behind
+    its energy reduction may start early only beside a grid of up to 38 blocks, or one
+    that fills the chip."""
+    eng = runtime.engine(n, 2, "c128")
+    h = vi.random_pauli_sum(n, 5 * n, 1)
+    eng.set_hamiltonian(h.x, h.z, h.c)
+    assert eng.set_apply_mode(0) == 0
+    runtime.reset()
+    eng.gradient(np.zeros(eng.n_params))
+    rows = runtime.events("launch")
+    at = [i for i, r in enumerate(rows) if "k_apply_h" in r[0]][0]
+    assert "k_energy_finish" in rows[at + 1][0] and rows[at + 1][2] == kind
