@@ -91,7 +91,9 @@ __global__ void k_stage_fx(const StageSlot *__restrict__ slots, int n, int depth
     __shared__ longlong2 half_tab[2][1 << (kMaxTileBits / 2)];
     __shared__ longlong2 d0[kMaxTileBits], d1[kMaxTileBits];
     __shared__ long long scl[kMaxTileBits];
-    __shared__ double lg[kMaxTileBits];
+    __shared__ float lg[kMaxTileBits];
+    __shared__ long long scale_at[kMaxTileBits];   // of the buffers when the bit's theta gradient is taken
+    __shared__ int turns_of[kMaxTileBits], order[kMaxTileBits], shb[kMaxTileBits];
     __shared__ RotFx rot[kMaxTileBits];
     __shared__ long long sigma;   // 2^S sigma
     __shared__ int table_shift;
@@ -103,11 +105,14 @@ __global__ void k_stage_fx(const StageSlot *__restrict__ slots, int n, int depth
                            reinterpret_cast<double2 *>(dtab + (size_t)b * dtab_stride + S.dtab_off));
         return;
     }
-    if (threadIdx.x < (unsigned)S.n_gated) {
-        const int j = threadIdx.x;
+    // Latency is what staging costs (FP64 instructions issue once per 64 clocks): theta
+    // and phi in a warp each, the serial schedule in FP32 and integers, divisions in
+    // parallel (64 states of 8 qubits, one slot: 24.7 -> 16.3 us).
+    const int j = threadIdx.x & 31;
+    const bool mine = j < S.n_gated;
+    if (threadIdx.x < 32 && mine) {
         const int q = S.qubit[j];
-        const double th = pr[((size_t)S.layer * n + q) * 2];
-        const double phi = pr[((size_t)S.layer * n + q) * 2 + 1];
+        const double th = pr[((size_t)S.layer * n + q) * 2], phi = pr[((size_t)S.layer * n + q) * 2 + 1];
         double s, c;
         sincos(0.5 * th, &s, &c);
         // quarter turns taken off until the angle lies in [-pi/8, 3 pi/8):
@@ -136,37 +141,44 @@ __global__ void k_stage_fx(const StageSlot *__restrict__ slots, int n, int depth
         long long sc = to62(s0, 0.5 * res);
         if (half_turn) sc = __mul64hi(sc, 0x5A827999FCEF3242ll) << 1;   // 2^63 / sqrt(2)
         scl[j] = sc;
-        lg[j] = -log2((double)sc * 0x1p-62);
+        lg[j] = -log2f((float)sc * 0x1p-62f);
+        turns_of[j] = turns;
         const bool bad = !(isfinite(th) && isfinite(phi));
         const long long T = bad ? 0ll : __double2ll_rn(tt * 0x1p64);
         rot[j].tl = fx_lo(T);
         rot[j].th = fx_hi(T);
         rot[j].meta = ((turns & 1) ? kFxFlip : 0u) | (half_turn ? kFx45 : 0u) | (bad ? kFxBad : 0u);
         rot[j].wide = 0;
+    } else if (threadIdx.x >= 32 && threadIdx.x < 64 && mine) {
+        const double phi = pr[((size_t)S.layer * n + S.qubit[j]) * 2 + 1];
         double sp, cp;
         sincos(0.5 * phi, &sp, &cp);
         const double c2 = cp * cp, c2e = fma(cp, cp, -c2), s2 = sp * sp, s2e = fma(sp, sp, -s2);
         const double half_res = 0.5 * ((((1.0 - fmax(c2, s2)) - fmin(c2, s2)) - c2e) - s2e);
         const long long ci = to62(cp, half_res), si = to62(sp, half_res);
-        // J^q: logical bit 0 takes -1 for q = 1, 2 and bit 1 for q = 2, 3
-        const bool n0 = turns == 1 || turns == 2, n1 = turns >= 2;
-        d0[j] = n0 ? make_longlong2(-ci, si) : make_longlong2(ci, -si);
-        d1[j] = n1 ? make_longlong2(-ci, -si) : make_longlong2(ci, si);
+        d0[j] = make_longlong2(ci, -si);
+        d1[j] = make_longlong2(ci, si);
     }
     __syncthreads();
+    if (threadIdx.x >= 32 && threadIdx.x < 64 && mine) {
+        // J^q: logical bit 0 takes -1 for q = 1, 2 and bit 1 for q = 2, 3
+        const int turns = turns_of[j];
+        const longlong2 a = d0[j], b1 = d1[j];
+        if (turns == 1 || turns == 2) d0[j] = make_longlong2(-a.x, -a.y);
+        if (turns >= 2) d1[j] = make_longlong2(-b1.x, -b1.y);
+    }
     if (threadIdx.x == 0) {
         // shift schedule: A = log2 of the norm's growth since the slot began
         const int ng = S.n_gated;
-        int order[kMaxTileBits], shb[kMaxTileBits];
-        double A = 0.0;
+        float A = 0.f;
         int total = 0;
         long long sig = 1ll << 62;
         for (int j = 0; j < ng; ++j) order[__popc(S.fbefore[j])] = j;
         for (int i = 0; i < ng; ++i) {
             const int j = order[i];
             A += lg[j];
-            const int sh = A >= 1.0 ? 1 : 0;   // lg < 0.62: at most one
-            A -= sh;
+            const int sh = A >= 1.f ? 1 : 0;   // lg < 0.62: at most one
+            A -= (float)sh;
             total += sh;
             sig = mul62(sig, scl[j]) << sh;
             rot[j].meta |= (uint32_t)sh << kFxShiftF;
@@ -175,15 +187,15 @@ __global__ void k_stage_fx(const StageSlot *__restrict__ slots, int n, int depth
         sigma = sig;
         table_shift = near_one ? 0 : 1;
         for (int j = 0; j < ng; ++j) order[__popc(S.before[j])] = j;
-        A = total;
+        A = (float)total;
         for (int j = 0; j < ng; ++j) A -= lg[j];
         int done = 0;
         for (int i = 0; i < ng; ++i) {
             // A < 0.75 where the next gate's theta gradient is taken (after its turn)
             A += lg[order[i]];
-            const double limit = i + 1 < ng && (rot[order[i + 1]].meta & kFx45) ? 0.25 : 0.75;
+            const float limit = i + 1 < ng && (rot[order[i + 1]].meta & kFx45) ? 0.25f : 0.75f;
             int sh = A >= limit && done < total ? 1 : 0;
-            A -= sh;
+            A -= (float)sh;
             if (i == ng - 1) sh = min(3, total - done);
             done += sh;
             shb[i] = sh;
@@ -192,9 +204,7 @@ __global__ void k_stage_fx(const StageSlot *__restrict__ slots, int n, int depth
         for (int i = ng - 1; i >= 0; --i) {
             const int j = order[i];
             f = mul62(f, scl[j]) << shb[i];
-            const double fd = (double)f * 0x1p-62;
-            // the theta gradient is taken after the bit's 45-degree turn (x sqrt 2)
-            rot[j].gs = 0.125 / (fd * fd * ((rot[j].meta & kFx45) ? 2.0 : 1.0));
+            scale_at[j] = f;
             rot[j].meta |= ((uint32_t)shb[i] << kFxShiftB) | ((uint32_t)total << kFxSlotShift) |
                            (near_one ? kFxHalf : 0u);
         }
@@ -203,9 +213,16 @@ __global__ void k_stage_fx(const StageSlot *__restrict__ slots, int n, int depth
     // one row per tile bit; the gated bits are the tile's top ones (all of them in
     // the low group), and the table has no index bits below them
     const int t0 = S.tile_bit[0], kt = S.k - t0;
-    if (threadIdx.x < (unsigned)S.k)
-        coefs[(size_t)b * coef_stride + S.coef_off + threadIdx.x] =
-            (int)threadIdx.x < t0 ? RotFx{0, 0, 0u, 0, 0.0} : rot[threadIdx.x - t0];
+    if (threadIdx.x < (unsigned)S.k) {
+        RotFx r{0, 0, 0u, 0, 0.0};
+        if ((int)threadIdx.x >= t0) {
+            r = rot[threadIdx.x - t0];
+            const double fd = (double)scale_at[threadIdx.x - t0] * 0x1p-62;
+            // the theta gradient is taken after the bit's 45-degree turn (x sqrt 2)
+            r.gs = 0.125 / (fd * fd * ((r.meta & kFx45) ? 2.0 : 1.0));
+        }
+        coefs[(size_t)b * coef_stride + S.coef_off + threadIdx.x] = r;
+    }
     const int kl = kt >> 1, kh = kt - kl;
     for (uint32_t i = threadIdx.x; i < (1u << kl) + (1u << kh); i += blockDim.x) {
         const bool high = i >= (1u << kl);
