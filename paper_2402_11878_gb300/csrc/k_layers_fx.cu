@@ -491,7 +491,7 @@ __device__ __noinline__ void wide_backward(const PassDesc &d, int n_ops, uint64_
 // are slower backward (348 and 375 against 276 ms).
 // Against the same passes in FP64 multiply-adds, whole calls: 28-qubit energy +
 // gradient (depth 8) 961 -> 395 ms, 64 energies at 20 qubits (depth 10) 54.6 ->
-// 24.7 ms, gradient at 13 qubits (depth 6) 713 -> 488 us.
+// 24.7 ms, gradient at 13 qubits (depth 6) 713 -> 433 us.
 template <bool BWD, int MAXT, int MINB>
 __global__ void __launch_bounds__(MAXT, MINB)
 k_pass_fx(const FxHead H, const PassDesc *__restrict__ desc, int init_zero, double2 *psi,
